@@ -249,7 +249,9 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_base_slot + 1);
     [[maybe_unused]] volatile unsigned int* item_slots = reinterpret_cast<volatile unsigned int*>(tmem_base_slot + 2);   // 4 words
 
-    const int warp = threadIdx.x >> 5;
+    // A shuffled warp number is one the compiler knows to be the same in all lanes: the roles below branch on it, their
+    // warps stay together, and addresses and descriptors are computed once per warp (see the MMA issuer).
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);
     const int lane = threadIdx.x & 31;
     const int num_tiles = prm.num_k_tiles * prm.num_p_tiles * prm.num_pos;
     constexpr uint32_t TMEM_COLS = 2 * GEMM_MAX_N;
@@ -327,7 +329,8 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
     __syncthreads();
     if constexpr (CTAS == 2) cluster_sync_all();   // the peer's barriers are initialised before anyone signals them
     tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_base_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_base_slot, 0);
+    const bool elected = elect_one() != 0;   // the lane that issues loads, MMAs and arrivals of a role
 
     const bool wt_ok = wt_hdr.x == WT_MAGIC && wt_hdr.y == static_cast<uint32_t>(prm.K) &&
                        wt_hdr.z == static_cast<uint32_t>(prm.C) && wt_hdr.w == static_cast<uint32_t>(prm.tile);
@@ -336,13 +339,14 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
         if (threadIdx.x == 0) atomicCAS(status_word, 0, 1 | (9 << 8));   // 1 = SDWINO_ERR_INVALID_ARG
     } else if (warp == 0) {
         // ------------------------------ TMA producer ------------------------------
-        if (resident && lane == 0) {
+        if (resident) {
             // filter-resident mode: the filter block of a (position, k-tile) is loaded once, V streams through the ring
             const uint32_t smem_base = smem_u32(smem);
             const uint32_t ures_a = smem_u32(ures_base);
             const uint32_t ures_full_a = smem_u32(ures_full_bar);
             const uint32_t full0 = smem_u32(&full_bar[0]);
             auto load_filters = [&](int pos, int kt) {
+                if (!elected) return;
                 mbar_arrive_expect_tx_a32(ures_full_a, static_cast<uint32_t>(ures_bytes));
                 for (int cb = 0; cb < prm.num_c_blocks; ++cb)
                     tma_load_5d_a32(ures_a + cb * ures_cb_bytes, &tmU, ures_full_a, cb, (kt * prm.n_tile) >> 4, pos);
@@ -368,7 +372,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                 decode(tile_of(i), pt, kt, pos);
                 if (pos * prm.num_k_tiles + kt != cur_key) {
                     // the MMAs of the previous run of tiles have finished reading the resident block
-                    ok = mbar_wait_bounded(ures_empty_bar, reloads & 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                    ok = mbar_wait_warp(ures_empty_bar, reloads & 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                     if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 5, cta_rank); break; }
                     ++reloads;
                     load_filters(pos, kt);
@@ -379,7 +383,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                     // V of this block of tiles is written by the transform warps of this launch.  The counter was read
                     // one tile ahead (the read is a round trip to L2 on this one thread's critical path).
                     if (seen_pt != pt || seen < static_cast<unsigned int>(pp.it_items)) {
-                        ok = wait_counter(&pp.v_ready[pt], static_cast<unsigned int>(pp.it_items), pp.abort_word, GEMM_WAIT_LIMIT_NS);
+                        ok = __all_sync(0xffffffffu, wait_counter(&pp.v_ready[pt], static_cast<unsigned int>(pp.it_items), pp.abort_word, GEMM_WAIT_LIMIT_NS)) != 0;
                         if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 12, cta_rank); break; }
                     }
                     fence_proxy_async_all();
@@ -391,18 +395,20 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                     }
                 }
                 for (int c0 = 0; c0 < prm.C; c0 += GEMM_BLOCK_C) {
-                    ok = mbar_wait_bounded(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                    ok = mbar_wait_warp(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                     if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 1, cta_rank); break; }
-                    mbar_arrive_expect_tx_a32(fb, L::A_BYTES);
-                    tma_load_3d_a32(sa, &tmV, fb, p0, c0, pos);
-                    tma_load_3d_a32(sa + L::A_BOX_BYTES, &tmV, fb, p0 + 64, c0, pos);
+                    if (elected) {
+                        mbar_arrive_expect_tx_a32(fb, L::A_BYTES);
+                        tma_load_3d_a32(sa, &tmV, fb, p0, c0, pos);
+                        tma_load_3d_a32(sa + L::A_BOX_BYTES, &tmV, fb, p0 + 64, c0, pos);
+                    }
                     sa += stage_bytes;
                     fb += 8;
                     if (++stage == stages) { stage = 0; phase ^= 1u; sa = smem_base; fb = full0; }
                 }
             }
             if (!ok) *abort_flag = 1;
-        } else if (U8 && lane == 0) {
+        } else if (U8) {
             // 8-bit filters.  Two streams from one thread: the raw filter boxes, which come from HBM and depend on
             // nothing, run `lead` steps ahead of the boxes of V through a ring of their own; a step's operand stage is
             // completed by V (this thread) and by the warps that expand the raw box into it.
@@ -427,11 +433,13 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
             }
             for (int j = 0; j < total + lead && ok; ++j) {
                 if (j < total) {
-                    ok = mbar_wait_bounded(&raw_empty_bar[r_slot], r_par, abort_flag, GEMM_WAIT_LIMIT_NS);
+                    ok = mbar_wait_warp(&raw_empty_bar[r_slot], r_par, abort_flag, GEMM_WAIT_LIMIT_NS);
                     if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 8, cta_rank); break; }
                     const uint32_t rb = smem_u32(&raw_full_bar[r_slot]);
-                    mbar_arrive_expect_tx_a32(rb, static_cast<uint32_t>(raw_slot_bytes));
-                    tma_load_5d_hint_a32(raw_base + r_slot * raw_slot_bytes, &tmU, rb, r_cb, r_kb, r_pos, u_policy);
+                    if (elected) {
+                        mbar_arrive_expect_tx_a32(rb, static_cast<uint32_t>(raw_slot_bytes));
+                        tma_load_5d_hint_a32(raw_base + r_slot * raw_slot_bytes, &tmU, rb, r_cb, r_kb, r_pos, u_policy);
+                    }
                     if (++r_slot == R) { r_slot = 0; r_par ^= 1u; }
                     if (++r_cb == spt) {
                         r_cb = 0;
@@ -444,13 +452,15 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                 }
                 if (j >= lead) {
                     if (j == lead) pdl_wait();                 // V is written by the preceding kernel
-                    ok = mbar_wait_bounded(&empty_bar[v_stage], v_par, abort_flag, GEMM_WAIT_LIMIT_NS);
+                    ok = mbar_wait_warp(&empty_bar[v_stage], v_par, abort_flag, GEMM_WAIT_LIMIT_NS);
                     if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 1, cta_rank); break; }
                     const uint32_t fb = smem_u32(&full_bar[v_stage]);
                     const uint32_t sa = smem_base + v_stage * stage_bytes;
-                    mbar_arrive_expect_tx_a32(fb, static_cast<uint32_t>(a_bytes));
-                    tma_load_3d_a32(sa, &tmV, fb, v_p0, v_cb * GEMM_BLOCK_C, v_pos);
-                    tma_load_3d_a32(sa + L::A_BOX_BYTES, &tmV, fb, v_p0 + 64, v_cb * GEMM_BLOCK_C, v_pos);
+                    if (elected) {
+                        mbar_arrive_expect_tx_a32(fb, static_cast<uint32_t>(a_bytes));
+                        tma_load_3d_a32(sa, &tmV, fb, v_p0, v_cb * GEMM_BLOCK_C, v_pos);
+                        tma_load_3d_a32(sa + L::A_BOX_BYTES, &tmV, fb, v_p0 + 64, v_cb * GEMM_BLOCK_C, v_pos);
+                    }
                     if (++v_stage == stages) { v_stage = 0; v_par ^= 1u; }
                     if (++v_cb == spt) {
                         v_cb = 0;
@@ -464,7 +474,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
             }
             if (total == 0) pdl_wait();
             if (!ok) *abort_flag = 1;
-        } else if (!resident && lane == 0) {
+        } else if (!resident) {
             // the full barrier of a pair lives in the leader and counts the bytes of both CTAs
             const uint32_t tx_bytes = CTAS * (a_bytes + L::b_bytes(b_rows));
             // single-thread loop: shared-memory and barrier addresses are running 32-bit values
@@ -491,13 +501,15 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                     decode(tile_of(i), pt, kt, pos);
                     const int p0 = pt * PT * GEMM_BLOCK_P;
                     for (int c0 = 0; c0 < prm.C; c0 += GEMM_BLOCK_C) {
-                        ok = mbar_wait_bounded(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                        ok = mbar_wait_warp(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                         if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 1, cta_rank); break; }
-                        mbar_arrive_expect_tx_a32(fb, static_cast<uint32_t>(a_bytes));
+                        if (elected) {
+                            mbar_arrive_expect_tx_a32(fb, static_cast<uint32_t>(a_bytes));
 #pragma unroll
-                        for (int sub = 0; sub < PT; ++sub) {
-                            tma_load_3d_a32(sa + sub * L::A_BYTES, &tmV, fb, p0 + sub * GEMM_BLOCK_P, c0, pos);
-                            tma_load_3d_a32(sa + sub * L::A_BYTES + L::A_BOX_BYTES, &tmV, fb, p0 + sub * GEMM_BLOCK_P + 64, c0, pos);
+                            for (int sub = 0; sub < PT; ++sub) {
+                                tma_load_3d_a32(sa + sub * L::A_BYTES, &tmV, fb, p0 + sub * GEMM_BLOCK_P, c0, pos);
+                                tma_load_3d_a32(sa + sub * L::A_BYTES + L::A_BOX_BYTES, &tmV, fb, p0 + sub * GEMM_BLOCK_P + 64, c0, pos);
+                            }
                         }
                         sa += stage_bytes;
                         fb += 8;
@@ -513,8 +525,10 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                     decode(tile_of(i), pt, kt, pos);
                     const int k0 = kt * prm.n_tile;
                     for (int c0 = 0; c0 < prm.C && pre < stages; c0 += GEMM_BLOCK_C) {
-                        mbar_arrive_expect_tx_a32(fb_u, tx_bytes);
-                        tma_load_5d_hint_a32(sa_u, &tmU, fb_u, c0 >> 6, k0 >> 4, pos, u_policy);
+                        if (elected) {
+                            mbar_arrive_expect_tx_a32(fb_u, tx_bytes);
+                            tma_load_5d_hint_a32(sa_u, &tmU, fb_u, c0 >> 6, k0 >> 4, pos, u_policy);
+                        }
                         sa_u += stage_bytes;
                         fb_u += 8;
                         ++pre;
@@ -536,7 +550,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                     // V of this block of tiles is written by the transform warps of this launch (counter read one
                     // tile ahead, as in the filter-resident producer)
                     if (seen_pt != pt || seen < static_cast<unsigned int>(pp.it_items)) {
-                        ok = wait_counter(&pp.v_ready[pt], static_cast<unsigned int>(pp.it_items), pp.abort_word, GEMM_WAIT_LIMIT_NS);
+                        ok = __all_sync(0xffffffffu, wait_counter(&pp.v_ready[pt], static_cast<unsigned int>(pp.it_items), pp.abort_word, GEMM_WAIT_LIMIT_NS)) != 0;
                         if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 12, cta_rank); break; }
                     }
                     fence_proxy_async_all();
@@ -552,7 +566,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                     if (issued < pre) {
                         // the barrier is armed and the filter box is on its way: add the boxes of V
 #pragma unroll
-                        for (int sub = 0; sub < PT; ++sub) {
+                        for (int sub = 0; sub < PT && elected; ++sub) {
                             tma_load_3d_a32(sa + sub * L::A_BYTES, &tmV, fb, p0 + sub * GEMM_BLOCK_P, c0, pos);
                             tma_load_3d_a32(sa + sub * L::A_BYTES + L::A_BOX_BYTES, &tmV, fb, p0 + sub * GEMM_BLOCK_P + 64, c0, pos);
                         }
@@ -563,9 +577,10 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                         if (++stage == stages) { stage = 0; phase ^= 1u; sa = smem_base; fb = full0; fb_local = full0_local; }
                         continue;
                     }
-                    ok = mbar_wait_bounded(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                    ok = mbar_wait_warp(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                     if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 1, cta_rank); break; }
-                    if constexpr (CTAS == 2) {
+                    if (!elected) {
+                    } else if constexpr (CTAS == 2) {
                         if (leader) mbar_arrive_expect_tx_a32(fb_local, tx_bytes);
                         tma_load_3d_pair(sa, &tmV, fb, p0, c0, pos);
                         tma_load_3d_pair(sa + L::A_BOX_BYTES, &tmV, fb, p0 + 64, c0, pos);
@@ -590,7 +605,11 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0 && leader) {
+        // The whole warp runs this loop and one elected lane issues.  Issued from a branch that only lane 0 takes, the
+        // descriptors pass through vector registers: an MMA then costs 52 cycles of issue and a wait on a barrier that
+        // has already completed about 270, i.e. 480 per stage against the 320 of its MMAs at n_tile 160 (in a loop of
+        // back-to-back MMAs 86 cycles each; as it stands 80 at N = 160, the tensor rate).
+        if (leader) {
             const uint32_t idesc = make_idesc_f16_f32(GEMM_BLOCK_P * CTAS, prm.n_tile, true, false);
             // This loop is executed by ONE thread, so every instruction in it costs its full latency: the
             // descriptors of stage 0 are built once and then only advanced by additions (the 14-bit
@@ -621,15 +640,15 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                 if (resident) {
                     key = static_cast<int>(fast_div(static_cast<uint32_t>(tile), prm.fd_p));      // pos * num_k_tiles + kt
                     if (key != cur_key) {
-                        ok = mbar_wait_bounded(ures_full_bar, loads_seen & 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                        ok = mbar_wait_warp(ures_full_bar, loads_seen & 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                         if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 6, cta_rank); break; }
                         ++loads_seen;
                         cur_key = key;
                     }
                 }
-                ok = mbar_wait_bounded(&acc_empty_bar[buf], acc_phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                ok = mbar_wait_warp(&acc_empty_bar[buf], acc_phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                 if constexpr (DUAL) {   // this tile fills both accumulator buffers
-                    if (ok) ok = mbar_wait_bounded(&acc_empty_bar[1], acc_phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                    if (ok) ok = mbar_wait_warp(&acc_empty_bar[1], acc_phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                 }
                 if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 2, cta_rank); break; }
                 tc_fence_after_sync();
@@ -637,13 +656,14 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                 [[maybe_unused]] const uint32_t d_tmem1 = tmem_base + static_cast<uint32_t>(GEMM_MAX_N);
                 [[maybe_unused]] constexpr uint64_t a_sub = static_cast<uint64_t>(L::A_BYTES >> 4);   // second block of tiles
                 for (int cb = 0; cb < prm.num_c_blocks; ++cb) {
-                    if (!mbar_try_wait_a32(full_a, phase)) {
-                        ok = mbar_wait_slow(&full_bar[stage], phase, abort_flag, GEMM_WAIT_LIMIT_NS);
+                    if (!__all_sync(0xffffffffu, mbar_try_wait_a32(full_a, phase))) {
+                        ok = __all_sync(0xffffffffu, mbar_wait_slow(&full_bar[stage], phase, abort_flag, GEMM_WAIT_LIMIT_NS)) != 0;
                         if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 3, cta_rank); break; }
                     }
                     tc_fence_after_sync();
                     const uint64_t bd = resident ? ures_desc0 + static_cast<uint64_t>(cb) * ures_step : bdesc;
-                    if (cb < full_blocks) {
+                    if (!elected) {
+                    } else if (cb < full_blocks) {
                         if constexpr (CTAS == 2) {
                             umma_f16_pair(d_tmem, adesc, bdesc, idesc, static_cast<uint32_t>(cb));
                             umma_f16_pair_acc(d_tmem, adesc + 128, bdesc + 2, idesc);
@@ -671,8 +691,10 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                                 umma_f16(d_tmem1, adesc + a_sub + 128 * s, bd + 2 * s, idesc, (cb > 0 || s > 0) ? 1u : 0u);
                         }
                     }
-                    if constexpr (CTAS == 2) umma_commit_pair_a32(empty_a);
-                    else umma_commit_a32(empty_a);
+                    if (elected) {
+                        if constexpr (CTAS == 2) umma_commit_pair_a32(empty_a);
+                        else umma_commit_a32(empty_a);
+                    }
                     adesc += stage_step;
                     bdesc += stage_step;
                     full_a += 8;
@@ -682,11 +704,13 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                     }
                 }
                 if (!ok) break;
-                if constexpr (CTAS == 2) umma_commit_pair(&acc_full_bar[buf]);
-                else umma_commit(&acc_full_bar[buf]);
-                if constexpr (DUAL) umma_commit(&acc_full_bar[1]);
+                if (elected) {
+                    if constexpr (CTAS == 2) umma_commit_pair(&acc_full_bar[buf]);
+                    else umma_commit(&acc_full_bar[buf]);
+                    if constexpr (DUAL) umma_commit(&acc_full_bar[1]);
+                }
                 // the last tile of a run: once its MMAs have completed the resident filters may be replaced
-                if (resident && i + 1 < my_count &&
+                if (resident && elected && i + 1 < my_count &&
                     static_cast<int>(fast_div(static_cast<uint32_t>(tile_of(i + 1)), prm.fd_p)) != key)
                     umma_commit(ures_empty_bar);
                 if constexpr (DUAL) {
@@ -977,7 +1001,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
         // The filters depend on nothing before this launch (see the comment in the first producer), so this thread
         // never waits for the preceding kernel: the first ring-full of boxes goes out at once, the rest as stages
         // are released.
-        if (lane == 0) {
+        {
             const uint32_t smem_base = smem_u32(smem);
             const uint32_t full0 = smem_u32(&full_bar[0]);
             const uint32_t u_bytes = static_cast<uint32_t>(L::b_bytes(b_rows));
@@ -991,10 +1015,12 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                 decode(tile_of(i), pt, kt, pos);
                 const int k0 = kt * prm.n_tile;
                 for (int c0 = 0; c0 < prm.C; c0 += GEMM_BLOCK_C) {
-                    ok = mbar_wait_bounded(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                    ok = mbar_wait_warp(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                     if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 11, cta_rank); break; }
-                    mbar_arrive_expect_tx_a32(fb, u_bytes);
-                    tma_load_5d_hint_a32(sa, &tmU, fb, c0 >> 6, k0 >> 4, pos, u_policy);
+                    if (elected) {
+                        mbar_arrive_expect_tx_a32(fb, u_bytes);
+                        tma_load_5d_hint_a32(sa, &tmU, fb, c0 >> 6, k0 >> 4, pos, u_policy);
+                    }
                     sa += stage_bytes;
                     fb += 8;
                     if (++stage == stages) { stage = 0; phase ^= 1u; sa = smem_base + a_bytes; fb = full0; }
