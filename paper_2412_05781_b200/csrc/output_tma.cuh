@@ -36,7 +36,7 @@ output_transform_f4_tma_kernel(const __grid_constant__ CUtensorMap tmM, const YT
     __shared__ int abort_flag;
     const int tid = threadIdx.x;
     pdl_launch_dependents();
-    const bool wt_ok = wt_check(chk);   // before the wait: see output_transform_kernel
+    const bool wt_ok = wt_check(chk);   // before the wait: see output_direct_kernel
     if (tid == 0) {
         for (int s = 0; s < OUT_TMA_STAGES; ++s) mbar_init(&full_bar[s], 1);
         abort_flag = 0;

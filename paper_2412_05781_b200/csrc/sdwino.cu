@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "transforms.cuh"
+#include "transforms_any.cuh"
 #include "wino_gemm.cuh"
 #include "fused_small_k.cuh"
 #include "input_tma.cuh"
@@ -445,7 +446,7 @@ int launch_input(const XT* x, __half* V, const TileGeom& geo, int C, long long p
     const long long units = static_cast<long long>(p_count / TPT) * C;   // one thread each
     if constexpr (M == 1) {
         const dim3 grid = grid_rows((p_count + 127) / 128, C);
-        e = launch_pdl(input_transform_kernel<M, XT>, grid, dim3(128), 0, st, 0, x, V, geo, C, p_begin, p_count, Pstride, amax);
+        e = launch_pdl(input_direct_kernel, grid, dim3(128), 0, st, 0, x, V, geo, C, p_begin, p_count, Pstride);
     } else if (geo.W % 8 == 0 && aligned(x, 16) && units < (1ll << 31) - 128) {
         if constexpr (M == 4) {
             constexpr int CH = 1;   // channels per thread
@@ -459,8 +460,8 @@ int launch_input(const XT* x, __half* V, const TileGeom& geo, int C, long long p
                            make_fastdiv(static_cast<uint32_t>(p_count / TPT)), Pstride, amax);
         }
     } else {
-        const dim3 grid = grid_rows((p_count + 127) / 128, C);
-        e = launch_pdl(input_transform_kernel<M, XT>, grid, dim3(128), 0, st, 0, x, V, geo, C, p_begin, p_count, Pstride, amax);
+        const dim3 grid = grid_rows((p_count / 2 + 127) / 128, C);
+        e = launch_pdl(input_transform_any_kernel<M, XT>, grid, dim3(128), 0, st, 0, x, V, geo, C, p_begin, p_count, Pstride, amax);
     }
     g_launches.fetch_add(1);
     return e == cudaSuccess ? SDWINO_OK : err_cuda(__LINE__);
@@ -620,6 +621,23 @@ int launch_output_tma(const __half* Mws, const YT* bias, YT* y, const TileGeom& 
     return e == cudaSuccess ? SDWINO_OK : err_cuda(__LINE__);
 }
 
+// The output transform of any width (see transforms_any.cuh).
+template <int M, typename YT>
+cudaError_t launch_output_any(const __half* Mws, const YT* bias, YT* y, const TileGeom& geo, int K, long long p_begin, int p_count,
+                              long long Pstride, const WtCheck& chk, const Epilogue& ep, cudaStream_t st) {
+    const int sms = sm_count();
+    if (sms <= 0) return cudaErrorInvalidDevice;
+    const unsigned blocks = static_cast<unsigned>((p_count / 2 + OUT_ANY_THREADS - 1) / OUT_ANY_THREADS);
+    // channels per CTA (the tiles are decoded once): as many as leave several waves of the six CTAs that fit an SM
+    const long long steps = std::max(1ll, std::min(4ll, static_cast<long long>(blocks) * K / (24ll * sms)));
+    const dim3 grid = grid_rows(blocks, (K + steps - 1) / steps);
+    if (ep.residual != nullptr || ep.act != 0)
+        return launch_pdl(output_transform_any_kernel<M, true, YT>, grid, dim3(OUT_ANY_THREADS), 0, st, 0, Mws, bias, y, geo, K, p_begin,
+                          p_count, Pstride, static_cast<int>(steps), chk, ep);
+    return launch_pdl(output_transform_any_kernel<M, false, YT>, grid, dim3(OUT_ANY_THREADS), 0, st, 0, Mws, bias, y, geo, K, p_begin,
+                      p_count, Pstride, static_cast<int>(steps), chk, ep);
+}
+
 template <int M, typename YT>
 int launch_output(const __half* Mws, const YT* bias, YT* y, const TileGeom& geo, int K,
                   long long p_begin, int p_count, long long Pstride, const WtCheck& chk, const Epilogue& ep,
@@ -630,7 +648,7 @@ int launch_output(const __half* Mws, const YT* bias, YT* y, const TileGeom& geo,
     const long long units = static_cast<long long>(p_count / TPT) * K;   // one thread each
     if constexpr (M == 1) {
         const dim3 grid = grid_rows((p_count + 127) / 128, K);
-        e = launch_pdl(output_transform_kernel<M, YT>, grid, dim3(128), 0, st, 0, Mws, bias, y, geo, K, p_begin, p_count,
+        e = launch_pdl(output_direct_kernel, grid, dim3(128), 0, st, 0, Mws, bias, y, geo, K, p_begin, p_count,
                        Pstride, chk, ep);
     } else if (geo.W % 8 == 0 && aligned(y, 16) && aligned(ep.residual, 16) && units < (1ll << 31) - 128) {
         dim3 grid(static_cast<unsigned>((units + 127) / 128));
@@ -642,9 +660,7 @@ int launch_output(const __half* Mws, const YT* bias, YT* y, const TileGeom& geo,
                            p_begin, make_fastdiv(static_cast<uint32_t>(p_count / TPT)), Pstride, chk, ep);
         }
     } else {
-        const dim3 grid = grid_rows((p_count + 127) / 128, K);
-        e = launch_pdl(output_transform_kernel<M, YT>, grid, dim3(128), 0, st, 0, Mws, bias, y, geo, K, p_begin, p_count,
-                       Pstride, chk, ep);
+        e = launch_output_any<M, YT>(Mws, bias, y, geo, K, p_begin, p_count, Pstride, chk, ep, st);
     }
     g_launches.fetch_add(1);
     return e == cudaSuccess ? SDWINO_OK : err_cuda(__LINE__);

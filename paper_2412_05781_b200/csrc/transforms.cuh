@@ -1,8 +1,8 @@
 // Steps (i) and (iii) of Section "Techniques": filter preprocess U = G g G^T, activation
 // preprocess V = B^T d B on overlapping (m+2)x(m+2) windows, and postprocess
 // Y = A^T M A followed by bias add, rounding to fp16 and a store masked at the image edge.
-// These kernels are bandwidth-bound: one thread per (channel, tile), consecutive threads on
-// consecutive tiles so that every global access of a warp is contiguous.
+// These kernels are bandwidth-bound: consecutive threads on consecutive tiles so that every global access of a warp is
+// contiguous.
 //
 // The paper prints no matrices; these are the Toom-Cook matrices of the construction it cites.
 // F(2x2,3x3) uses the points {0, 1, -1, inf}; F(4x4,3x3) uses {0, 3/4, -3/4, 3/2, -3/2, inf},
@@ -344,15 +344,12 @@ __device__ __forceinline__ void decode_tile(const TileGeom& geo, long long p, lo
     n = img;
 }
 
-// Activation preprocess.  V layout: [a*a][C][Pstride] with the chunk-local tile index
-// (p - p_begin) contiguous.  Threads past the last tile write zeros so that the GEMM reads
-// defined data.
-template <int M, typename XT = __half>
+// Activation step of the direct form: the nine shifted copies of x.  V layout (of all activation kernels): [a*a][C][Pstride]
+// with the chunk-local tile index (p - p_begin) contiguous.  Threads past the last tile write zeros so that the GEMM
+// reads defined data.
 __global__ void __launch_bounds__(128)
-input_transform_kernel(const XT* __restrict__ x, __half* __restrict__ V, TileGeom geo, int C, long long p_begin,
-                       int p_count, long long Pstride, const float* __restrict__ amax) {
-    using Wm = Wino<M>;
-    constexpr int A = Wm::A;
+input_direct_kernel(const __half* __restrict__ x, __half* __restrict__ V, TileGeom geo, int C, long long p_begin,
+                    int p_count, long long Pstride) {
     // Wait first, release the GEMM second: once the GEMM runs, everything before this kernel has completed,
     // which is what lets it fetch its filters (written at the latest by the kernel before this one) early.
     pdl_wait();
@@ -361,54 +358,29 @@ input_transform_kernel(const XT* __restrict__ x, __half* __restrict__ V, TileGeo
     const int c = static_cast<int>(blockIdx.z * gridDim.y + blockIdx.y);   // grid.z continues grid.y past 65535
     if (pl >= p_count || c >= C) return;
     const long long p = p_begin + pl;
-    float d[A][A];
-    [[maybe_unused]] float xs = 1.f;
-    if constexpr (sizeof(XT) == 4) xs = scalbnf(1.f, -range_exponent(amax));
+    __half d[3][3];
+    int i0 = 0, j0 = 0;
+    const __half* img = x;
     if (p < geo.P) {
         int tw, th;
         long long n;
         decode_tile(geo, p, n, th, tw);
-        const XT* img = x + (n * C + c) * static_cast<long long>(geo.H) * geo.W;
-        const int step = M == 1 ? geo.stride : M;          // distance of neighbouring windows
-        const int i0 = step * th - 1, j0 = step * tw - 1;
+        img = x + (n * C + c) * static_cast<long long>(geo.H) * geo.W;
+        i0 = geo.stride * th - 1;
+        j0 = geo.stride * tw - 1;
+    }
 #pragma unroll
-        for (int r = 0; r < A; ++r) {
-            const int i = i0 + r;
-            const bool rin = (i >= 0) && (i < geo.H);
+    for (int r = 0; r < 3; ++r)
 #pragma unroll
-            for (int s = 0; s < A; ++s) {
-                const int j = j0 + s;
-                d[r][s] = (rin && j >= 0 && j < geo.W) ? to_f32(__ldg(img + static_cast<long long>(i) * geo.W + j))
-                                                        : 0.f;
-                if constexpr (sizeof(XT) == 4) d[r][s] *= xs;
-            }
+        for (int s = 0; s < 3; ++s) {
+            const int i = i0 + r, j = j0 + s;
+            const bool in = p < geo.P && i >= 0 && i < geo.H && j >= 0 && j < geo.W;
+            d[r][s] = in ? __ldg(img + static_cast<long long>(i) * geo.W + j) : __float2half_rn(0.f);
         }
-    } else {
-#pragma unroll
-        for (int r = 0; r < A; ++r)
-#pragma unroll
-            for (int s = 0; s < A; ++s) d[r][s] = 0.f;
-    }
-    // t = B^T d (column by column), v = t B (row by row)
-    float t[A][A];
-#pragma unroll
-    for (int s = 0; s < A; ++s) {
-        float col[A], o[A];
-#pragma unroll
-        for (int r = 0; r < A; ++r) col[r] = d[r][s];
-        mat_apply<A, A>(typename Wm::Bt{}, col, o);
-#pragma unroll
-        for (int r = 0; r < A; ++r) t[r][s] = o[r];
-    }
     const long long plane = static_cast<long long>(C) * Pstride;
     __half* dst = V + static_cast<long long>(c) * Pstride + pl;
 #pragma unroll
-    for (int r = 0; r < A; ++r) {
-        float o[A];
-        mat_apply<A, A>(typename Wm::Bt{}, t[r], o);
-#pragma unroll
-        for (int s = 0; s < A; ++s) dst[(r * A + s) * plane] = __float2half_rn(o[s]);
-    }
+    for (int t = 0; t < 9; ++t) dst[t * plane] = d[t / 3][t % 3];
 }
 
 // What follows the postprocess in the same kernel: y = act(A^T M A + bias + residual).  The paper's operator ends at
@@ -424,14 +396,10 @@ __device__ __forceinline__ float epilogue_act(float v, int act) {
     return act == 1 ? __fdividef(v, 1.f + __expf(-v)) : v;   // fast division: 2 ulp, far below the fp16 rounding that follows
 }
 
-// Postprocess + bias + cast + masked store.  Mws layout: [a*a][K][Pstride]; y is NCHW.
-template <int M, typename YT = __half>
+// Output step of the direct form: the nine partial sums, bias, cast.  Mws layout: [a*a][K][Pstride]; y is NCHW.
 __global__ void __launch_bounds__(128)
-output_transform_kernel(const __half* __restrict__ Mws, const YT* __restrict__ bias, YT* __restrict__ y,
-                        TileGeom geo, int K, long long p_begin, int p_count, long long Pstride, WtCheck chk,
-                        Epilogue ep) {
-    using Wm = Wino<M>;
-    constexpr int A = Wm::A;
+output_direct_kernel(const __half* __restrict__ Mws, const __half* __restrict__ bias, __half* __restrict__ y,
+                     TileGeom geo, int K, long long p_begin, int p_count, long long Pstride, WtCheck chk, Epilogue ep) {
     pdl_launch_dependents();
     // the header is older than the activation transform two kernels back, which waited for everything before
     // it: reading it before this kernel's own wait takes the load off the critical path
@@ -445,75 +413,19 @@ output_transform_kernel(const __half* __restrict__ Mws, const YT* __restrict__ b
     if (p >= geo.P) return;
     const long long plane = static_cast<long long>(K) * Pstride;
     const __half* src = Mws + static_cast<long long>(k) * Pstride + pl;
-    float mm[A][A];
+    float m[9];
 #pragma unroll
-    for (int r = 0; r < A; ++r)
+    for (int t = 0; t < 9; ++t) m[t] = __half2float(__ldg(src + t * plane));
+    float v = 0.f;
 #pragma unroll
-        for (int s = 0; s < A; ++s) mm[r][s] = __half2float(__ldg(src + (r * A + s) * plane));
-    // t = A^T mm (M x A), Y = t A (M x M)
-    float t[M][A];
-#pragma unroll
-    for (int s = 0; s < A; ++s) {
-        float col[A], o[M];
-#pragma unroll
-        for (int r = 0; r < A; ++r) col[r] = mm[r][s];
-        mat_apply<M, A>(typename Wm::At{}, col, o);
-#pragma unroll
-        for (int i = 0; i < M; ++i) t[i][s] = o[i];
-    }
+    for (int s = 0; s < 3; ++s) v += (m[s] + m[3 + s]) + m[6 + s];
     int tw, th;
     long long n;
     decode_tile(geo, p, n, th, tw);
-    const float b = load_bias(bias, k);
-    [[maybe_unused]] float ys = 1.f;
-    if constexpr (sizeof(YT) == 4) ys = scalbnf(1.f, range_exponent(ep.amax));
-    YT* img = y + (n * K + k) * static_cast<long long>(geo.H) * geo.W;
-    const int i0 = M * th, j0 = M * tw;
-    const bool vec_ok = ((geo.W & 1) == 0) && ((reinterpret_cast<uintptr_t>(y) & 3) == 0);
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-        float o[M];
-        mat_apply<M, A>(typename Wm::At{}, t[i], o);
-        const int oi = i0 + i;
-        if (oi >= geo.H) continue;
-        if constexpr (sizeof(YT) == 4) {   // fp32 output: no residual, no activation, no rounding
-            float* rowf = reinterpret_cast<float*>(img) + static_cast<long long>(oi) * geo.W + j0;
-            const float* resf = ep.residual ? static_cast<const float*>(ep.residual) + (rowf - reinterpret_cast<float*>(y))
-                                            : nullptr;
-#pragma unroll
-            for (int j = 0; j < M; ++j)
-                if (j0 + j < geo.W) {
-                    float v = fmaf(o[j], ys, b);
-                    if (resf) v += resf[j];
-                    rowf[j] = epilogue_act(v, ep.act);
-                }
-            continue;
-        } else {
-        __half* rowp = img + static_cast<long long>(oi) * geo.W + j0;
-        const __half* resp = ep.residual ? static_cast<const __half*>(ep.residual) + (rowp - y) : nullptr;
-        if constexpr (M == 1) {   // one output pixel per tile
-            float v0 = o[0] + b;
-            if (resp) v0 += __half2float(resp[0]);
-            rowp[0] = __float2half_rn(epilogue_act(v0, ep.act));
-        } else {
-#pragma unroll
-        for (int j = 0; j < M; j += 2) {
-            float v0 = o[j] + b, v1 = o[j + 1] + b;
-            if (resp) {
-                if (j0 + j < geo.W) v0 += __half2float(resp[j]);
-                if (j0 + j + 1 < geo.W) v1 += __half2float(resp[j + 1]);
-            }
-            const __half h0 = __float2half_rn(epilogue_act(v0, ep.act)), h1 = __float2half_rn(epilogue_act(v1, ep.act));
-            if (vec_ok && (j0 + j + 1 < geo.W)) {
-                *reinterpret_cast<__half2*>(rowp + j) = __halves2half2(h0, h1);
-            } else {
-                if (j0 + j < geo.W) rowp[j] = h0;
-                if (j0 + j + 1 < geo.W) rowp[j + 1] = h1;
-            }
-        }
-        }   // M > 1
-        }   // fp16 output
-    }
+    const long long o = (n * K + k) * static_cast<long long>(geo.H) * geo.W + static_cast<long long>(th) * geo.W + tw;
+    v += load_bias(bias, k);
+    if (ep.residual) v += __half2float(static_cast<const __half*>(ep.residual)[o]);
+    y[o] = __float2half_rn(epilogue_act(v, ep.act));
 }
 
 
@@ -522,7 +434,7 @@ output_transform_kernel(const __half* __restrict__ Mws, const YT* __restrict__ b
 // a thread owns TPT consecutive tiles of one tile row (m * TPT = 8 pixels), so each input or
 // output row segment is one aligned 16-byte access, the halo pixels left and right of it are two
 // scalar loads, and each transform position is stored / loaded as TPT packed fp16 values.
-// Arithmetic is fp32 as in the scalar kernels (the row and column passes run in the other order).
+// Arithmetic is fp32.  Other widths: transforms_any.cuh.
 // Requirements (checked by the host): W % 8 == 0, x / y 16-byte aligned, m * TPT == 8.
 // ---------------------------------------------------------------------------------------
 template <int N> struct PackedHalf;
@@ -1004,7 +916,7 @@ output_transform_vec_kernel(const __half* __restrict__ Mws, const YT* __restrict
                             TileGeom geo, int K, long long p_begin, FastDiv gdiv, long long Pstride, WtCheck chk,
                             Epilogue ep) {
     pdl_launch_dependents();
-    const bool wt_ok = wt_check(chk);   // before the wait: see output_transform_kernel
+    const bool wt_ok = wt_check(chk);   // before the wait: see output_direct_kernel
     pdl_wait();
     if (!wt_ok) return;
     output_unit_vec<M, TPT, EP, YT>(Mws, bias, y, geo, K, p_begin, gdiv, Pstride, blockIdx.x * blockDim.x + threadIdx.x, ep);
@@ -1145,7 +1057,7 @@ fused_small_c_kernel(const __half* __restrict__ x, const uint32_t* __restrict__ 
 //     2t, 2t+1 of the 16 x 64 block; channels past C and rows past K are stored as zeros);
 //   * after the 16 MMAs it holds all 16 positions of output channels g, g+8 for tiles 2t, 2t+1, so the
 //     output transform, bias and store stay in the lane.
-// About 2 instructions per output value against 90 for the scalar kernel above (which stays for F(4x4):
+// About 2 instructions per output value against 90 for the one-tile-per-thread kernel above (which stays for F(4x4):
 // 36 positions x 4 accumulators would not fit the registers).  tcgen05 is not used here: its smallest tile
 // (64 x 8 x 16 per instruction, operands staged in shared memory) does not pay for a contraction of 4.
 // ---------------------------------------------------------------------------------------

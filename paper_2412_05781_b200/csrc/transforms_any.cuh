@@ -1,0 +1,288 @@
+// Steps (i) and (iii) of Section "Techniques" for image widths that are not multiples of 8, and for pointers without
+// 16-byte alignment: the F(2x2) and F(4x4) transforms where no 16-byte access fits a row.
+//
+// As in the vector kernels a thread owns TWO consecutive tiles of V / M (an even index and the next one, wherever in
+// the image they lie: the pair may straddle a tile row or an image), so that V is stored and M is loaded as packed
+// pairs and the arithmetic runs in two-wide fp32.  With one tile per thread, 2-byte loads of x, 2-byte stores of V and
+// 2-byte stores of y -- each of them a partial write of its 32-byte sector -- both steps were bound by the number of
+// their accesses.
+//   activation: the six (four) pixels of a window row are cut out of the aligned 4-byte words that hold them.
+//   output: a warp gathers its output rows in shared memory and writes them with neighbouring lanes on neighbouring pixels.
+// Against one tile per thread (B200, whole layers, F(4x4), batch 1 or 2): 640->640 at 50x37 37.2 -> 31.7 us, 320->320 at
+// 113x89 55.8 -> 42.1, 512->512 at 180x148 107.9 -> 86.0, 256->256 at 324x300 156.7 -> 121.4 (activation step 74 -> 45 us,
+// output step 47.5 -> 45 us: instruction issue at half of the slots, DRAM at a third of its bandwidth).
+// Measured slower for the output: rows gathered by the whole CTA and copied as 16-byte pieces (two barriers per channel),
+// with M loaded by TMA or from the registers: 50-66 us on the last of these layers.
+#pragma once
+#include <cuda_fp16.h>
+
+#include <type_traits>
+
+#include "transforms.cuh"
+
+namespace sdw {
+
+template <int M>
+__device__ __forceinline__ void bt_packed(const float2 (&d)[M + 2], float2 (&o)[M + 2]) {
+    if constexpr (M == 4) {
+        bt4_packed(d, o);
+    } else {
+        o[0] = __ffma2_rn(f2s(-1.f), d[2], d[0]);
+        o[1] = __fadd2_rn(d[1], d[2]);
+        o[2] = __ffma2_rn(f2s(-1.f), d[1], d[2]);
+        o[3] = __ffma2_rn(f2s(-1.f), d[3], d[1]);
+    }
+}
+template <int M>
+__device__ __forceinline__ void at_packed(const float2 (&m)[M + 2], float2 (&o)[M]) {
+    if constexpr (M == 4) {
+        at4_packed(m, o);
+    } else {
+        o[0] = __fadd2_rn(__fadd2_rn(m[0], m[1]), m[2]);
+        o[1] = __ffma2_rn(f2s(-1.f), m[3], __ffma2_rn(f2s(-1.f), m[2], m[1]));
+    }
+}
+
+// Window rows of one tile, all A of them: row r in h[r] as A / 2 words of two pixels, zeros outside the image.  Every
+// word that is loaded holds at least one pixel of the row (the other one may lie outside: it shares the aligned word).
+// (Reading whole rows without these tests, masked afterwards, measured 5-8 % slower.)
+template <int M>
+__device__ __forceinline__ void load_window(const __half* __restrict__ img, const TileGeom& geo, int i0, int j0, bool valid,
+                                            uint32_t (&h)[M + 2][(M + 2) / 2]) {
+    constexpr int A = M + 2;
+    const int lo = j0 < 0 ? -j0 : 0;
+    const int hi = geo.W - j0 < A ? geo.W - j0 : A;
+    uint32_t mask[A / 2];
+#pragma unroll
+    for (int i = 0; i < A / 2; ++i)
+        mask[i] = (2 * i >= lo && 2 * i < hi ? 0x0000FFFFu : 0u) | (2 * i + 1 >= lo && 2 * i + 1 < hi ? 0xFFFF0000u : 0u);
+#pragma unroll
+    for (int r = 0; r < A; ++r) {
+        const bool row_ok = valid && static_cast<unsigned>(i0 + r) < static_cast<unsigned>(geo.H);
+        const uintptr_t a = reinterpret_cast<uintptr_t>(img) + (static_cast<long long>(i0 + r) * geo.W + j0) * 2;
+        const int par = static_cast<int>((a >> 1) & 1);
+        const uint32_t* wp = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
+        uint32_t w[A / 2 + 1];
+#pragma unroll
+        for (int i = 0; i <= A / 2; ++i) {
+            // word i holds the pixels 2 i - par and 2 i - par + 1 of the row
+            w[i] = 0u;
+            if (row_ok && 2 * i - par + 1 >= lo && 2 * i - par < hi) w[i] = __ldg(wp + i);
+        }
+        const uint32_t sel = par ? 0x5432u : 0x3210u;
+#pragma unroll
+        for (int i = 0; i < A / 2; ++i) h[r][i] = __byte_perm(w[i], w[i + 1], sel) & mask[i];
+    }
+}
+
+// Activation preprocess of the pair (p, p + 1) for one channel; p - p_begin even.  Tiles past the last one are zeros.
+template <int M, typename XT = __half>
+__global__ void __launch_bounds__(128)
+input_transform_any_kernel(const XT* __restrict__ x, __half* __restrict__ V, TileGeom geo, int C, long long p_begin,
+                           int p_count, long long Pstride, const float* __restrict__ amax) {
+    constexpr int A = M + 2;
+    const int pl = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x) * 2;
+    const int c = static_cast<int>(blockIdx.z * gridDim.y + blockIdx.y);   // grid.z continues grid.y past 65535
+    const long long hw = static_cast<long long>(geo.H) * geo.W;
+    int i0[2] = {0, 0}, j0[2] = {0, 0};
+    bool valid[2];
+    const XT* img[2] = {x, x};
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const long long p = p_begin + pl + t;
+        valid[t] = p < geo.P && pl < p_count && c < C;
+        if (valid[t]) {
+            int tw, th;
+            long long n;
+            decode_tile(geo, p, n, th, tw);
+            img[t] = x + (n * C + c) * hw;
+            i0[t] = M * th - 1;
+            j0[t] = M * tw - 1;
+        }
+    }
+    // Wait first, release the GEMM second (see input_direct_kernel); the index arithmetic needs nothing from memory.
+    pdl_wait();
+    pdl_launch_dependents();
+    if (pl >= p_count || c >= C) return;
+    float2 e2[A][A];   // rows transformed along the columns, (tile 0, tile 1)
+    if constexpr (sizeof(XT) == 2) {
+        uint32_t h0[A][A / 2], h1[A][A / 2];
+        load_window<M>(img[0], geo, i0[0], j0[0], valid[0], h0);
+        load_window<M>(img[1], geo, i0[1], j0[1], valid[1], h1);
+#pragma unroll
+        for (int r = 0; r < A; ++r) {
+            float2 d[A];
+#pragma unroll
+            for (int i = 0; i < A / 2; ++i) {
+                const uint32_t a = __byte_perm(h0[r][i], h1[r][i], 0x5410), b = __byte_perm(h0[r][i], h1[r][i], 0x7632);
+                d[2 * i] = __half22float2(*reinterpret_cast<const __half2*>(&a));
+                d[2 * i + 1] = __half22float2(*reinterpret_cast<const __half2*>(&b));
+            }
+            bt_packed<M>(d, e2[r]);
+        }
+    } else {
+        const float xs = scalbnf(1.f, -range_exponent(amax));
+#pragma unroll
+        for (int r = 0; r < A; ++r) {
+            float2 d[A];
+#pragma unroll
+            for (int s = 0; s < A; ++s) {
+                float v[2] = {0.f, 0.f};
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+                    if (valid[t] && static_cast<unsigned>(i0[t] + r) < static_cast<unsigned>(geo.H) &&
+                        static_cast<unsigned>(j0[t] + s) < static_cast<unsigned>(geo.W))
+                        v[t] = to_f32(__ldg(img[t] + static_cast<long long>(i0[t] + r) * geo.W + j0[t] + s));
+                d[s] = make_float2(v[0] * xs, v[1] * xs);
+            }
+            bt_packed<M>(d, e2[r]);
+        }
+    }
+    const long long plane = static_cast<long long>(C) * Pstride;
+    __half* dst = V + static_cast<long long>(c) * Pstride + pl;
+#pragma unroll
+    for (int nu = 0; nu < A; ++nu) {
+        float2 col[A], o[A];
+#pragma unroll
+        for (int r = 0; r < A; ++r) col[r] = e2[r][nu];
+        bt_packed<M>(col, o);
+#pragma unroll
+        for (int xi = 0; xi < A; ++xi) *reinterpret_cast<uint32_t*>(dst + (xi * A + nu) * plane) = pack2(o[xi].x, o[xi].y);
+    }
+}
+
+// Postprocess.  A warp owns 64 consecutive tiles, two per thread, and walks `steps` output channels.  Stored from the
+// registers, a warp's rows of eight pixels would leave as 4-byte or 2-byte pieces 16 bytes apart, each of them a partial
+// write of its sector; the output rows of the warp's tiles go through shared memory instead ([M][64 tiles][M pixels],
+// private to the warp) and leave with neighbouring lanes on neighbouring pixel pairs.
+constexpr int OUT_ANY_THREADS = 128;
+
+template <int M, bool EP, typename YT = __half>
+__global__ void __launch_bounds__(OUT_ANY_THREADS)
+output_transform_any_kernel(const __half* __restrict__ Mws, const YT* __restrict__ bias, YT* __restrict__ y, TileGeom geo,
+                            int K, long long p_begin, int p_count, long long Pstride, int steps, WtCheck chk, Epilogue ep) {
+    constexpr int A = M + 2;
+    constexpr int WORDS = M;                     // pixel pairs per thread and output row: 64 tiles * M pixels / 2 / 32
+    // with something to add after the convolution the gathered values are not rounded yet
+    using ST = typename std::conditional<EP || sizeof(YT) == 4, float, __half>::type;
+    __shared__ __align__(16) ST gather[OUT_ANY_THREADS / 32][M][64 * M];
+    pdl_launch_dependents();
+    const bool wt_ok = wt_check(chk);            // before the wait: see output_direct_kernel
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int pl0 = (static_cast<int>(blockIdx.x) * (OUT_ANY_THREADS / 32) + warp) * 64;     // first tile of the warp in the pass
+    const long long hw = static_cast<long long>(geo.H) * geo.W;
+    const int k_first = static_cast<int>(blockIdx.z * gridDim.y + blockIdx.y) * steps;       // grid.z continues grid.y
+    const int k_end = min(K, k_first + steps);
+    // the pixel pairs this lane stores: pair w = j * 32 + lane of a row of 64 * M pixels
+    long long off[WORDS];                        // first output row of the pair in channel 0 of its image
+    int rows[WORDS], cols[WORDS];                // rows of its tile inside the image; pixels of the pair inside it
+#pragma unroll
+    for (int j = 0; j < WORDS; ++j) {
+        const int px = (j * 32 + lane) * 2;
+        const long long p = p_begin + pl0 + px / M;
+        off[j] = 0;
+        rows[j] = cols[j] = 0;
+        if (pl0 < p_count && p < geo.P) {
+            int tw, th;
+            long long n;
+            decode_tile(geo, p, n, th, tw);
+            const int c = tw * M + (px & (M - 1));
+            off[j] = n * K * hw + static_cast<long long>(th) * M * geo.W + c;
+            rows[j] = geo.H - th * M;
+            cols[j] = geo.W - c;
+        }
+    }
+    pdl_wait();
+    if (!wt_ok || pl0 >= p_count) return;
+    [[maybe_unused]] float ys = 1.f;
+    if constexpr (sizeof(YT) == 4) ys = scalbnf(1.f, range_exponent(ep.amax));
+    const long long plane = static_cast<long long>(K) * Pstride;
+    ST(*g)[64 * M] = gather[warp];
+    for (int k = k_first; k < k_end; ++k) {
+        const __half* src = Mws + static_cast<long long>(k) * Pstride + pl0 + 2 * lane;
+        float2 tt[M][A];                         // A^T m, one column at a time; every float2 holds (tile 0, tile 1)
+#pragma unroll
+        for (int s = 0; s < A; ++s) {
+            float2 col[A], o[M];
+#pragma unroll
+            for (int r = 0; r < A; ++r) {
+                const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(src + (r * A + s) * plane));
+                col[r] = __half22float2(*reinterpret_cast<const __half2*>(&w));
+            }
+            at_packed<M>(col, o);
+#pragma unroll
+            for (int i = 0; i < M; ++i) tt[i][s] = o[i];
+        }
+        const float b = load_bias(bias, k);
+        __syncwarp();                            // the channel before has been read
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            float2 o[M];
+            at_packed<M>(tt[i], o);
+            float v[2][M];
+#pragma unroll
+            for (int j = 0; j < M; ++j) {
+                v[0][j] = sizeof(YT) == 4 ? fmaf(o[j].x, ys, b) : o[j].x + b;
+                v[1][j] = sizeof(YT) == 4 ? fmaf(o[j].y, ys, b) : o[j].y + b;
+            }
+            ST* q = &g[i][2 * lane * M];
+            if constexpr (sizeof(ST) == 2) {
+                if constexpr (M == 4)
+                    *reinterpret_cast<uint4*>(q) = make_uint4(pack2(v[0][0], v[0][1]), pack2(v[0][2], v[0][3]),
+                                                              pack2(v[1][0], v[1][1]), pack2(v[1][2], v[1][3]));
+                else
+                    *reinterpret_cast<uint2*>(q) = make_uint2(pack2(v[0][0], v[0][1]), pack2(v[1][0], v[1][1]));
+            } else {
+#pragma unroll
+                for (int j = 0; j < 2 * M; j += 4)
+                    *reinterpret_cast<float4*>(q + j) = make_float4(v[j / M][j % M], v[j / M][j % M + 1], v[(j + 2) / M][(j + 2) % M],
+                                                                    v[(j + 2) / M][(j + 2) % M + 1]);
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < WORDS; ++j) {
+            const long long o0 = off[j] + k * hw;
+            YT* yp = y + o0;
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                if (i >= rows[j]) continue;
+                YT* q = yp + i * geo.W;
+                if constexpr (sizeof(ST) == 2) {
+                    const uint32_t w = *reinterpret_cast<const uint32_t*>(&g[i][(j * 32 + lane) * 2]);
+                    if (cols[j] > 1 && (reinterpret_cast<uintptr_t>(q) & 2) == 0) {
+                        *reinterpret_cast<uint32_t*>(q) = w;
+                    } else {
+                        if (cols[j] > 0) *reinterpret_cast<unsigned short*>(q) = static_cast<unsigned short>(w);
+                        if (cols[j] > 1) *reinterpret_cast<unsigned short*>(q + 1) = static_cast<unsigned short>(w >> 16);
+                    }
+                } else {
+                    float2 v = *reinterpret_cast<const float2*>(&g[i][(j * 32 + lane) * 2]);
+                    if constexpr (EP) {
+                        if (ep.residual) {
+                            const YT* rp = static_cast<const YT*>(ep.residual) + o0 + i * geo.W;
+                            if (cols[j] > 0) v.x += to_f32(rp[0]);
+                            if (cols[j] > 1) v.y += to_f32(rp[1]);
+                        }
+                        v.x = epilogue_act(v.x, ep.act);
+                        v.y = epilogue_act(v.y, ep.act);
+                    }
+                    if constexpr (sizeof(YT) == 4) {
+                        if (cols[j] > 0) q[0] = v.x;
+                        if (cols[j] > 1) q[1] = v.y;
+                    } else {
+                        const __half2 h = __floats2half2_rn(v.x, v.y);
+                        if (cols[j] > 1 && (reinterpret_cast<uintptr_t>(q) & 2) == 0) {
+                            *reinterpret_cast<__half2*>(q) = h;
+                        } else {
+                            if (cols[j] > 0) q[0] = __low2half(h);
+                            if (cols[j] > 1) q[1] = __high2half(h);
+                        }
+                    }
+                }
+            }
+        }
+    }
+}
+
+}  // namespace sdw

@@ -1,0 +1,55 @@
+"""The transforms of any width (W % 8 != 0, or x / y without 16-byte alignment) where they can go wrong: pairs of tiles
+that straddle a tile row or an image, rows that begin at odd pixels, images narrower than a tile, the last pixels of the
+tensor, several output channels per CTA.  Bar: the parity bound 1e-2 * max|ref| (2.5e-3 for F(2x2)) against the fp64
+oracle, and nothing written outside y."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2412_05781_b200 import workloads
+from paper_2412_05781_b200.workloads import ConvLayer
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2412_05781_b200 import build_library
+    build_library()
+    from paper_2412_05781_b200 import binding
+    assert torch.cuda.is_available()
+    return binding
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("tile", [2, 4])
+@pytest.mark.parametrize("shape", [
+    # C, K, H, W, N
+    (9, 10, 5, 1, 3), (10, 9, 3, 2, 5), (12, 12, 7, 3, 2), (9, 16, 4, 5, 4), (16, 9, 9, 13, 3), (24, 40, 17, 31, 2),
+    (16, 24, 65, 63, 1), (9, 9, 33, 129, 1), (12, 10, 6, 257, 2), (16, 16, 8, 8, 2), (9, 1200, 19, 37, 2),
+])
+def test_any_width_and_alignment(B, shape, tile, offset):
+    C, K, H, W, N = shape
+    layer = ConvLayer(C=C, K=K, H=H, W=W, N=N)
+    x, w, b = workloads.make_inputs(layer, seed=sum(shape) + offset)
+    # x and y one element into their buffers: 2-byte aligned pointers, canaries around y
+    xb = torch.zeros(x.numel() + 1, dtype=torch.float16, device="cuda")
+    xb[offset:offset + x.numel()] = x.flatten().cuda()
+    n, pad = N * K * H * W, 64
+    canary = torch.full((n + 2 * pad + 1,), 1234.0, dtype=torch.float16, device="cuda")
+    xd, y = xb[offset:offset + x.numel()].view(x.shape), canary[pad + offset:pad + offset + n].view(N, K, H, W)
+    wT = B.sdwino_filter_transform(w.cuda(), tile)
+    ws = B.alloc_workspace(B.sdwino_workspace_bytes(N, C, H, W, K, tile))
+    B.sdwino_conv3x3(xd, wT, b.cuda(), K, tile, y=y, workspace=ws)
+    assert B.sdwino_last_device_status() == B.OK
+    ref = oracle.direct_conv3x3(x.numpy(), w.numpy(), b.numpy())
+    bound = (2.5e-3 if tile == 2 else 1e-2) * np.abs(ref).max()
+    assert np.abs(y.cpu().double().numpy() - ref).max() <= bound
+    assert bool((canary[:pad + offset] == 1234.0).all()) and bool((canary[pad + offset + n:] == 1234.0).all())
+    # with a residual and SiLU, which leave through the unrounded gather
+    res = torch.randn(N, K, H, W, generator=torch.Generator().manual_seed(1)).half()
+    B.sdwino_conv3x3_ex(xd, wT, b.cuda(), res.cuda(), K, tile, B.ACT_SILU, ws, y=y)
+    refe = oracle.epilogue(ref, res.numpy(), "silu")
+    assert np.abs(y.cpu().double().numpy() - refe).max() <= 1e-2 * np.abs(refe).max()
+    assert bool((canary[:pad + offset] == 1234.0).all()) and bool((canary[pad + offset + n:] == 1234.0).all())
