@@ -818,7 +818,7 @@ int launch_gemm_shape(const CUtensorMap& tmU, const CUtensorMap& tmV, const CUte
     const int grid = static_cast<int>(tiles < workers ? tiles : workers) * CTAS;
     ProfScope prof(KIND_GEMM, st);
     const cudaError_t e =
-        launch_pdl(wino_gemm_kernel<CTAS, RES, DUAL, false, U8, STM>, dim3(grid), dim3(GEMM_LAUNCH_THREADS),
+        launch_pdl(wino_gemm_kernel<CTAS, RES, DUAL, false, U8, STM>, dim3(grid), dim3(U8 ? GEMM_U8_THREADS : GEMM_LAUNCH_THREADS),
                    static_cast<size_t>(L::dyn_bytes(RES ? 0 : prm.n_tile / CTAS, prm.stages, prm.epi_rows,
                                                     prm.epi_alias ? 0 : prm.epi_bufs,
                                                     RES ? prm.num_c_blocks * L::b_bytes(prm.n_tile)
@@ -1169,6 +1169,12 @@ int conv_impl(const void* x, const void* wT, const void* bias, void* y, int N, i
     if (q8) {
         // 8-bit filters: give up one operand stage (down to three at least) for a ring of raw filter boxes, which is
         // what keeps the weight stream from HBM deep: a raw slot is a third of an operand stage or less
+        // The epilogue stages 32 channels at a time where that divides its half of the tile: the rings are short of memory
+        // (2560->1280 at 26x45, batch 4, n_tile 256: 155-176 -> 138 us; 16 at a time, for n_tile 160, costs 3-8 %).
+        if (!prm.epi_alias && prm.epi_rows > 32 && prm.epi_rows % 32 == 0) {
+            prm.epi_chunks = prm.epi_rows / 32;
+            prm.epi_rows = 32;
+        }
         const int room = MAX_DYN_SMEM - GemmSmemLayout::dyn_bytes(b_rows, 0, prm.epi_rows, prm.epi_alias ? 0 : prm.epi_bufs);
         const int raw = GemmSmemLayout::raw_bytes(b_rows), stage = GemmSmemLayout::stage_bytes(b_rows);
         int best_s = 0, best_r = 0;
