@@ -142,9 +142,17 @@ def _check(status: int, where: str) -> None:
         raise SdwinoError(status, where)
 
 
+# The current stream as the integer it is: making a torch.cuda.Stream object of it first costs 3 us, a third of what a whole
+# convolution call costs the host (three kernel launches, 9 us).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -250,6 +258,9 @@ def sdwino_profile_records(capacity: int = 1 << 16, keep: bool = False):
 def alloc_workspace(nbytes: int, device="cuda") -> torch.Tensor:
     """Device scratch of `nbytes` bytes (torch allocations are at least 512-byte aligned;
     the returned view starts on a 1024-byte boundary)."""
+    buf = torch.empty(nbytes, dtype=torch.uint8, device=device)
+    if buf.data_ptr() % 1024 == 0:
+        return buf
     buf = torch.empty(nbytes + 1024, dtype=torch.uint8, device=device)
     off = (-buf.data_ptr()) % 1024
     return buf[off:off + nbytes]
@@ -258,8 +269,8 @@ def alloc_workspace(nbytes: int, device="cuda") -> torch.Tensor:
 def sdwino_filter_transform(w: torch.Tensor, tile: int, stream=None) -> torch.Tensor:
     """w: fp16 CUDA [K, C, 3, 3] contiguous -> wT (opaque uint8 CUDA tensor, tile-specific)."""
     assert w.is_cuda and w.dtype == torch.float16 and w.is_contiguous() and w.dim() == 4
-    K, C = int(w.shape[0]), int(w.shape[1])
-    assert tuple(w.shape[2:]) == (3, 3)
+    K, C, R, S = w.shape
+    assert R == 3 and S == 3
     nbytes = sdwino_filter_bytes(K, C, tile)
     if nbytes == 0:
         raise SdwinoError(ERR_UNSUPPORTED if tile not in (1, 2, 4) else ERR_INVALID_ARG, "sdwino_filter_bytes")
@@ -273,7 +284,7 @@ def sdwino_set_workspace(workspace: Optional[torch.Tensor]) -> None:
     if workspace is None:
         _check(lib.sdwino_set_workspace(None, 0), "sdwino_set_workspace")
     else:
-        _check(lib.sdwino_set_workspace(workspace.data_ptr(), workspace.numel() * workspace.element_size()),
+        _check(lib.sdwino_set_workspace(workspace.data_ptr(), workspace.nbytes),
                "sdwino_set_workspace")
 
 
@@ -283,10 +294,10 @@ def sdwino_conv3x3(x: torch.Tensor, wT: torch.Tensor, bias: Optional[torch.Tenso
     """x: fp16 CUDA [N, C, H, W]; returns y fp16 [N, K, H, W].  With `workspace=None` the scratch
     registered by sdwino_set_workspace is used."""
     assert x.is_cuda and x.dtype == torch.float16 and x.is_contiguous() and x.dim() == 4
-    N, C, H, W = (int(v) for v in x.shape)
+    N, C, H, W = x.shape
     if y is None:
         y = torch.empty((N, K, H, W), dtype=torch.float16, device=x.device)
-    assert y.is_contiguous() and y.dtype == torch.float16 and tuple(y.shape) == (N, K, H, W)
+    assert y.is_contiguous() and y.dtype == torch.float16 and y.shape == (N, K, H, W)
     if bias is not None:
         assert bias.is_cuda and bias.dtype == torch.float16 and bias.numel() == K and bias.is_contiguous()
     if workspace is None:
@@ -294,7 +305,7 @@ def sdwino_conv3x3(x: torch.Tensor, wT: torch.Tensor, bias: Optional[torch.Tenso
                                 _stream_ptr(stream))
     else:
         rc = lib.sdwino_conv3x3_ws(x.data_ptr(), wT.data_ptr(), _ptr(bias), y.data_ptr(), N, C, H, W, K, tile,
-                                   workspace.data_ptr(), workspace.numel() * workspace.element_size(),
+                                   workspace.data_ptr(), workspace.nbytes,
                                    _stream_ptr(stream))
     _check(rc, "sdwino_conv3x3")
     return y
@@ -309,10 +320,10 @@ def sdwino_conv3x3_ex(x: torch.Tensor, wT: torch.Tensor, bias: Optional[torch.Te
     """y = act(conv3x3(x) + bias + residual): residual fp16 CUDA [N, K, H, W] or None (may be y itself),
     activation ACT_NONE or ACT_SILU."""
     assert x.is_cuda and x.dtype == torch.float16 and x.is_contiguous() and x.dim() == 4
-    N, C, H, W = (int(v) for v in x.shape)
+    N, C, H, W = x.shape
     if y is None:
         y = torch.empty((N, K, H, W), dtype=torch.float16, device=x.device)
-    assert y.is_contiguous() and y.dtype == torch.float16 and tuple(y.shape) == (N, K, H, W)
+    assert y.is_contiguous() and y.dtype == torch.float16 and y.shape == (N, K, H, W)
     if bias is not None:
         assert bias.is_cuda and bias.dtype == torch.float16 and bias.numel() == K and bias.is_contiguous()
     if residual is not None:
@@ -320,7 +331,7 @@ def sdwino_conv3x3_ex(x: torch.Tensor, wT: torch.Tensor, bias: Optional[torch.Te
         assert tuple(residual.shape) == (N, K, H, W)
     rc = lib.sdwino_conv3x3_ex(x.data_ptr(), wT.data_ptr(), _ptr(bias), _ptr(residual), y.data_ptr(), N, C, H, W, K,
                                tile, int(activation), workspace.data_ptr(),
-                               workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+                               workspace.nbytes, _stream_ptr(stream))
     _check(rc, "sdwino_conv3x3_ex")
     return y
 
@@ -328,8 +339,8 @@ def sdwino_conv3x3_ex(x: torch.Tensor, wT: torch.Tensor, bias: Optional[torch.Te
 def sdwino_filter_transform_f32(w: torch.Tensor, tile: int, stream=None) -> torch.Tensor:
     """w: fp32 CUDA [K, C, 3, 3] contiguous -> wT (the same opaque buffer sdwino_filter_transform makes)."""
     assert w.is_cuda and w.dtype == torch.float32 and w.is_contiguous() and w.dim() == 4
-    K, C = int(w.shape[0]), int(w.shape[1])
-    assert tuple(w.shape[2:]) == (3, 3)
+    K, C, R, S = w.shape
+    assert R == 3 and S == 3
     nbytes = sdwino_filter_bytes(K, C, tile)
     if nbytes == 0:
         raise SdwinoError(ERR_UNSUPPORTED if tile not in (1, 2, 4) else ERR_INVALID_ARG, "sdwino_filter_bytes")
@@ -345,15 +356,15 @@ def sdwino_conv3x3_f32(x: torch.Tensor, wT: torch.Tensor, bias: Optional[torch.T
     """The convolution with fp32 x [N, C, H, W], bias [K] (or None) and y [N, K, H, W].  scaled=True calls
     sdwino_conv3x3_f32_scaled: activations of any fp32 magnitude."""
     assert x.is_cuda and x.dtype == torch.float32 and x.is_contiguous() and x.dim() == 4
-    N, C, H, W = (int(v) for v in x.shape)
+    N, C, H, W = x.shape
     if y is None:
         y = torch.empty((N, K, H, W), dtype=torch.float32, device=x.device)
-    assert y.is_cuda and y.is_contiguous() and y.dtype == torch.float32 and tuple(y.shape) == (N, K, H, W)
+    assert y.is_cuda and y.is_contiguous() and y.dtype == torch.float32 and y.shape == (N, K, H, W)
     if bias is not None:
         assert bias.is_cuda and bias.dtype == torch.float32 and bias.numel() == K and bias.is_contiguous()
     fn = lib.sdwino_conv3x3_f32_scaled if scaled else lib.sdwino_conv3x3_f32
     rc = fn(x.data_ptr(), wT.data_ptr(), _ptr(bias), y.data_ptr(), N, C, H, W, K, tile,
-            workspace.data_ptr(), workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+            workspace.data_ptr(), workspace.nbytes, _stream_ptr(stream))
     _check(rc, "sdwino_conv3x3_f32_scaled" if scaled else "sdwino_conv3x3_f32")
     return y
 
@@ -363,10 +374,10 @@ def sdwino_conv3x3_f32_ex(x: torch.Tensor, wT: torch.Tensor, bias: Optional[torc
                           stream=None) -> torch.Tensor:
     """y = act(conv3x3(x) + bias + residual) with fp32 tensors (residual may be y itself)."""
     assert x.is_cuda and x.dtype == torch.float32 and x.is_contiguous() and x.dim() == 4
-    N, C, H, W = (int(v) for v in x.shape)
+    N, C, H, W = x.shape
     if y is None:
         y = torch.empty((N, K, H, W), dtype=torch.float32, device=x.device)
-    assert y.is_cuda and y.is_contiguous() and y.dtype == torch.float32 and tuple(y.shape) == (N, K, H, W)
+    assert y.is_cuda and y.is_contiguous() and y.dtype == torch.float32 and y.shape == (N, K, H, W)
     if bias is not None:
         assert bias.is_cuda and bias.dtype == torch.float32 and bias.numel() == K and bias.is_contiguous()
     if residual is not None:
@@ -374,7 +385,7 @@ def sdwino_conv3x3_f32_ex(x: torch.Tensor, wT: torch.Tensor, bias: Optional[torc
         assert tuple(residual.shape) == (N, K, H, W)
     rc = lib.sdwino_conv3x3_f32_ex(x.data_ptr(), wT.data_ptr(), _ptr(bias), _ptr(residual), y.data_ptr(), N, C, H, W, K,
                                    tile, int(activation), workspace.data_ptr(),
-                                   workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+                                   workspace.nbytes, _stream_ptr(stream))
     _check(rc, "sdwino_conv3x3_f32_ex")
     return y
 
@@ -389,8 +400,8 @@ def sdwino_conv3x3_static(x: torch.Tensor, wT: torch.Tensor, bias: Optional[torc
     nothing either.  Layers whose smallest pass does not fit the STATIC_SCRATCH_BYTES array raise
     SdwinoError(ERR_WORKSPACE).  Calls share the array, so do not let two of them overlap on the GPU."""
     assert x.is_cuda and x.dtype == torch.float16 and x.is_contiguous() and x.dim() == 4
-    N, C, H, W = (int(v) for v in x.shape)
-    assert y.is_cuda and y.is_contiguous() and y.dtype == torch.float16 and tuple(y.shape) == (N, K, H, W)
+    N, C, H, W = x.shape
+    assert y.is_cuda and y.is_contiguous() and y.dtype == torch.float16 and y.shape == (N, K, H, W)
     rc = lib.sdwino_conv3x3_static(x.data_ptr(), wT.data_ptr(), _ptr(bias), y.data_ptr(), N, C, H, W, K, tile,
                                    _stream_ptr(stream))
     _check(rc, "sdwino_conv3x3_static")
@@ -413,11 +424,11 @@ def sdwino_conv3x3_host(x: torch.Tensor, wT: torch.Tensor, bias: Optional[torch.
     enqueued: y is complete after sdwino_host_join(stream) and a synchronisation of the stream."""
     assert not x.is_cuda and not y.is_cuda and x.dtype == torch.float16 and y.dtype == torch.float16
     assert x.is_contiguous() and y.is_contiguous()
-    N, C, H, W = (int(v) for v in x.shape)
+    N, C, H, W = x.shape
     K = int(y.shape[1])
     fn = lib.sdwino_conv3x3_host if wait else lib.sdwino_conv3x3_host_async
     rc = fn(x.data_ptr(), wT.data_ptr(), _ptr(bias), y.data_ptr(), N, C, H, W, K, tile,
-            workspace.data_ptr(), workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+            workspace.data_ptr(), workspace.nbytes, _stream_ptr(stream))
     _check(rc, "sdwino_conv3x3_host" if wait else "sdwino_conv3x3_host_async")
     return y
 
@@ -428,11 +439,11 @@ def sdwino_conv3x3_host_f32(x: torch.Tensor, wT: torch.Tensor, bias: Optional[to
     sdwino_host_staging_bytes_f32(...) in front of the scratch."""
     assert not x.is_cuda and not y.is_cuda and x.dtype == torch.float32 and y.dtype == torch.float32
     assert x.is_contiguous() and y.is_contiguous() and (bias is None or bias.dtype == torch.float32)
-    N, C, H, W = (int(v) for v in x.shape)
+    N, C, H, W = x.shape
     K = int(y.shape[1])
     fn = lib.sdwino_conv3x3_host_f32 if wait else lib.sdwino_conv3x3_host_f32_async
     rc = fn(x.data_ptr(), wT.data_ptr(), _ptr(bias), y.data_ptr(), N, C, H, W, K, tile,
-            workspace.data_ptr(), workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+            workspace.data_ptr(), workspace.nbytes, _stream_ptr(stream))
     _check(rc, "sdwino_conv3x3_host_f32" if wait else "sdwino_conv3x3_host_f32_async")
     return y
 
@@ -456,12 +467,12 @@ def sdwino_conv3x3_q8(x: torch.Tensor, wTq: torch.Tensor, bias: Optional[torch.T
                       workspace: torch.Tensor, y: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """The convolution with an 8-bit transformed filter (fp16 x, bias, y)."""
     assert x.is_cuda and x.dtype == torch.float16 and x.is_contiguous() and x.dim() == 4
-    N, C, H, W = (int(v) for v in x.shape)
+    N, C, H, W = x.shape
     if y is None:
         y = torch.empty((N, K, H, W), dtype=torch.float16, device=x.device)
-    assert y.is_cuda and y.is_contiguous() and y.dtype == torch.float16 and tuple(y.shape) == (N, K, H, W)
+    assert y.is_cuda and y.is_contiguous() and y.dtype == torch.float16 and y.shape == (N, K, H, W)
     rc = lib.sdwino_conv3x3_q8(x.data_ptr(), wTq.data_ptr(), _ptr(bias), y.data_ptr(), N, C, H, W, K, tile,
-                               workspace.data_ptr(), workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+                               workspace.data_ptr(), workspace.nbytes, _stream_ptr(stream))
     _check(rc, "sdwino_conv3x3_q8")
     return y
 
@@ -474,13 +485,13 @@ def sdwino_conv3x3_direct(x: torch.Tensor, wT: torch.Tensor, bias: Optional[torc
                           workspace: torch.Tensor, y: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """The direct 3x3 convolution (pad 1) with stride 1 or 2: wT from sdwino_filter_transform(w, 1)."""
     assert x.is_cuda and x.dtype == torch.float16 and x.is_contiguous() and x.dim() == 4
-    N, C, H, W = (int(v) for v in x.shape)
+    N, C, H, W = x.shape
     Ho, Wo = (H - 1) // max(stride, 1) + 1, (W - 1) // max(stride, 1) + 1
     if y is None:
         y = torch.empty((N, K, Ho, Wo), dtype=torch.float16, device=x.device)
     assert y.is_cuda and y.is_contiguous() and y.dtype == torch.float16 and tuple(y.shape) == (N, K, Ho, Wo)
     rc = lib.sdwino_conv3x3_direct(x.data_ptr(), wT.data_ptr(), _ptr(bias), y.data_ptr(), N, C, H, W, K, stride,
-                                   workspace.data_ptr(), workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+                                   workspace.data_ptr(), workspace.nbytes, _stream_ptr(stream))
     _check(rc, "sdwino_conv3x3_direct")
     return y
 
@@ -491,8 +502,8 @@ def make_sequence(layers) -> "ctypes.Array":
     arr = (SdwinoLayer * len(layers))()
     for d, (x, wT, bias, y, K, tile) in zip(arr, layers):
         assert x.is_cuda and x.dtype == torch.float16 and x.is_contiguous() and x.dim() == 4
-        N, C, H, W = (int(v) for v in x.shape)
-        assert y.is_cuda and y.dtype == torch.float16 and y.is_contiguous() and tuple(y.shape) == (N, K, H, W)
+        N, C, H, W = x.shape
+        assert y.is_cuda and y.dtype == torch.float16 and y.is_contiguous() and y.shape == (N, K, H, W)
         d.x, d.wT, d.bias, d.y = x.data_ptr(), wT.data_ptr(), _ptr(bias), y.data_ptr()
         d.N, d.C, d.H, d.W, d.K, d.tile = N, C, H, W, K, tile
     return arr
@@ -505,6 +516,6 @@ def sdwino_workspace_bytes_sequence(seq) -> int:
 def sdwino_conv3x3_sequence(seq, workspace: torch.Tensor, prefetch_bytes: int = 0, stream=None) -> None:
     """Runs the layers of `seq` (see make_sequence) in order on `stream`; prefetch_bytes > 0 also sends that much of each
     layer's filters towards L2 while the layer before it computes."""
-    rc = lib.sdwino_conv3x3_sequence(seq, len(seq), workspace.data_ptr(), workspace.numel() * workspace.element_size(),
+    rc = lib.sdwino_conv3x3_sequence(seq, len(seq), workspace.data_ptr(), workspace.nbytes,
                                      prefetch_bytes, _stream_ptr(stream))
     _check(rc, "sdwino_conv3x3_sequence")
