@@ -744,65 +744,71 @@ int launch_fused_small_c_mma(const T* x, const void* wT, const T* bias, T* y, co
     return e == cudaSuccess ? SDWINO_OK : err_cuda(__LINE__);
 }
 
-// Shape of the GEMM launch: CTA pairs or single CTAs, and the output channels per tile (UMMA N, a
-// multiple of 16 up to 256).  The candidate with the smallest modelled time wins: a tile costs its
-// pipeline stages, each limited by the tensor pipe (2 n cycles per stage) or by the bytes the CTA must
-// fetch from L2 per stage (about 40 bytes per cycle per SM were measured), plus an epilogue that is
-// hidden unless the tile is short; tiles run in waves over the SMs.
+// The epilogue staging of a GEMM shape and the stages that fit beside it.  Two groups of epilogue warps each take half a
+// tile when that is a multiple of 16 channels.  The ring is short of stages against its round trip (a stage's loads take
+// 2-3.5 thousand cycles to arrive under load, its MMAs 300-500): a group that stages its channels 64 or 32 at a time
+// instead of all at once leaves room for one more stage in most shapes.  Measured: CTA pairs at n_tile 256 go from five to
+// six stages, 1280->1280 at 64x64 (batch 2) 63.8 -> 58.3 us, 512->512 at 512x512 363 -> 345 us; 16 at a time costs more in
+// the epilogue than the stage returns (320->320 at 128x128: 28 -> 35 us).
+struct EpiPlan { int rows, bufs, chunks, stages; };
+EpiPlan plan_epilogue(int n_tile, int ctas, bool dual, bool alias, bool chunked) {
+    const int b_rows = n_tile / ctas;
+    const bool split = (n_tile / 2) % 16 == 0;
+    const int grp = split ? n_tile / 2 : n_tile, bufs = split ? 2 : 1;
+    const int stage = GemmSmemLayout::stage_bytes(b_rows) + (dual ? GemmSmemLayout::A_BYTES : 0);
+    auto stages_for = [&](int rows) {
+        const int st = (MAX_DYN_SMEM - GemmSmemLayout::dyn_bytes(b_rows, 0, rows, alias ? 0 : bufs)) / stage;
+        return st > GEMM_MAX_STAGES ? GEMM_MAX_STAGES : st;
+    };
+    EpiPlan e{grp, bufs, 1, stages_for(grp)};
+    for (int rows = 64; rows >= 32 && chunked && !alias; rows >>= 1)
+        if (rows < grp && grp % rows == 0 && stages_for(rows) > e.stages) e = EpiPlan{rows, bufs, grp / rows, stages_for(rows)};
+    return e;
+}
+
+// Shape of the GEMM launch: CTA pairs or single CTAs, one or two blocks of 128 tiles per CTA tile, and the output channels
+// per tile (UMMA N, a multiple of 16 up to 256).  The candidate with the smallest modelled time (cycles) wins: a tile costs
+// its pipeline stages, each limited by the tensor pipe or by the bytes the CTA fetches from L2 per stage, more with a ring
+// of few stages, plus an epilogue that is hidden unless the tile is short; tiles run in waves over the SMs.
 //
-// A CTA pair fetches half of the filter rows per CTA.  Measured over the layers of all workloads it is 4-10 % faster
-// for the layer where the mainloop dominates (C >= 512, several waves of 256-channel tiles), and slower where
-// tiles are short (its epilogue hand-off crosses two CTAs), where an odd number of 128-tile blocks leaves half a
-// pair idle, and for short launches (it runs without programmatic dependent launch, see launch_gemm_shape).  The
-// constants below reproduce that: 35 bytes per cycle per CTA of a pair (on the scale where a single CTA gets 40),
-// epilogue x 1.35 and a fixed charge for the lost overlap.
+// The constants are a fit to 91 layers of the UNet and VAE sweeps (batch 1-8, ragged sizes among them), each timed with every
+// shape: the choice is on average 0.4 % slower than the best shape of a layer, at most 5 %.  What the fit says: a single
+// CTA takes in 41 bytes per cycle, a CTA of a pair 34; a stage missing from a ring of four (pairs: five) costs 7.5 %
+// (n_tile 224 fits three: 1280->640 at 48x48, batch 4, 79.8 us with it, 69.0 with 160); a pair costs 9500 cycles per launch
+// more (it runs without programmatic dependent launch, see launch_gemm_shape; 512->512 at 128x128 44.6 us as pairs, 41.1
+// as single CTAs), and its epilogue, which crosses two CTAs, 1.66 times as much; tiles of fewer than 8 stages and launches
+// of one or two tiles per pair measured 4-35 % slower as pairs and are not offered.  Two blocks of tiles per CTA
+// tile (see wino_gemm.cuh) share a filter box, but their epilogues are added to the mainloop.
 struct GemmShape { int ctas; int n_tile; int dual; };   // dual: two blocks of 128 tiles per CTA tile (single CTAs)
 GemmShape choose_gemm_shape(int K, int C, long long p_tiles128, int a2, int sms, int force_ctas) {
     const long long cblocks = (C + GEMM_BLOCK_C - 1) / GEMM_BLOCK_C;
     GemmShape best{1, 16, 0};
     double best_cost = 1e300;
-    // a pair needs two blocks of 128 tiles; with fewer than 8 stages per tile it measured 4-35 % slower
     const int max_ctas = p_tiles128 >= 2 && (cblocks >= 8 || force_ctas == 2) ? 2 : 1;
-    for (int ctas = 1; ctas <= max_ctas; ++ctas) {
+    for (int kind = 0; kind < 3; ++kind) {            // single CTAs, CTA pairs, single CTAs with two blocks of tiles
+        const int ctas = kind == 1 ? 2 : 1;
+        const bool dual = kind == 2;
+        if (ctas > max_ctas || (dual && (force_ctas != 0 || p_tiles128 < 2))) continue;
         if (force_ctas != 0 && ctas != (force_ctas < max_ctas ? force_ctas : max_ctas)) continue;
-        const long long p_tiles = (p_tiles128 + ctas - 1) / ctas;
+        const int blocks = kind == 0 ? 1 : 2;         // blocks of 128 tiles per tile of the launch
+        const long long p_tiles = (p_tiles128 + blocks - 1) / blocks;
         const long long workers = sms / ctas;
-        const int step = 16 * ctas;   // each CTA of a pair loads whole 16-row blocks
-        for (int n = step; n <= GEMM_MAX_N; n += step) {
+        const int step = 16 * ctas;                   // each CTA of a pair loads whole 16-row blocks
+        for (int n = step; n <= (dual ? 192 : GEMM_MAX_N); n += step) {
             const long long ktiles = (K + n - 1) / n;
-            if (n > step && (ktiles == (K + n - step - 1) / (n - step))) continue;  // a smaller n needs as many tiles
+            if (n > step && ktiles == (K + n - step - 1) / (n - step)) continue;  // a smaller n needs as many tiles
             const long long tiles = ktiles * p_tiles * a2;
             const long long waves = (tiles + workers - 1) / workers;
-            // with one or two tiles per pair the fixed cost of a pair is not paid back (measured 9-12 % slower)
             if (ctas == 2 && force_ctas != 2 && waves < 3) continue;
-            const double mma = 2.0 * n;
-            const double load = ctas == 1 ? (GemmSmemLayout::A_BYTES + 128.0 * n) / 40.0
-                                          : (GemmSmemLayout::A_BYTES + 64.0 * n) / 35.0;
-            const double main = cblocks * (mma > load ? mma : load);
-            const double epi = (300.0 + 14.0 * n) * (ctas == 2 ? 1.35 : 1.0);
-            const double per_tile = (main > epi ? main : epi) + (ctas == 2 ? 400.0 : 200.0);
-            const double fixed = ctas == 2 ? 7000.0 : 0.0;
-            const double cost = waves * per_tile + epi + fixed;
-            if (cost < best_cost) { best_cost = cost; best = GemmShape{ctas, n, 0}; }
-        }
-    }
-    // Single CTAs with two blocks of 128 tiles per CTA tile (see wino_gemm.cuh): the filter box is fetched once per
-    // 256 tiles and there are half as many CTA tiles, but the accumulators are not double-buffered across tiles, so
-    // the epilogues of a tile are added to its mainloop.  n_tile up to 192 leaves room for three stages.
-    // Taken for layers of 2 to 15 blocks of tiles (larger ones have the filter-resident mode and CTA pairs).
-    if (force_ctas == 0 && p_tiles128 >= 2 && p_tiles128 < 16) {
-        const long long p_tiles = (p_tiles128 + 1) / 2;
-        for (int n = 16; n <= 192; n += 16) {
-            const long long ktiles = (K + n - 1) / n;
-            if (n > 16 && (ktiles == (K + n - 17) / (n - 16))) continue;
-            const long long tiles = ktiles * p_tiles * a2;
-            const long long waves = (tiles + sms - 1) / sms;
-            const double mma = 4.0 * n;
-            const double load = (2.0 * GemmSmemLayout::A_BYTES + 128.0 * n) / 40.0;
-            const double main = cblocks * (mma > load ? mma : load);
-            const double epi = 300.0 + 14.0 * n;
-            const double cost = 1.08 * waves * (main + 2.0 * epi + 200.0);   // measured gains are 5-10 %, not the modelled 20
-            if (cost < best_cost) { best_cost = cost; best = GemmShape{1, n, 1}; }
+            const int stages = plan_epilogue(n, ctas, dual, ctas == 1 && tiles <= sms, true).stages;
+            const double ring = 1.0 + 0.075 * std::max(0, (ctas == 1 ? 4 : 5) - stages);
+            const double mma = 2.0 * n * (dual ? 2 : 1);
+            const double load = ((dual ? 2.0 : 1.0) * GemmSmemLayout::A_BYTES + 128.0 / ctas * n) / (ctas == 1 ? 41.4 : 34.2);
+            const double main = cblocks * std::max(mma, load) * ring;
+            const double epi = (310.0 + 19.6 * n) * (ctas == 2 ? 1.66 : 1.0);
+            const double cost = dual ? 1.01 * waves * (main + 2.0 * epi + 200.0)
+                                     : waves * (std::max(main, epi) + (ctas == 2 ? 460.0 : 200.0)) + epi + (ctas == 2 ? 9500.0 : 0.0);
+            if (cost < best_cost) { best_cost = cost; best = GemmShape{ctas, n, dual ? 1 : 0}; }
         }
     }
     return best;
@@ -1229,25 +1235,10 @@ int conv_impl(const void* x, const void* wT, const void* bias, void* y, int N, i
     }
 
     if (!prm.resident && !prm.epi_alias && !q8 && force_ctas == 0 && force_n_tile == 0) {
-        // The ring is short of stages against its round trip (a stage's loads take 2-3.5 thousand cycles to arrive
-        // under load, its MMAs 300-500): an epilogue group that stages its channels 64 or 32 at a time instead of all
-        // at once leaves room for one more stage in most shapes.  Measured: CTA pairs at n_tile 256 go from five to
-        // six stages, 1280->1280 at 64x64 (batch 2) 63.8 -> 58.3 us, 512->512 at 512x512 363 -> 345 us; 16 at a time
-        // costs more in the epilogue than the stage returns (320->320 at 128x128: 28 -> 35 us).
-        const int stage = GemmSmemLayout::stage_bytes(b_rows) + (shape.dual ? GemmSmemLayout::A_BYTES : 0);
-        auto stages_for = [&](int rows) {
-            const int st = (MAX_DYN_SMEM - GemmSmemLayout::dyn_bytes(b_rows, 0, rows, prm.epi_bufs)) / stage;
-            return st > GEMM_MAX_STAGES ? GEMM_MAX_STAGES : st;
-        };
-        const int grp = prm.epi_rows;
-        int best_rows = grp, best_stages = stages_for(grp);
-        for (int rows = 64; rows >= 32; rows >>= 1) {
-            if (rows >= grp || grp % rows != 0) continue;
-            if (stages_for(rows) > best_stages) { best_stages = stages_for(rows); best_rows = rows; }
-        }
-        prm.epi_chunks = grp / best_rows;
-        prm.epi_rows = best_rows;
-        prm.stages = best_stages;
+        const EpiPlan e = plan_epilogue(prm.n_tile, shape.ctas, shape.dual != 0, false, true);
+        prm.epi_chunks = e.chunks;
+        prm.epi_rows = e.rows;
+        prm.stages = e.stages;
     }
     // Epilogue staging: stmatrix into swizzled boxes where a CTA has several tiles (throughput: 3-8 % on those GEMMs),
     // plain 2-byte stores into one box where it has one (its two TMA stores of 128-byte rows drain later at the tail
