@@ -72,10 +72,12 @@ input_transform_f4_tma_kernel(const __grid_constant__ CUtensorMap tmX, __half* _
     int steps = (prm.C - c_first + prm.cpb - 1) / prm.cpb;
     steps = steps < prm.steps ? steps : prm.steps;
 
-    if (tid == 0) {
-        for (int s = 0; s < IN_TMA_STAGES; ++s) mbar_init(&full_bar[s], 1);
-        abort_flag = 0;
+    if (tid < IN_TMA_STAGES) {
+        mbar_init(&full_bar[tid], 1);
         fence_barrier_init();
+    }
+    if (tid == 32) {
+        abort_flag = 0;
         prefetch_tmap(&tmX);
     }
     __syncthreads();

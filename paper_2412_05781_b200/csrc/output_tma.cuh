@@ -37,10 +37,12 @@ output_transform_f4_tma_kernel(const __grid_constant__ CUtensorMap tmM, const YT
     const int tid = threadIdx.x;
     pdl_launch_dependents();
     const bool wt_ok = wt_check(chk);   // before the wait: see output_direct_kernel
-    if (tid == 0) {
-        for (int s = 0; s < OUT_TMA_STAGES; ++s) mbar_init(&full_bar[s], 1);
-        abort_flag = 0;
+    if (tid < OUT_TMA_STAGES) {
+        mbar_init(&full_bar[tid], 1);
         fence_barrier_init();
+    }
+    if (tid == 32) {
+        abort_flag = 0;
         prefetch_tmap(&tmM);
     }
     __syncthreads();

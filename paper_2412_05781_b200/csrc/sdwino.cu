@@ -766,6 +766,9 @@ EpiPlan plan_epilogue(int n_tile, int ctas, bool dual, bool alias, bool chunked)
     return e;
 }
 
+// Accumulators of n_tile columns in the 512 columns of tensor memory, for two blocks of tiles per CTA tile.
+int dual_acc_bufs(int n_tile) { return std::max(2, std::min(GEMM_MAX_ACC, 2 * GEMM_MAX_N / n_tile)); }
+
 // Shape of the GEMM launch: CTA pairs or single CTAs, one or two blocks of 128 tiles per CTA tile, and the output channels
 // per tile (UMMA N, a multiple of 16 up to 256).  The candidate with the smallest modelled time (cycles) wins: a tile costs
 // its pipeline stages, each limited by the tensor pipe or by the bytes the CTA fetches from L2 per stage, more with a ring
@@ -806,7 +809,9 @@ GemmShape choose_gemm_shape(int K, int C, long long p_tiles128, int a2, int sms,
             const double load = ((dual ? 2.0 : 1.0) * GemmSmemLayout::A_BYTES + 128.0 / ctas * n) / (ctas == 1 ? 41.4 : 34.2);
             const double main = cblocks * std::max(mma, load) * ring;
             const double epi = (310.0 + 19.6 * n) * (ctas == 2 ? 1.66 : 1.0);
-            const double cost = dual ? 1.01 * waves * (main + 2.0 * epi + 200.0)
+            const int acc = dual_acc_bufs(n);
+            const double dual_tile = acc == 4 ? std::max(main, 2.0 * epi) : (acc == 3 ? std::max(main, epi) + epi : main + 2.0 * epi);
+            const double cost = dual ? 1.04 * (waves * (dual_tile + 200.0) + (acc - 2) * epi)
                                      : waves * (std::max(main, epi) + (ctas == 2 ? 460.0 : 200.0)) + epi + (ctas == 2 ? 9500.0 : 0.0);
             if (cost < best_cost) { best_cost = cost; best = GemmShape{ctas, n, dual ? 1 : 0}; }
         }
@@ -966,6 +971,8 @@ int launch_pipeline(const __half* x, const void* wT, const __half* bias, __half*
     prm.group = pq.group;
     prm.epi_alias = 0;
     prm.dual = 0;
+    prm.acc_bufs = 2;
+    prm.acc_stride = GEMM_MAX_N;
     prm.p_stride = ring_p;
     prm.scales = nullptr;
     prm.kpad = pl.Kb * 16;
@@ -1151,6 +1158,8 @@ int conv_impl(const void* x, const void* wT, const void* bias, void* y, int N, i
     const int b_rows = prm.n_tile / shape.ctas;
     if (force_n_tile != 0) shape.dual = 0;
     prm.dual = shape.dual;
+    prm.acc_bufs = dual_acc_bufs(prm.n_tile);
+    prm.acc_stride = prm.acc_bufs == 2 ? GEMM_MAX_N : prm.n_tile;
     // epilogue staging: two groups of epilogue warps each take half a tile when that is a multiple of 16 channels
     const bool split = (prm.n_tile / 2) % 16 == 0;
     prm.epi_rows = split ? prm.n_tile / 2 : prm.n_tile;

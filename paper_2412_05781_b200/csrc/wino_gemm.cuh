@@ -25,8 +25,13 @@
 // issues one MMA per block of 128 tiles into the two accumulator buffers, which the epilogue then drains one after
 // the other.  The filter box is fetched once per 256 instead of once per 128 tiles (like a CTA pair, but on one SM
 // and with programmatic dependent launch), and a layer of 2 j blocks of tiles makes half as many CTA tiles, which
-// turns two waves into one where the tiles number about twice the SMs.  The accumulators are no longer
-// double-buffered across tiles, so this pays where a CTA has one or two tiles or many stages per tile.
+// turns two waves into one where the tiles number about twice the SMs.
+// Tensor memory holds as many accumulators of n_tile columns as fit 512 (four up to 128 channels, three up to 160): with
+// four the epilogues of a tile overlap the next tile as in the other modes, with three all but the first of them, with two
+// (n_tile 176, 192) none.  The middle sizes are bound by the bytes that cross from L2: 320->320 at 96x96 (batch 4) reads
+// 233 MB at the 16 TB/s that L2 delivers and writes 53 MB at 7.3 in 23.5 us (14.8 without the writes); a tile of two blocks
+// reads a quarter fewer.  1920->1280 at 24x24 (batch 4) 61.0 -> 59.8 us with the third accumulator, 1280->640 at 64x64
+// (batch 2) 51.3 -> 50.1.
 //
 // One persistent CTA (pair) per SM (pair) walks the list of (pos, k-tile, p-tile) output tiles.
 //   warp 0   : TMA producer        (one lane)
@@ -60,13 +65,14 @@ constexpr int PIPE_THREADS = GEMM_THREADS + PIPE_TRANSFORM_THREADS;
 constexpr int GEMM_U8_GROUP_WARPS = 4;    // 8-bit filters: warps 10-17 expand the filter bytes, two groups on alternate steps
 constexpr int GEMM_U8_THREADS = GEMM_THREADS + 2 * GEMM_U8_GROUP_WARPS * 32 + 32;   // ... and warp 18: producer of the raw boxes
 constexpr int GEMM_MAX_STAGES = 8;
+constexpr int GEMM_MAX_ACC = 4;       // accumulators in tensor memory (two, except with two blocks of tiles per CTA tile)
 constexpr uint64_t GEMM_WAIT_LIMIT_NS = 2000000000ull;  // a wait longer than 2 s is reported, not spun on
 
 struct GemmSmemLayout {
     static constexpr int A_BYTES = GEMM_BLOCK_P * GEMM_BLOCK_C * 2;          // two [64 p][64 c] boxes
     static constexpr int A_BOX_BYTES = 64 * GEMM_BLOCK_C * 2;
     static constexpr int EPI_ROW_BYTES = GEMM_BLOCK_P * 2;                   // one staged row: 128 p fp16
-    static constexpr int BAR_BYTES = (4 * GEMM_MAX_STAGES + 6) * 8 + 16 + 16;   // barriers, two words, four item slots
+    static constexpr int BAR_BYTES = (4 * GEMM_MAX_STAGES + 2 * GEMM_MAX_ACC + 2) * 8 + 16 + 16;   // barriers, two words, four item slots
     // `rows` = rows of U this CTA loads per stage: n_tile (single CTA) or n_tile / 2 (CTA pair)
     __host__ __device__ static constexpr int b_bytes(int rows) { return rows * GEMM_BLOCK_C * 2; }
     __host__ __device__ static constexpr int stage_bytes(int rows) {
@@ -110,6 +116,8 @@ struct GemmParams {
     int group;         // filter-resident mode: CTAs that share out the tiles of one (position, k-tile) pair
     int epi_alias;     // 1: no CTA has more than one tile, so the epilogue stages its rows in the (by then idle) first
                        // pipeline stages instead of a buffer of its own, which leaves room for one more stage
+    int acc_bufs;      // accumulators in tensor memory and their distance in columns (only used with dual)
+    int acc_stride;
     int dual;          // 1: the kernel instantiation with two blocks of 128 tiles per CTA tile (host side only)
     long long p_stride;  // tiles per pass (row pitch of V and M)
     const float* scales; // 8-bit filters: S[pos][kpad], the factor of every (position, output channel) row
@@ -240,8 +248,8 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                                                      (prm.epi_alias ? 0 : L::epi_bytes(prm.epi_rows, prm.epi_bufs)));
     uint64_t* empty_bar = full_bar + GEMM_MAX_STAGES;
     uint64_t* acc_full_bar = empty_bar + GEMM_MAX_STAGES;
-    uint64_t* acc_empty_bar = acc_full_bar + 2;
-    uint64_t* ures_full_bar = acc_empty_bar + 2;     // the resident filter block has arrived
+    uint64_t* acc_empty_bar = acc_full_bar + GEMM_MAX_ACC;
+    uint64_t* ures_full_bar = acc_empty_bar + GEMM_MAX_ACC;     // the resident filter block has arrived
     uint64_t* ures_empty_bar = ures_full_bar + 1;    // the MMAs that read it have completed
     uint64_t* raw_full_bar = ures_empty_bar + 1;     // 8-bit filters: the bytes of a raw slot have arrived
     uint64_t* raw_empty_bar = raw_full_bar + GEMM_MAX_STAGES;   // ... and have been expanded
@@ -255,6 +263,8 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
     const int lane = threadIdx.x & 31;
     const int num_tiles = prm.num_k_tiles * prm.num_p_tiles * prm.num_pos;
     constexpr uint32_t TMEM_COLS = 2 * GEMM_MAX_N;
+    const int acc_bufs = DUAL ? prm.acc_bufs : 2;
+    const int acc_stride = DUAL ? prm.acc_stride : GEMM_MAX_N;
     // The tiles of this worker, numbered i = 0 .. my_count - 1.  Streaming mode: every num_workers-th tile of the
     // list.  Filter-resident mode: the workers form groups of `group` CTAs; a group takes every num_groups-th
     // (position, k-tile) pair and its CTAs share out the tiles p of the pair round-robin, so that a CTA stays with
@@ -299,23 +309,20 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
         }
     };
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < stages; ++s) {
-            mbar_init(&full_bar[s], U8 ? 1 + GEMM_U8_GROUP_WARPS : (SPLIT ? 2 : 1));   // 8-bit filters: the producer of V and a group
-            mbar_init(&empty_bar[s], 1);
-        }
-        for (int s = 0; s < GEMM_MAX_STAGES; ++s) {
-            mbar_init(&raw_full_bar[s], 1);
-            mbar_init(&raw_empty_bar[s], GEMM_U8_GROUP_WARPS);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&acc_full_bar[b], 1);
-            mbar_init(&acc_empty_bar[b], 8 * CTAS);   // one arrival per epilogue warp of every CTA
-        }
-        mbar_init(ures_full_bar, 1);
-        mbar_init(ures_empty_bar, 1);
-        *abort_flag = 0;
+    // One thread per barrier: this stands before the first load of the launch (with one thread for all of them, four more
+    // accumulator barriers made the launches of one tile per CTA 0.5 us longer).
+    if (threadIdx.x < 4 * GEMM_MAX_STAGES + 2 * GEMM_MAX_ACC + 2) {
+        const int b = threadIdx.x;                     // in the order of the pointers above
+        constexpr int ACC = 2 * GEMM_MAX_STAGES, URES = ACC + 2 * GEMM_MAX_ACC, RAW_EMPTY = URES + 2 + GEMM_MAX_STAGES;
+        uint32_t count = 1;
+        if (b < GEMM_MAX_STAGES) count = U8 ? 1 + GEMM_U8_GROUP_WARPS : (SPLIT ? 2 : 1);   // 8-bit filters: the producer of V and a group
+        else if (b >= ACC + GEMM_MAX_ACC && b < URES) count = 8 * CTAS;                    // one arrival per epilogue warp of every CTA
+        else if (b >= RAW_EMPTY) count = GEMM_U8_GROUP_WARPS;
+        mbar_init(&full_bar[b], count);
         fence_barrier_init();
+    }
+    if (threadIdx.x == GEMM_THREADS) {
+        *abort_flag = 0;
         prefetch_tmap(&tmU);
         prefetch_tmap(&tmV);
         prefetch_tmap(&tmM);
@@ -581,13 +588,15 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                     }
                 }
                 ok = mbar_wait_warp(&acc_empty_bar[buf], acc_phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
-                if constexpr (DUAL) {   // this tile fills both accumulator buffers
-                    if (ok) ok = mbar_wait_warp(&acc_empty_bar[1], acc_phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                [[maybe_unused]] const int buf1 = buf + 1 == acc_bufs ? 0 : buf + 1;
+                if constexpr (DUAL) {   // this tile fills two accumulators
+                    const uint32_t phase1 = buf1 == 0 ? acc_phase ^ 1u : acc_phase;
+                    if (ok) ok = mbar_wait_warp(&acc_empty_bar[buf1], phase1 ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                 }
                 if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 2, cta_rank); break; }
                 tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * GEMM_MAX_N);
-                [[maybe_unused]] const uint32_t d_tmem1 = tmem_base + static_cast<uint32_t>(GEMM_MAX_N);
+                const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * acc_stride);
+                [[maybe_unused]] const uint32_t d_tmem1 = tmem_base + static_cast<uint32_t>(buf1 * acc_stride);
                 [[maybe_unused]] constexpr uint64_t a_sub = static_cast<uint64_t>(L::A_BYTES >> 4);   // second block of tiles
                 for (int cb = 0; cb < prm.num_c_blocks; ++cb) {
                     if (!__all_sync(0xffffffffu, mbar_try_wait_a32(full_a, phase))) {
@@ -641,18 +650,15 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                 if (elected) {
                     if constexpr (CTAS == 2) umma_commit_pair(&acc_full_bar[buf]);
                     else umma_commit(&acc_full_bar[buf]);
-                    if constexpr (DUAL) umma_commit(&acc_full_bar[1]);
+                    if constexpr (DUAL) umma_commit(&acc_full_bar[buf1]);
                 }
                 // the last tile of a run: once its MMAs have completed the resident filters may be replaced
                 if (resident && elected && i + 1 < my_count &&
                     static_cast<int>(fast_div(static_cast<uint32_t>(tile_of(i + 1)), prm.fd_p)) != key)
                     umma_commit(ures_empty_bar);
-                if constexpr (DUAL) {
-                    acc_phase ^= 1u;          // both buffers were used: buf stays 0
-                } else {
-                    buf ^= 1;
-                    if (buf == 0) acc_phase ^= 1u;
-                }
+#pragma unroll
+                for (int u = 0; u < PT; ++u)
+                    if (++buf == acc_bufs) { buf = 0; acc_phase ^= 1u; }
             }
             if (!ok) *abort_flag = 1;
         }
@@ -666,7 +672,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
         uint32_t acc_phase = 0;
         // the accumulator-empty barrier of a pair lives in the leader
         const uint32_t acc_empty_addr0 = CTAS == 2 ? map_to_cta(smem_u32(&acc_empty_bar[0]), 0) : 0u;
-        // one iteration per accumulator: a tile of two blocks of 128 tiles p (DUAL) fills both buffers, which are
+        // one iteration per accumulator: a tile of two blocks of 128 tiles p (DUAL) fills two, which are
         // drained in turn exactly as two consecutive tiles would be
         int stg_seq = 0;                       // pieces staged so far by this group (selects the staging buffer)
         [[maybe_unused]] int pend_pt = -1;     // pipelined mode, group_tid 0: block whose stores are to be announced
@@ -693,7 +699,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
             }
             tc_fence_after_sync();
             const uint32_t t_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) +
-                                    static_cast<uint32_t>(buf * GEMM_MAX_N);
+                                    static_cast<uint32_t>(buf * acc_stride);
             const int p0 = ((PIPE ? pt % pp.ring : pt * CTAS) + static_cast<int>(cta_rank)) * GEMM_BLOCK_P + quarter * 32;
             const int k0 = kt * prm.n_tile;
             const bool p_ok = p0 < prm.p_stride;   // the second CTA of the last pair may hang over the pass
@@ -859,8 +865,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                 if constexpr (CTAS == 2) mbar_arrive_cluster(acc_empty_addr0 + static_cast<uint32_t>(buf) * 8u);
                 else mbar_arrive(&acc_empty_bar[buf]);
             }
-            buf ^= 1;
-            if (buf == 0) acc_phase ^= 1u;
+            if (++buf == acc_bufs) { buf = 0; acc_phase ^= 1u; }
         }
         if (group_tid == 0) {
             tma_store_wait_all();
