@@ -93,6 +93,12 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
     if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
     return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort_flag, limit_ns)) != 0;
 }
+// ... with the barrier's shared-memory address at hand as well.
+__device__ __forceinline__ bool mbar_wait_warp_a32(uint32_t bar_a, uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                                   uint64_t limit_ns) {
+    if (__all_sync(0xffffffffu, mbar_try_wait_a32(bar_a, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort_flag, limit_ns)) != 0;
+}
 
 // ---- TMA --------------------------------------------------------------------
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* m) {
@@ -109,6 +115,13 @@ __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* m
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
         ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z)
         : "memory");
+}
+// Untiled copy of `bytes` contiguous bytes into shared memory, completion counted on an mbarrier; both addresses and the
+// size are multiples of 16.
+__device__ __forceinline__ void bulk_load_a32(uint32_t smem_dst, const void* gptr, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_dst),
+                 "l"(gptr), "r"(bytes), "r"(bar)
+                 : "memory");
 }
 // The same with shared-memory addresses already converted (the producer is a single thread and
 // keeps them as running 32-bit values).
@@ -223,6 +236,16 @@ __device__ __forceinline__ void tmem_ld_32x16_sync(uint32_t taddr, uint32_t (&r)
         "tcgen05.wait::ld.sync.aligned;"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
+
+// The same for 8 columns.
+__device__ __forceinline__ void tmem_ld_32x8_sync(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
         : "r"(taddr)
         : "memory");
 }

@@ -21,6 +21,7 @@
 #include "fused_small_k.cuh"
 #include "input_tma.cuh"
 #include "output_tma.cuh"
+#include "direct_conv.cuh"
 
 namespace {
 
@@ -192,13 +193,13 @@ CUresult encode_tiled(CUtensorMap* m, cuuint32_t rank, const void* base, const c
 }
 
 // fp16 tensor [d2][d1][d0] (d0 contiguous, row pitch `pitch0` elements, plane pitch `pitch1`
-// elements) with a {b0, b1, 1} box, with the 128-byte swizzle or none.  Encoding costs about a
+// elements) with a {b0, b1, b2} box, with the 128-byte swizzle or none.  Encoding costs about a
 // microsecond of host time, so the last few maps are kept (a map depends only on these arguments).
 struct MapKey {
-    const void* base; uint64_t d0, d1, d2, pitch0, pitch1; uint32_t b0, b1; bool sw;
+    const void* base; uint64_t d0, d1, d2, pitch0, pitch1; uint32_t b0, b1; bool sw; uint32_t b2 = 1;
     bool operator==(const MapKey& o) const {
         return base == o.base && d0 == o.d0 && d1 == o.d1 && d2 == o.d2 && pitch0 == o.pitch0 && pitch1 == o.pitch1 &&
-               b0 == o.b0 && b1 == o.b1 && sw == o.sw;
+               b0 == o.b0 && b1 == o.b1 && sw == o.sw && b2 == o.b2;
     }
 };
 struct MapSlot { MapKey key; CUtensorMap map; bool used = false; };
@@ -207,17 +208,17 @@ MapSlot g_map_cache[MAP_CACHE_SLOTS];
 std::mutex g_map_mutex;
 
 bool encode_map_uncached(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t pitch0,
-                         uint64_t pitch1, uint32_t b0, uint32_t b1, bool swizzle128);
+                         uint64_t pitch1, uint32_t b0, uint32_t b1, bool swizzle128, uint32_t b2);
 
 bool encode_map(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t pitch0,
-                uint64_t pitch1, uint32_t b0, uint32_t b1, bool swizzle128) {
-    const MapKey key{base, d0, d1, d2, pitch0, pitch1, b0, b1, swizzle128};
+                uint64_t pitch1, uint32_t b0, uint32_t b1, bool swizzle128, uint32_t b2 = 1) {
+    const MapKey key{base, d0, d1, d2, pitch0, pitch1, b0, b1, swizzle128, b2};
     uint64_t h = reinterpret_cast<uintptr_t>(base) >> 8;
     h = h * 1000003u ^ d0 * 31u ^ d1 * 131u ^ pitch0 * 7u ^ (static_cast<uint64_t>(b1) << 20) ^ (b0 << 3) ^ swizzle128;
     MapSlot& slot = g_map_cache[h % MAP_CACHE_SLOTS];
     std::lock_guard<std::mutex> lock(g_map_mutex);
     if (slot.used && slot.key == key) { *m = slot.map; return true; }
-    if (!encode_map_uncached(m, base, d0, d1, d2, pitch0, pitch1, b0, b1, swizzle128)) return false;
+    if (!encode_map_uncached(m, base, d0, d1, d2, pitch0, pitch1, b0, b1, swizzle128, b2)) return false;
     slot.key = key;
     slot.map = *m;
     slot.used = true;
@@ -225,10 +226,10 @@ bool encode_map(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint
 }
 
 bool encode_map_uncached(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t pitch0,
-                         uint64_t pitch1, uint32_t b0, uint32_t b1, bool swizzle128) {
+                         uint64_t pitch1, uint32_t b0, uint32_t b1, bool swizzle128, uint32_t b2) {
     cuuint64_t dims[3] = {d0, d1, d2};
     cuuint64_t strides[2] = {pitch0 * sizeof(__half), pitch1 * sizeof(__half)};
-    cuuint32_t box[3] = {b0, b1, 1};
+    cuuint32_t box[3] = {b0, b1, b2};
     cuuint32_t estr[3] = {1, 1, 1};
     const CUresult r = encode_tiled(m, 3, base, dims, strides, box, estr,
                                     swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE);
@@ -1033,6 +1034,213 @@ int launch_pipeline(const __half* x, const void* wT, const __half* bias, __half*
     return e == cudaSuccess ? SDWINO_OK : err_cuda(__LINE__);
 }
 
+// ---- the direct convolution (tile 1) as an implicit GEMM: see direct_conv.cuh ----
+// Taken instead of the three steps from this many output pixels on.  Below, too few tiles of 128 pixels are left for the
+// SMs: stride 2 (times in us, three steps / this), 1280 -> 1280 128 pixels 13.9 / 20, 320 -> 320 512 pixels 9.8 / 10.6,
+// 640 -> 640 512 pixels 14.1 / 14.4, 64 -> 96 625 pixels 7.6 / 7.5, 320 -> 320 1024 pixels 12.9 / 12.0, 1280 -> 1280 1024
+// pixels 48.9 / 40; stride 1, 128 pixels 13.7 / 17, 512 pixels 9.9 / 9.3 (320) and 14.1 / 12.3 (640).
+// Channels come in blocks of 64, padded with zeros, so it also wants half a block.
+constexpr int DIRECT_MIN_CHANNELS = 32;
+bool use_direct_conv(const Plan& pl, int N, int C, int stride) {
+    return C >= DIRECT_MIN_CHANNELS && static_cast<long long>(N) * pl.Ho * pl.Wo >= (stride == 1 ? 512 : 640);
+}
+
+struct DirectShape { int flat, n_tile, splits; };   // n_tile 0: none
+
+// Fills the geometry of a candidate; false where its patch does not fit in shared memory or an index in 32 bits.
+bool direct_geometry(const Plan& pl, int N, int C, int H, int W, int K, int stride, const DirectShape& sh, DirectParams* q) {
+    q->N = N; q->C = C; q->H = H; q->W = W; q->K = K;
+    q->Ho = pl.Ho; q->Wo = pl.Wo; q->stride = stride;
+    q->n_tile = sh.n_tile;
+    q->num_k_tiles = (K + sh.n_tile - 1) / sh.n_tile;
+    q->num_cb = (C + 63) / 64;
+    q->splits = sh.splits;
+    q->cb_per_split = (q->num_cb + sh.splits - 1) / sh.splits;
+    q->flat = sh.flat;
+    const int halo = stride == 1 ? 2 : 1;
+    long long pp, num_m;
+    q->rows_img = pl.Ho + 1;
+    q->pk_pitch = pl.Wo + 1;
+    q->pk_pieces = q->num_cb * 8;
+    q->lead = 0;
+    q->tiles_c = q->tiles_r = 1;
+    const long long positions = static_cast<long long>(N) * q->rows_img * q->pk_pitch;
+    if (positions + 4096 >= (1ll << 31)) return false;
+    if (sh.flat) {
+        q->pitch = q->pk_pitch;
+        if (stride == 1) q->lead = q->pitch + 1;
+        pp = 128ll + static_cast<long long>(halo) * (q->pitch + 1);
+        num_m = (positions - q->pitch + 127) / 128;   // the last row is padding
+        q->sbo = 8;
+        q->pk_positions = (num_m - 1) * 128 + pp;         // what the last patch reads
+    } else {
+        q->pitch = 8 + halo;
+        pp = (16 + halo) * static_cast<long long>(q->pitch);
+        q->tiles_c = (pl.Wo + 7) / 8;
+        q->tiles_r = (pl.Ho + 15) / 16;
+        num_m = static_cast<long long>(N) * q->tiles_c * q->tiles_r;
+        q->sbo = q->pitch;
+        q->pk_positions = positions;
+    }
+    if (pp > 1024 || num_m * q->num_k_tiles * sh.splits >= (1ll << 30) || q->pk_positions >= (1ll << 31) - 256 ||
+        q->pk_pieces > 65535)
+        return false;
+    q->PP = static_cast<int>(pp);
+    q->num_m = static_cast<int>(num_m);
+    q->planes = stride == 1 ? 1 : 4;
+    q->a_stage_bytes = q->PP * 128;
+    // a patch serves all nine taps (two stages hide its latency), with stride 2 one to four of them (as many stages as
+    // leave half of the memory to the filters)
+    const int room = MAX_DYN_SMEM - 1024 - DC_BAR_BYTES - DC_EPI_WARPS * DC_STG_BYTES;
+    q->a_stages = stride == 1 ? 2 : std::max(2, std::min(DC_MAX_A_STAGES, room / 2 / q->a_stage_bytes));
+    const int b_room = room - q->a_stages * q->a_stage_bytes;
+    q->b_stages = b_room > 0 ? std::min(DC_MAX_B_STAGES, b_room / (sh.n_tile * 128)) : 0;
+    return q->b_stages >= 2;
+}
+// What only the shape that is launched needs: the divisors.
+void direct_finish(DirectParams* q) {
+    q->fd_pitch = make_fastdiv(static_cast<uint32_t>(q->pitch));
+    q->fd_rows = make_fastdiv(static_cast<uint32_t>(q->rows_img));
+    q->fd_k = make_fastdiv(static_cast<uint32_t>(q->num_k_tiles));
+    q->fd_s = make_fastdiv(static_cast<uint32_t>(q->splits));
+    q->fd_tc = make_fastdiv(static_cast<uint32_t>(q->tiles_c));
+    q->fd_tr = make_fastdiv(static_cast<uint32_t>(q->tiles_r));
+    q->fd_pkp = make_fastdiv(static_cast<uint32_t>(q->pk_pitch));
+}
+
+size_t direct_packed_bytes(const DirectParams& q) {
+    return (static_cast<size_t>(q.planes) * q.pk_pieces * q.pk_positions * 16 + WS_ALIGN - 1) / WS_ALIGN * WS_ALIGN;
+}
+size_t direct_part_bytes(const DirectParams& q) {   // of one (pixel tile, k tile) pair
+    return q.splits > 1 ? static_cast<size_t>(q.splits) * q.n_tile * 512 : 0;
+}
+
+// Modelled cycles of a candidate, fitted to 24 layers with 16 to 50 shapes each (the shape it picks is within 3 % of the
+// fastest on all of them): a tap costs its four MMAs (n / 2 cycles each, at least 52) and what stands around them; a
+// channel of the epilogue 4 as fp32 parts, 12 as 16-byte pieces of y, 49 as single values; parts are read once more.
+double direct_cost(const DirectParams& q, bool vec, int sms) {
+    const double main = q.cb_per_split * 9.0 * (4.0 * std::max(q.n_tile / 2.0, 52.0) + 29.0);
+    const double epi = 650.0 + q.n_tile * (q.splits > 1 ? 4.0 : (vec ? 12.0 : 49.0));
+    const long long items = static_cast<long long>(q.num_m) * q.num_k_tiles * q.splits;
+    const long long waves = (items + sms - 1) / sms;
+    const double cost = waves * std::max(main, epi) + epi;
+    return q.splits == 1 ? cost : cost + 2300.0 + static_cast<double>(items) * q.n_tile * 512.0 / 2000.0;
+}
+
+// The cheapest modelled shape; n_tile == 0 where none fits.  It depends on the layer alone and not on the workspace that was
+// passed (the order of the sums, and with it the bits, follow from it): parts may take what a one-pass workspace has
+// beside the packed copy.  Some hundred candidates are looked at, so the last choices are kept (by the layer's sizes).
+DirectShape choose_direct_shape(const Plan& pl, int N, int C, int H, int W, int K, int stride, int sms) {
+    struct Slot { int key[7]; DirectShape shape; bool used; };
+    static Slot slots[64];
+    static std::mutex mutex;
+    const int key[7] = {N, C, H, W, K, stride, sms};
+    uint64_t h = 0;
+    for (int v : key) h = h * 1000003u + static_cast<uint32_t>(v);
+    Slot& slot = slots[(h >> 7) % 64];
+    {
+        std::lock_guard<std::mutex> lock(mutex);
+        if (slot.used && std::equal(key, key + 7, slot.key)) return slot.shape;
+    }
+    const size_t full = static_cast<size_t>(tiles_per_pass(pl, static_cast<size_t>(-1) / 2)) * pl.per_tile;
+    DirectShape best{0, 0, 0};
+    double best_cost = 1e300;
+    const int num_cb = (C + 63) / 64;
+    DirectParams q;
+    for (int flat = 0; flat < 2; ++flat)
+        for (int n = 16; n <= 256; n += 16) {
+            const int ktiles = (K + n - 1) / n;
+            if (n > 16 && ktiles == (K + n - 17) / (n - 16)) continue;   // a smaller n needs as many tiles
+            for (int s = 1; s <= num_cb && s <= 16; ++s) {
+                const int per = (num_cb + s - 1) / s;
+                if ((num_cb + per - 1) / per != s) continue;             // a smaller s has parts as long
+                const DirectShape sh{flat, n, s};
+                if (!direct_geometry(pl, N, C, H, W, K, stride, sh, &q)) break;
+                const long long pairs = static_cast<long long>(q.num_m) * ktiles;
+                if (s > 1 && (pairs * (s - 1) >= 2ll * sms || direct_packed_bytes(q) + pairs * direct_part_bytes(q) > full))
+                    break;
+                const double cost = direct_cost(q, !flat && pl.Wo % 8 == 0, sms);
+                if (cost < best_cost) { best_cost = cost; best = sh; }
+            }
+        }
+    std::lock_guard<std::mutex> lock(mutex);
+    std::copy(key, key + 7, slot.key);
+    slot.shape = best;
+    slot.used = true;
+    return best;
+}
+
+template <int STRIDE>
+int launch_direct_as(const CUtensorMap& tmU, DirectParams& q, void* ws, size_t ws_bytes, cudaStream_t st) {
+    const int sms = sm_count();
+    int* status = status_word_ptr();
+    if (sms <= 0 || !status) return err_cuda(__LINE__);
+    if (!ensure_dyn_smem(reinterpret_cast<const void*>(direct_conv_kernel<STRIDE>), MAX_DYN_SMEM)) return err_cuda(__LINE__);
+    const size_t smem = static_cast<size_t>(q.b_stages) * q.n_tile * 128 + q.a_stages * q.a_stage_bytes +
+                        DC_EPI_WARPS * DC_STG_BYTES + DC_BAR_BYTES + 1024;
+    const size_t packed_bytes = direct_packed_bytes(q);
+    q.packed = static_cast<const __half*>(ws);
+    q.part = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + packed_bytes);
+    CUtensorMap tmX = tmU;
+    if (!q.flat && !encode_map(&tmX, q.packed, static_cast<uint64_t>(q.pk_pitch) * 8, static_cast<uint64_t>(q.N) * q.rows_img,
+                               static_cast<uint64_t>(q.planes) * q.pk_pieces, static_cast<uint64_t>(q.pk_pitch) * 8,
+                               static_cast<uint64_t>(q.pk_positions) * 8, q.pitch * 8, 16 + (STRIDE == 1 ? 2 : 1), false,
+                               8))
+        return err_cuda(__LINE__);
+    {
+        ProfScope prof(KIND_INPUT, st);
+        const dim3 grid(static_cast<unsigned>((q.pk_positions + 255) / 256), q.pk_pieces, q.planes);
+        const cudaError_t e = launch_pdl(direct_pack_kernel, grid, dim3(256), 0, st, 0, q.x,
+                                         reinterpret_cast<uint4*>(const_cast<__half*>(q.packed)), q);
+        g_launches.fetch_add(1);
+        if (e != cudaSuccess) return err_cuda(__LINE__);
+    }
+    // the parts of as many (pixel tile, k tile) pairs as the workspace holds at a time
+    const int pairs = q.num_m * q.num_k_tiles;
+    const size_t per_pair = direct_part_bytes(q);
+    const int chunk = per_pair ? static_cast<int>(std::min<size_t>(pairs, (ws_bytes - packed_bytes) / per_pair)) : pairs;
+    for (int p0 = 0; p0 < pairs; p0 += chunk) {
+        q.pair_begin = p0;
+        q.pair_end = std::min(pairs, p0 + chunk);
+        const long long items = static_cast<long long>(q.pair_end - p0) * q.splits;
+        {
+            ProfScope prof(KIND_FUSED, st);
+            const cudaError_t e = launch_pdl(direct_conv_kernel<STRIDE>, dim3(static_cast<unsigned>(std::min<long long>(items, sms))),
+                                             dim3(DC_THREADS), smem, st, 0, tmU, tmX, q, status);
+            g_launches.fetch_add(1);
+            if (e != cudaSuccess) return err_cuda(__LINE__);
+        }
+        if (q.splits > 1) {
+            ProfScope prof(KIND_OUTPUT, st);
+            const dim3 grid(static_cast<unsigned>(q.pair_end - p0), static_cast<unsigned>(q.n_tile / 2));
+            const cudaError_t e = launch_pdl(direct_reduce_kernel, grid, dim3(128), 0, st, 0, q, status);
+            g_launches.fetch_add(1);
+            if (e != cudaSuccess) return err_cuda(__LINE__);
+        }
+    }
+    return SDWINO_OK;
+}
+
+// SDWINO_ERR_UNSUPPORTED: the workspace does not hold the packed copy of x (the caller then takes the three steps).
+int launch_direct(const __half* x, const void* wT, const __half* bias, __half* y, const Plan& pl, int N, int C, int H, int W,
+                  int K, int stride, void* ws, size_t ws_bytes, const Epilogue& ep, cudaStream_t st) {
+    const int sms = sm_count();
+    if (sms <= 0) return err_cuda(__LINE__);
+    DirectParams q;
+    const DirectShape best = choose_direct_shape(pl, N, C, H, W, K, stride, sms);
+    if (best.n_tile == 0 || !direct_geometry(pl, N, C, H, W, K, stride, best, &q)) return SDWINO_ERR_UNSUPPORTED;
+    if (direct_packed_bytes(q) + direct_part_bytes(q) > ws_bytes) return SDWINO_ERR_UNSUPPORTED;
+    direct_finish(&q);
+    q.wt_header = wt_header_of(wT);
+    q.x = x; q.bias = bias; q.y = y;
+    q.residual = static_cast<const __half*>(ep.residual);
+    q.act = ep.act;
+    q.vec_store = !q.flat && pl.Wo % 8 == 0 && aligned(y, 16) && aligned(ep.residual, 16);
+    CUtensorMap tmU;
+    if (!encode_filter_map(&tmU, wt_filters_of(wT), pl.Cb, pl.Kb, 9, best.n_tile / 16)) return err_cuda(__LINE__);
+    return stride == 1 ? launch_direct_as<1>(tmU, q, ws, ws_bytes, st) : launch_direct_as<2>(tmU, q, ws, ws_bytes, st);
+}
+
 
 int conv_impl(const void* x, const void* wT, const void* bias, void* y, int N, int C, int H, int W, int K, int tile,
               void* ws, size_t ws_bytes, cudaStream_t st, const Epilogue& ep_in = Epilogue{nullptr, 0, nullptr},
@@ -1057,6 +1265,11 @@ int conv_impl(const void* x, const void* wT, const void* bias, void* y, int N, i
     long long pc = tiles_per_pass(pl, ws_bytes);
     if (pc < GEMM_BLOCK_P) return SDWINO_ERR_WORKSPACE;
     ProfScope layer_prof(KIND_LAYER, st);   // profile mode 2: one record for the whole call
+    if (tile == 1 && !disable_fused && use_direct_conv(pl, N, C, stride)) {
+        const int rc = launch_direct(static_cast<const __half*>(x), wT, static_cast<const __half*>(bias), static_cast<__half*>(y), pl,
+                                     N, C, H, W, K, stride, ws, ws_bytes, ep_in, st);
+        if (rc != SDWINO_ERR_UNSUPPORTED) return rc;
+    }
     if (tile == 4 && pc < pl.P128) {
         // several passes: cut them at whole tile rows where that keeps the TMA-staged activation transform usable
         const TileGeom g0 = make_geom(H, W, pl.TH, pl.TW, pl.P);
