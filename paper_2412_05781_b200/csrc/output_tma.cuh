@@ -75,6 +75,18 @@ output_transform_f4_tma_kernel(const __grid_constant__ CUtensorMap tmM, const YT
     for (int it = 0; it < steps; ++it) {
         const int s = it % OUT_TMA_STAGES;
         const uint32_t parity = static_cast<uint32_t>(it / OUT_TMA_STAGES) & 1u;
+        // The residual rows are asked for before the wait for M: behind it, their latency stood between the two halves of
+        // the transform of every channel (512 -> 512 at 128x128 with residual: 12.3 -> 10.3 us, 8.5 without residual).
+        [[maybe_unused]] uint4 res[M];
+        if constexpr (EP && sizeof(YT) == 2) {
+            const __half* rp = static_cast<const __half*>(ep.residual) + (n * K + k_first + it) * hw + pix;
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                res[i] = make_uint4(0u, 0u, 0u, 0u);
+                if (ep.residual && tile_ok && i0 + i < geo.H)
+                    res[i] = __ldg(reinterpret_cast<const uint4*>(rp + static_cast<long long>(i) * geo.W));
+            }
+        }
         const bool ok = mbar_wait_bounded(&full_bar[s], parity, &abort_flag, OUT_TMA_WAIT_LIMIT_NS);
         float2 tt[M][A];   // A^T m, one column nu at a time; every float2 holds (tile 0, tile 1)
         if (ok) {
@@ -107,16 +119,6 @@ output_transform_f4_tma_kernel(const __grid_constant__ CUtensorMap tmM, const YT
         const int k = k_first + it;
         const float b = load_bias(bias, k);
         YT* img = y + (n * K + k) * hw + pix;
-        uint4 res[M];
-        if constexpr (EP && sizeof(YT) == 2) {
-#pragma unroll
-            for (int i = 0; i < M; ++i) {
-                res[i] = make_uint4(0u, 0u, 0u, 0u);
-                if (ep.residual && i0 + i < geo.H)
-                    res[i] = __ldg(reinterpret_cast<const uint4*>(static_cast<const __half*>(ep.residual) + (img - y) +
-                                                                   static_cast<long long>(i) * geo.W));
-            }
-        }
         [[maybe_unused]] float4 resf[M][2];   // fp32 residual rows, loaded ahead of the second half of the transform
         if constexpr (EP && sizeof(YT) == 4) {
 #pragma unroll
