@@ -480,12 +480,14 @@ bool use_input_tma(const TileGeom& geo, int N, int C, const void* x, long long p
     const bool possible = input_tma_possible(geo, N, C, x) && p_begin % geo.TW == 0 &&
                           (p_count % geo.TW == 0 || p_begin + p_count >= geo.P);
     if (!possible || g_input_staging == 0) return false;
-    // Faster where a block row is a whole number of 32-byte sectors of V (W % 64 == 0: 15.8 against 17.0 us on
-    // 960->320 at 64x64, 45.6 against 60.5 us on 512->512 at 256x256).  Image widths of 32 (8 tiles per row,
-    // four channel images per step) come out even, widths of 24, 48 and 96 up to 2x slower: their rows of 6, 12
-    // and 24 tiles leave runs of V that start and end inside sectors, where the register-only kernel, whose
-    // threads follow the tile index, always stores whole 128-byte lines.
-    return g_input_staging == 2 || geo.TW % 16 == 0;
+    // Faster where V is more than twice the L2 cache and a block row is a whole number of its 32-byte sectors (W % 64 == 0):
+    // 512 channels at 512x512 147 us against 176 with the register-only kernel, 256 channels at 1024x1024 293 / 316, at
+    // 768x768 177 / 187.  Below, the register-only kernel is, whose warps do not wait for one another: 320 channels at 64x64,
+    // batch 8, 15.7 / 12.1, 512 channels at 128x128 12.8 / 9.4, at 256x256 50 / 41 (V 151 MB), 256 channels at 512x512
+    // 82 / 80 (302 MB).  Other widths are up to 2x slower at any size: their rows leave runs of V that start and end inside
+    // sectors, where the register-only kernel, whose threads follow the tile index, always stores whole 128-byte lines.
+    const bool large = 72ll * C * p_count > (304ll << 20);
+    return g_input_staging == 2 || (geo.TW % 16 == 0 && large);
 }
 
 int launch_input_tma(const __half* x, __half* V, const TileGeom& geo, int N, int C, long long p_begin, long long p_count,
