@@ -603,7 +603,8 @@ input_transform_vec_kernel(const XT* __restrict__ x, __half* __restrict__ V, Til
 // EARLY (fp16 input): all six row segments of a channel are loaded before the first one is used, so that a thread
 // pays one memory latency per channel instead of several, also with 20 warps per SM: 320 channels at 96x96, batch 4,
 // 19.2 -> 13.9 us (77 MB: 4.0 -> 5.5 TB/s), 960 channels 64 -> 44, 1920 channels at 48x48 36 -> 25.6.  (With four CTAs per
-// SM instead of five 14.5, 47 and 28.7.)
+// SM instead of five 14.5, 47 and 28.7.)  fp32 input, three rows at a time: 640 channels at 64x64, batch 2, 9.4 -> 8.0 us,
+// 320 at 96x96, batch 4, 23.5 -> 18.6.
 template <int CH, typename XT = __half, bool PDL = true, bool EARLY = false>
 __device__ __forceinline__ void input_unit_f4(const XT* __restrict__ x, __half* __restrict__ V, const TileGeom& geo,
                                               int C, long long p_begin, const FastDiv& gdiv, long long Pstride,
@@ -645,6 +646,8 @@ __device__ __forceinline__ void input_unit_f4(const XT* __restrict__ x, __half* 
     if constexpr (sizeof(XT) == 4) xs = scalbnf(1.f, -range_exponent(amax));
     for (int cc = 0; cc < cend; ++cc) {
         float2 e2[A][A];   // e2[r][nu]: rows transformed along the columns, (tile 0, tile 1)
+        [[maybe_unused]] float4 fa[3], fb[3];   // fp32 input: three rows
+        [[maybe_unused]] float fl[3], fr[3];
         [[maybe_unused]] uint4 raw_v[A];
         [[maybe_unused]] uint32_t raw_l[A], raw_r[A];
         if constexpr (EARLY && sizeof(XT) == 2) {
@@ -665,15 +668,23 @@ __device__ __forceinline__ void input_unit_f4(const XT* __restrict__ x, __half* 
             float2 d[A];
             if constexpr (sizeof(XT) == 4) {
                 // fp32 input: pixels px0..px7 = a.x .. b.w, L and R the neighbours; pairs are (tile 0, tile 1)
-                float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-                float L = 0.f, R = 0.f;
-                if ((rowmask >> r) & 1) {
-                    const XT* rp = xp + r * geo.W;
-                    a = __ldg(reinterpret_cast<const float4*>(rp));
-                    b = __ldg(reinterpret_cast<const float4*>(rp) + 1);
-                    if (left_ok) L = to_f32(__ldg(rp - 1));
-                    if (right_ok) R = to_f32(__ldg(rp + 8));
+                // (three rows loaded at a time: all six leave too few registers for five CTAs)
+                if (r % 3 == 0) {
+#pragma unroll
+                    for (int g = 0; g < 3; ++g) {
+                        fa[g] = fb[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        fl[g] = fr[g] = 0.f;
+                        if ((rowmask >> (r + g)) & 1) {
+                            const XT* rp = xp + (r + g) * geo.W;
+                            fa[g] = __ldg(reinterpret_cast<const float4*>(rp));
+                            fb[g] = __ldg(reinterpret_cast<const float4*>(rp) + 1);
+                            if (left_ok) fl[g] = to_f32(__ldg(rp - 1));
+                            if (right_ok) fr[g] = to_f32(__ldg(rp + 8));
+                        }
+                    }
                 }
+                const float4 a = fa[r % 3], b = fb[r % 3];
+                const float L = fl[r % 3], R = fr[r % 3];
                 d[0] = make_float2(L * xs, a.w * xs);
                 d[1] = make_float2(a.x * xs, b.x * xs);
                 d[2] = make_float2(a.y * xs, b.y * xs);
