@@ -10,7 +10,7 @@
 //   output: a warp gathers its output rows in shared memory and writes them with neighbouring lanes on neighbouring pixels.
 // Against one tile per thread (B200, whole layers, F(4x4), batch 1 or 2): 640->640 at 50x37 37.2 -> 31.7 us, 320->320 at
 // 113x89 55.8 -> 42.1, 512->512 at 180x148 107.9 -> 86.0, 256->256 at 324x300 156.7 -> 121.4 (activation step 74 -> 45 us,
-// output step 47.5 -> 45 us: instruction issue at half of the slots, DRAM at a third of its bandwidth).
+// output step 47.5 -> 45 us; see there).
 // Measured slower for the output: rows gathered by the whole CTA and copied as 16-byte pieces (two barriers per channel),
 // with M loaded by TMA or from the registers: 50-66 us on the last of these layers.
 #pragma once
@@ -155,10 +155,13 @@ input_transform_any_kernel(const XT* __restrict__ x, __half* __restrict__ V, Til
 // registers, a warp's rows of eight pixels would leave as 4-byte or 2-byte pieces 16 bytes apart, each of them a partial
 // write of its sector; the output rows of the warp's tiles go through shared memory instead ([M][64 tiles][M pixels],
 // private to the warp) and leave with neighbouring lanes on neighbouring pixel pairs.
+// Five CTAs per SM: left to itself the compiler keeps to 80 registers (six CTAs) and so to a few loads of M at a time;
+// 256 channels at 324x300 40.5 -> 35.3 us, 640 at 50x37, batch 2, 9.2 -> 8.4.  (All 36 loads first: the same; the next
+// channel's loads ahead, four CTAs: 7.9 on the latter, 37.5 on the former, 20 % slower on 1280 channels at 25x19.)
 constexpr int OUT_ANY_THREADS = 128;
 
 template <int M, bool EP, typename YT = __half>
-__global__ void __launch_bounds__(OUT_ANY_THREADS)
+__global__ void __launch_bounds__(OUT_ANY_THREADS, 5)
 output_transform_any_kernel(const __half* __restrict__ Mws, const YT* __restrict__ bias, YT* __restrict__ y, TileGeom geo,
                             int K, long long p_begin, int p_count, long long Pstride, int steps, WtCheck chk, Epilogue ep) {
     constexpr int A = M + 2;
