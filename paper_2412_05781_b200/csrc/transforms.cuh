@@ -814,14 +814,21 @@ __device__ __forceinline__ void output_unit_vec(const __half* __restrict__ Mws, 
     const __half* src = Mws + static_cast<long long>(k) * Pstride + pl;
     if constexpr (M == 4) {
         // packed path: every float2 holds (tile 0, tile 1)
+        uint32_t raw[A][A];
+#pragma unroll
+        for (int s = 0; s < A; ++s)
+#pragma unroll
+            for (int r = 0; r < A; ++r) {
+                const uint32_t* wp = reinterpret_cast<const uint32_t*>(src + (r * A + s) * plane);
+                raw[r][s] = LIVE ? __ldcg(wp) : __ldg(wp);
+            }
         float2 tt[M][A];   // A^T m, one column nu at a time
 #pragma unroll
         for (int s = 0; s < A; ++s) {
             float2 col[A], o[M];
 #pragma unroll
             for (int r = 0; r < A; ++r) {
-                const uint32_t* wp = reinterpret_cast<const uint32_t*>(src + (r * A + s) * plane);
-                const uint32_t w = LIVE ? __ldcg(wp) : __ldg(wp);
+                const uint32_t w = raw[r][s];
                 col[r] = __half22float2(*reinterpret_cast<const __half2*>(&w));
             }
             at4_packed(col, o);
@@ -922,9 +929,12 @@ __device__ __forceinline__ void output_unit_vec(const __half* __restrict__ Mws, 
     }   // M != 4
 }
 
-// EP = false: the plain convolution (the epilogue argument is ignored and costs no register)
+// EP = false: the plain convolution (the epilogue argument is ignored and costs no register).
+// Bound by the latency of its loads where a layer has few tiles, so all of M is asked for before any of it is used (six
+// CTAs per SM, with five or four the same): F(2x2) 1280 channels at 16x16, batch 2, 2.56 -> 2.22 us (the layer 17.75 ->
+// 17.14), 640 at 32x32, batch 1, layer 13.46 -> 12.64; F(4x4) 1280 at 32x32, batch 2, 5.4 -> 5.1.
 template <int M, int TPT, bool EP, typename YT = __half>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, 6)
 output_transform_vec_kernel(const __half* __restrict__ Mws, const YT* __restrict__ bias, YT* __restrict__ y,
                             TileGeom geo, int K, long long p_begin, FastDiv gdiv, long long Pstride, WtCheck chk,
                             Epilogue ep) {
