@@ -319,6 +319,13 @@ int sdwino_last_device_status(void *stream);
  */
 int sdwino_selftest_wait_timeout(unsigned long long limit_ns, void *stream);
 
+/*
+ * Host-only self test of the addresses that the activation transforms of any width (W % 8 != 0, or x not 16-byte
+ * aligned) load from a fp16 x [N][C][H][W], two pixels at a time: the bytes before the first and after the last element of
+ * x that any of them touches (0 and 0), for an x that starts at an even or (odd_start != 0) an odd 2-byte element.
+ */
+int sdwino_selftest_window_reads(int N, int C, int H, int W, int tile, int odd_start, long long *before, long long *after);
+
 /* Kernel launches made by this library in the calling process so far (all entry points). */
 unsigned long long sdwino_launch_count(void);
 

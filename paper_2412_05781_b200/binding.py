@@ -27,7 +27,7 @@ EXPORTS = [
     "sdwino_host_staging_bytes_f32", "sdwino_conv3x3_host_f32", "sdwino_conv3x3_host_f32_async", "sdwino_set_pipeline",
     "sdwino_conv3x3_f32_scaled", "sdwino_filter_q8_bytes", "sdwino_filter_quantize", "sdwino_conv3x3_q8",
     "sdwino_workspace_bytes_direct", "sdwino_conv3x3_direct", "sdwino_choose_algorithm",
-    "sdwino_workspace_bytes_sequence", "sdwino_conv3x3_sequence",
+    "sdwino_workspace_bytes_sequence", "sdwino_conv3x3_sequence", "sdwino_selftest_window_reads",
 ]
 
 class SdwinoLayer(ctypes.Structure):
@@ -101,6 +101,8 @@ def _load() -> ctypes.CDLL:
     lib.sdwino_set_input_staging.argtypes = [i]
     lib.sdwino_selftest_wait_timeout.restype = i
     lib.sdwino_selftest_wait_timeout.argtypes = [ctypes.c_ulonglong, vp]
+    lib.sdwino_selftest_window_reads.restype = i
+    lib.sdwino_selftest_window_reads.argtypes = [i, i, i, i, i, i, ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(ctypes.c_longlong)]
     lib.sdwino_choose_tile.restype = i
     lib.sdwino_choose_tile.argtypes = [i, i, i, i, i]
     lib.sdwino_choose_algorithm.restype = i
@@ -190,6 +192,13 @@ def sdwino_last_device_status(stream: Optional[torch.cuda.Stream] = None) -> int
 def sdwino_selftest_wait_timeout(limit_ns: int, stream: Optional[torch.cuda.Stream] = None) -> None:
     """Launch the bounded-wait self-test; sdwino_last_device_status() reports ERR_TIMEOUT afterwards."""
     _check(lib.sdwino_selftest_wait_timeout(limit_ns, _stream_ptr(stream)), "sdwino_selftest_wait_timeout")
+
+
+def sdwino_selftest_window_reads(N: int, C: int, H: int, W: int, tile: int, odd_start: bool):
+    """-> (bytes before, bytes after) x that the any-width activation transforms touch; see include/sdwino.h."""
+    before, after = ctypes.c_longlong(-1), ctypes.c_longlong(-1)
+    _check(lib.sdwino_selftest_window_reads(N, C, H, W, tile, int(odd_start), before, after), "sdwino_selftest_window_reads")
+    return before.value, after.value
 
 
 def sdwino_set_gemm_shape(ctas: int = 0, n_tile: int = 0) -> None:

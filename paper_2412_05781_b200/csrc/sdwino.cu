@@ -462,7 +462,13 @@ int launch_input(const XT* x, __half* V, const TileGeom& geo, int C, long long p
         }
     } else {
         const dim3 grid = grid_rows((p_count / 2 + 127) / 128, C);
-        e = launch_pdl(input_transform_any_kernel<M, XT>, grid, dim3(128), 0, st, 0, x, V, geo, C, p_begin, p_count, Pstride, amax);
+        const long long elems = geo.P / geo.TH / geo.TW * C * geo.H * geo.W;
+        bool edge = false;
+        if constexpr (sizeof(XT) == 2) edge = x_cuts_words(reinterpret_cast<uintptr_t>(x), elems);
+        e = edge ? launch_pdl(input_transform_any_kernel<M, XT, sizeof(XT) == 2>, grid, dim3(128), 0, st, 0, x, V, geo, C, p_begin,
+                              p_count, Pstride, amax, elems)
+                 : launch_pdl(input_transform_any_kernel<M, XT>, grid, dim3(128), 0, st, 0, x, V, geo, C, p_begin, p_count, Pstride,
+                              amax, elems);
     }
     g_launches.fetch_add(1);
     return e == cudaSuccess ? SDWINO_OK : err_cuda(__LINE__);
@@ -1966,6 +1972,47 @@ int sdwino_selftest_wait_timeout(unsigned long long limit_ns, void* stream) {
     return cudaGetLastError() == cudaSuccess ? SDWINO_OK : err_cuda(__LINE__);
 }
 
+}  // extern "C"
+
+namespace {
+template <int M>
+void window_reads(int N, int C, int H, int W, uintptr_t x, long long* before, long long* after) {
+    constexpr int A = M + 2;
+    const long long elems = static_cast<long long>(N) * C * H * W;
+    const uintptr_t x_hi = x + 2 * static_cast<uintptr_t>(elems);
+    const bool edge = x_cuts_words(x, elems);
+    uintptr_t first = x_hi, last = x;
+    for (long long img = 0; img < static_cast<long long>(N) * C; ++img)
+        for (int i0 = -1; i0 < H; i0 += M)
+            for (int j0 = -1; j0 < W; j0 += M) {
+                int lo, hi;
+                window_columns<A>(j0, W, lo, hi);
+                for (int r = 0; r < A; ++r) {
+                    if (i0 + r < 0 || i0 + r >= H) continue;
+                    const uintptr_t a = x + static_cast<uintptr_t>((img * H + i0 + r) * W + j0) * 2;
+                    for (int i = 0; i <= A / 2; ++i) {
+                        uintptr_t word;
+                        if (!window_word(a, i, lo, hi, &word)) continue;
+                        const int in = edge && (img % C == 0 || img % C == C - 1) ? word_pixels_in_x(word, x, x_hi) : 3;
+                        first = std::min(first, in & 1 ? word : word + 2);
+                        last = std::max(last, in & 2 ? word + 4 : word + 2);
+                    }
+                }
+            }
+    *before = first < x ? static_cast<long long>(x - first) : 0;
+    *after = last > x_hi ? static_cast<long long>(last - x_hi) : 0;
+}
+}  // namespace
+
+extern "C" {
+int sdwino_selftest_window_reads(int N, int C, int H, int W, int tile, int odd_start, long long* before, long long* after) {
+    if (N <= 0 || C <= 0 || H <= 0 || W <= 0 || !before || !after) return SDWINO_ERR_INVALID_ARG;
+    if (tile != 2 && tile != 4) return SDWINO_ERR_UNSUPPORTED;
+    const uintptr_t x = (uintptr_t(1) << 20) + (odd_start ? 2 : 0);     // an address to compute with
+    if (tile == 2) window_reads<2>(N, C, H, W, x, before, after);
+    else window_reads<4>(N, C, H, W, x, before, after);
+    return SDWINO_OK;
+}
 }  // extern "C"
 
 namespace {

@@ -43,15 +43,51 @@ __device__ __forceinline__ void at_packed(const float2 (&m)[M + 2], float2 (&o)[
     }
 }
 
+// Which bytes of the aligned 4-byte word at `word` lie in x, the bytes [x_lo, x_hi): bit 0 the lower pixel, bit 1 the upper
+// one.  Only the word of the first pixel of x (x at an odd pixel) or of its last one can have a pixel outside.
+__host__ __device__ __forceinline__ int word_pixels_in_x(uintptr_t word, uintptr_t x_lo, uintptr_t x_hi) {
+    return (word >= x_lo ? 1 : 0) | (word + 4 <= x_hi ? 2 : 0);
+}
+// Whether x begins or ends inside a word.
+inline bool x_cuts_words(uintptr_t x, long long elems) {
+    return (x & 3) != 0 || ((x + 2 * static_cast<uintptr_t>(elems)) & 3) != 0;
+}
+// The columns [lo, hi) of a window that lie inside the image; j0 is the image column of its column 0.
+template <int A>
+__host__ __device__ __forceinline__ void window_columns(int j0, int W, int& lo, int& hi) {
+    lo = j0 < 0 ? -j0 : 0;
+    hi = W - j0 < A ? W - j0 : A;
+}
+// Word i of a window row that begins at address `a` (its pixel 0) and has the pixels [lo, hi) inside the image: it holds the
+// pixels 2 i - par and 2 i - par + 1 and is loaded if one of them is inside.
+__host__ __device__ __forceinline__ bool window_word(uintptr_t a, int i, int lo, int hi, uintptr_t* word) {
+    const int par = static_cast<int>((a >> 1) & 1);
+    *word = (a & ~uintptr_t(3)) + 4 * static_cast<uintptr_t>(i);
+    return 2 * i - par + 1 >= lo && 2 * i - par < hi;
+}
+
+// Predicated, so that the loads of a window stay together (as branches they wait for one another).
+__device__ __forceinline__ void ld_nc_u32_if(uint32_t& v, const void* p, bool pred) {
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q ld.global.nc.b32 %0, [%1];\n\t}"
+        : "+r"(v) : "l"(p), "r"(static_cast<int>(pred)));
+}
+
 // Window rows of one tile, all A of them: row r in h[r] as A / 2 words of two pixels, zeros outside the image.  Every
 // word that is loaded holds at least one pixel of the row (the other one may lie outside: it shares the aligned word).
-// (Reading whole rows without these tests, masked afterwards, measured 5-8 % slower.)
-template <int M>
+// EDGE: x begins or ends in the middle of a word, whose other half is not x's to read: that pixel is loaded alone.
+// (Tested on every word of the layer, 256 channels at 324x300, x odd, took 70 us instead of 46; only the first and last channel do, and go first.)
+// (Reading whole rows without the tests of window_word, masked afterwards, measured 5-8 % slower.)
+template <int M, bool EDGE>
 __device__ __forceinline__ void load_window(const __half* __restrict__ img, const TileGeom& geo, int i0, int j0, bool valid,
-                                            uint32_t (&h)[M + 2][(M + 2) / 2]) {
+                                            uintptr_t x_lo, uintptr_t x_hi, uint32_t (&h)[M + 2][(M + 2) / 2]) {
     constexpr int A = M + 2;
-    const int lo = j0 < 0 ? -j0 : 0;
-    const int hi = geo.W - j0 < A ? geo.W - j0 : A;
+    int lo, hi;
+    window_columns<A>(j0, geo.W, lo, hi);
+    [[maybe_unused]] uint32_t first = 0u, last = 0u;      // the pixels that share a word with something else, in their places
+    if constexpr (EDGE) {
+        first = static_cast<uint32_t>(__ldg(reinterpret_cast<const unsigned short*>(x_lo))) << 16;
+        last = __ldg(reinterpret_cast<const unsigned short*>(x_hi) - 1);
+    }
     uint32_t mask[A / 2];
 #pragma unroll
     for (int i = 0; i < A / 2; ++i)
@@ -60,29 +96,36 @@ __device__ __forceinline__ void load_window(const __half* __restrict__ img, cons
     for (int r = 0; r < A; ++r) {
         const bool row_ok = valid && static_cast<unsigned>(i0 + r) < static_cast<unsigned>(geo.H);
         const uintptr_t a = reinterpret_cast<uintptr_t>(img) + (static_cast<long long>(i0 + r) * geo.W + j0) * 2;
-        const int par = static_cast<int>((a >> 1) & 1);
-        const uint32_t* wp = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
         uint32_t w[A / 2 + 1];
 #pragma unroll
         for (int i = 0; i <= A / 2; ++i) {
-            // word i holds the pixels 2 i - par and 2 i - par + 1 of the row
             w[i] = 0u;
-            if (row_ok && 2 * i - par + 1 >= lo && 2 * i - par < hi) w[i] = __ldg(wp + i);
+            uintptr_t word;
+            const bool want = window_word(a, i, lo, hi, &word) && row_ok;
+            if constexpr (EDGE) {
+                const int in = word_pixels_in_x(word, x_lo, x_hi);
+                if (want && in != 3) w[i] = in == 2 ? first : last;
+                ld_nc_u32_if(w[i], reinterpret_cast<const void*>(word), want && in == 3);
+            } else if (want) {
+                w[i] = __ldg(reinterpret_cast<const uint32_t*>(word));
+            }
         }
-        const uint32_t sel = par ? 0x5432u : 0x3210u;
+        const uint32_t sel = (a >> 1) & 1 ? 0x5432u : 0x3210u;
 #pragma unroll
         for (int i = 0; i < A / 2; ++i) h[r][i] = __byte_perm(w[i], w[i + 1], sel) & mask[i];
     }
 }
 
 // Activation preprocess of the pair (p, p + 1) for one channel; p - p_begin even.  Tiles past the last one are zeros.
-template <int M, typename XT = __half>
+// x_elems: the elements of x (only used with EDGE, see load_window).
+template <int M, typename XT = __half, bool EDGE = false>
 __global__ void __launch_bounds__(128)
 input_transform_any_kernel(const XT* __restrict__ x, __half* __restrict__ V, TileGeom geo, int C, long long p_begin,
-                           int p_count, long long Pstride, const float* __restrict__ amax) {
+                           int p_count, long long Pstride, const float* __restrict__ amax, long long x_elems) {
     constexpr int A = M + 2;
     const int pl = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x) * 2;
-    const int c = static_cast<int>(blockIdx.z * gridDim.y + blockIdx.y);   // grid.z continues grid.y past 65535
+    int c = static_cast<int>(blockIdx.z * gridDim.y + blockIdx.y);   // grid.z continues grid.y past 65535
+    if (EDGE && c < C) c = c == 0 ? C - 1 : c - 1;     // the two channels that take longer go first (1-2 us less)
     const long long hw = static_cast<long long>(geo.H) * geo.W;
     int i0[2] = {0, 0}, j0[2] = {0, 0};
     bool valid[2];
@@ -107,8 +150,14 @@ input_transform_any_kernel(const XT* __restrict__ x, __half* __restrict__ V, Til
     float2 e2[A][A];   // rows transformed along the columns, (tile 0, tile 1)
     if constexpr (sizeof(XT) == 2) {
         uint32_t h0[A][A / 2], h1[A][A / 2];
-        load_window<M>(img[0], geo, i0[0], j0[0], valid[0], h0);
-        load_window<M>(img[1], geo, i0[1], j0[1], valid[1], h1);
+        const uintptr_t x_lo = reinterpret_cast<uintptr_t>(x), x_hi = x_lo + 2 * static_cast<uintptr_t>(x_elems);
+        if (EDGE && (c == 0 || c == C - 1)) {    // the first and the last pixel of x are in these channels
+            load_window<M, EDGE>(img[0], geo, i0[0], j0[0], valid[0], x_lo, x_hi, h0);
+            load_window<M, EDGE>(img[1], geo, i0[1], j0[1], valid[1], x_lo, x_hi, h1);
+        } else {
+            load_window<M, false>(img[0], geo, i0[0], j0[0], valid[0], x_lo, x_hi, h0);
+            load_window<M, false>(img[1], geo, i0[1], j0[1], valid[1], x_lo, x_hi, h1);
+        }
 #pragma unroll
         for (int r = 0; r < A; ++r) {
             float2 d[A];
