@@ -187,12 +187,13 @@ int sdwino_conv3x3_q8(const void *x, const void *wTq, const void *bias, void *y,
  * gathers the nine shifted copies of x (V[tap][c][pixel]), the tcgen05 GEMM contracts the channels per tap, the output
  * step adds the nine partial sums and the bias.  It streams 9 instead of 16 (tile 2) filter values per weight, at
  * 2.25 times the tensor work per output pixel.
- * From 512 output pixels (stride 2: 640) and 32 channels on, where the workspace has room for one rearranged copy of x,
- * a single GEMM kernel forms the nine taps out of that copy instead and keeps their sum in fp32.
+ * From 512 output pixels (stride 2: 640) and 32 channels on, a single GEMM kernel forms the nine taps out of one
+ * rearranged copy of x instead and keeps their sum in fp32.  Which of the two a layer takes depends on its sizes alone; where
+ * the workspace does not hold the copy, it is made and used window by window (some images, rows or columns at a time).
  *   filters: sdwino_filter_bytes / sdwino_filter_transform with tile = 1 (the weights reordered tap by tap).
  *   y: fp16 [N][K][Ho][Wo] with Ho = (H - 1) / stride + 1, Wo = (W - 1) / stride + 1; stride 1 or 2
  *   (SDWINO_ERR_UNSUPPORTED above 2, SDWINO_ERR_INVALID_ARG below 1).  Workspace: sdwino_workspace_bytes_direct for
- *   one pass; smaller workspaces take several passes as in sdwino_conv3x3_ws.  Other arguments and errors as
+ *   one pass; smaller workspaces take several passes, with the same bits, as in sdwino_conv3x3_ws.  Other arguments and errors as
  *   sdwino_conv3x3_ws.
  */
 size_t sdwino_workspace_bytes_direct(int N, int C, int H, int W, int K, int stride);

@@ -57,10 +57,13 @@ struct DirectParams {
     const __half* packed;     // see direct_pack_kernel
     float* part;              // splits > 1: fp32 parts [(pixel tile, k tile)][split][n_tile][128]
     int act;
-    int N, C, H, W, K, Ho, Wo, stride;
+    int N, C, H, W, K, Ho, Wo, stride; // N: images of this launch; x, y and residual point at its first output
     int n_tile, num_k_tiles, num_m;    // output channels per CTA tile, tiles along k and along the pixels
     int pair_begin, pair_end;          // (pixel tile, k tile) pairs of this launch
     int splits, cb_per_split, num_cb;  // parts of the channel blocks
+    int win_h, win_w;                  // output rows and columns of this launch (all, unless the workspace is small)
+    int row0, col0;                    // row and column of x at position (0, 0) of the packed copy
+    int org;                           // grid: position of a patch's first row and column for output row and column 0
     int flat, pitch, rows_img;         // layout of the pixels; rows_img: rows per image, padding included
     int lead;                          // flat, stride 1: positions of zeros before the first pixel
     int tiles_c, tiles_r;              // grid: tiles per image
@@ -99,7 +102,7 @@ __device__ __forceinline__ bool direct_out_pixel(const DirectParams& q, int m, i
         const uint32_t img = fast_div(v, q.fd_rows);
         r = static_cast<int>(v - img * static_cast<uint32_t>(q.rows_img));
         n = static_cast<int>(img);
-        return n < q.N && r < q.Ho && c < q.Wo;
+        return n < q.N && r < q.win_h && c < q.win_w;
     }
     const uint32_t row_blk = fast_div(static_cast<uint32_t>(m), q.fd_tc);
     const uint32_t img = fast_div(row_blk, q.fd_tr);
@@ -108,7 +111,7 @@ __device__ __forceinline__ bool direct_out_pixel(const DirectParams& q, int m, i
     n = static_cast<int>(img);
     r = rb * 16 + (l >> 3);
     c = cb * 8 + (l & 7);
-    return r < q.Ho && c < q.Wo;
+    return r < q.win_h && c < q.win_w;
 }
 
 template <int STRIDE>
@@ -295,7 +298,7 @@ direct_conv_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constan
                         const int k = k0 + col + ch;
                         const float4 a = *reinterpret_cast<const float4*>(stg + ch * 32 + row * 8);
                         const float4 b = *reinterpret_cast<const float4*>(stg + ch * 32 + row * 8 + 4);
-                        if (oy + row < q.Ho && ox < q.Wo && k < q.K) {
+                        if (oy + row < q.win_h && ox < q.win_w && k < q.K) {
                             const float bk = load_bias(q.bias, k);
                             float v[8] = {a.x + bk, a.y + bk, a.z + bk, a.w + bk, b.x + bk, b.y + bk, b.z + bk, b.w + bk};
                             const long long o = (static_cast<long long>(n) * q.K + k) * hw_o + static_cast<long long>(oy + row) * q.Wo + ox;
@@ -364,11 +367,10 @@ direct_conv_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constan
             decode(wi, m, kt, cb0, cb1);
             int row0 = 0, col0 = 0;
             if (!q.flat) {
-                const int org = q.stride == 1 ? -1 : 0;     // the packed planes of stride 2 start at row and column -1
                 const uint32_t row_blk = fast_div(static_cast<uint32_t>(m), q.fd_tc);
                 const uint32_t img = fast_div(row_blk, q.fd_tr);
-                col0 = ((m - static_cast<int>(row_blk) * q.tiles_c) * 8 + org) * 8;
-                row0 = static_cast<int>(img) * q.rows_img + (static_cast<int>(row_blk) - static_cast<int>(img) * q.tiles_r) * 16 + org;
+                col0 = ((m - static_cast<int>(row_blk) * q.tiles_c) * 8 + q.org) * 8;
+                row0 = static_cast<int>(img) * q.rows_img + (static_cast<int>(row_blk) - static_cast<int>(img) * q.tiles_r) * 16 + q.org;
             }
             for (int cb = cb0; cb < cb1 && ok; ++cb) {
                 for (int pl = 0; pl < q.planes; ++pl) {
@@ -444,7 +446,8 @@ direct_reduce_kernel(const __grid_constant__ DirectParams q, int* __restrict__ s
 // x [N][C][H][W] -> [plane][ceil(C / 64) * 8 pieces][positions][8 channels]: the pixels in the order of the flat layout
 // (one column and one row of zeros between neighbours, `lead` positions of zeros in front), so that a patch of either
 // layout is a few contiguous runs of 16-byte pieces.  Stride 2: plane (a, b) holds pixel (2 r + a - 1, 2 c + b - 1) at
-// row r, column c.  One thread per piece: eight 2-byte loads, coalesced over the pixels, one 16-byte store.
+// row r, column c.  A copy of part of the image (see DirectWindow) begins with its halo at row and column -1 of the part, stride
+// 1 as well.  One thread per piece: eight 2-byte loads, coalesced over the pixels, one 16-byte store.
 __global__ void __launch_bounds__(256)
 direct_pack_kernel(const __half* __restrict__ x, uint4* __restrict__ packed, const __grid_constant__ DirectParams q) {
     const long long idx = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;
@@ -453,9 +456,8 @@ direct_pack_kernel(const __half* __restrict__ x, uint4* __restrict__ packed, con
     const uint32_t Qu = static_cast<uint32_t>(Q < 0 ? 0 : Q);
     const uint32_t v = fast_div(Qu, q.fd_pkp);
     const uint32_t img = fast_div(v, q.fd_rows);
-    const int org = q.stride == 1 ? 0 : -1;
-    const int i = static_cast<int>(v - img * static_cast<uint32_t>(q.rows_img)) * q.stride + (pl >> 1) + org;
-    const int j = static_cast<int>(Qu - v * static_cast<uint32_t>(q.pk_pitch)) * q.stride + (pl & 1) + org;
+    const int i = static_cast<int>(v - img * static_cast<uint32_t>(q.rows_img)) * q.stride + (pl >> 1) + q.row0;
+    const int j = static_cast<int>(Qu - v * static_cast<uint32_t>(q.pk_pitch)) * q.stride + (pl & 1) + q.col0;
     const bool live = Q >= 0 && static_cast<int>(img) < q.N && static_cast<unsigned>(i) < static_cast<unsigned>(q.H) &&
                       static_cast<unsigned>(j) < static_cast<unsigned>(q.W);
     const long long hw = static_cast<long long>(q.H) * q.W;

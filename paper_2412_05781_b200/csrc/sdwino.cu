@@ -1048,17 +1048,30 @@ int launch_pipeline(const __half* x, const void* wT, const __half* bias, __half*
 // 640 -> 640 512 pixels 14.1 / 14.4, 64 -> 96 625 pixels 7.6 / 7.5, 320 -> 320 1024 pixels 12.9 / 12.0, 1280 -> 1280 1024
 // pixels 48.9 / 40; stride 1, 128 pixels 13.7 / 17, 512 pixels 9.9 / 9.3 (320) and 14.1 / 12.3 (640).
 // Channels come in blocks of 64, padded with zeros, so it also wants half a block.
+// With less workspace than the copy takes (window by window) it is faster than the three steps in several passes as well:
+// 320 -> 320 at 64x64, stride 2, batch 2, in an eighth of the one-pass workspace 77 / 26 us, in the smallest 114 / 50;
+// 128 -> 128 at 512x512, stride 2, an eighth 222 / 64.
 constexpr int DIRECT_MIN_CHANNELS = 32;
 bool use_direct_conv(const Plan& pl, int N, int C, int stride) {
     return C >= DIRECT_MIN_CHANNELS && static_cast<long long>(N) * pl.Ho * pl.Wo >= (stride == 1 ? 512 : 640);
 }
 
 struct DirectShape { int flat, n_tile, splits; };   // n_tile 0: none
+// The outputs of a launch: images n0 .. n0 + n - 1, rows r0 .. r0 + h - 1, columns c0 .. c0 + w - 1 of y.  All of them where the
+// workspace holds the packed copy of x; otherwise the layer runs window by window, each with a packed copy of its own.
+// The sum of an output takes the same channels in the same order in every window, so its bits do not depend on them.
+struct DirectWindow { int n0, n, r0, h, c0, w; };
 
 // Fills the geometry of a candidate; false where its patch does not fit in shared memory or an index in 32 bits.
-bool direct_geometry(const Plan& pl, int N, int C, int H, int W, int K, int stride, const DirectShape& sh, DirectParams* q) {
-    q->N = N; q->C = C; q->H = H; q->W = W; q->K = K;
+bool direct_geometry(const Plan& pl, const DirectWindow& win, int C, int H, int W, int K, int stride, const DirectShape& sh,
+                     DirectParams* q) {
+    const bool part = win.h != pl.Ho || win.w != pl.Wo;   // a copy of part of an image has its halo on all sides
+    q->N = win.n; q->C = C; q->H = H; q->W = W; q->K = K;
     q->Ho = pl.Ho; q->Wo = pl.Wo; q->stride = stride;
+    q->win_h = win.h; q->win_w = win.w;
+    q->org = stride == 1 && !part ? -1 : 0;               // the planes of stride 2 begin at row and column -1 anyway
+    q->row0 = win.r0 * stride - (stride == 1 && !part ? 0 : 1);
+    q->col0 = win.c0 * stride - (stride == 1 && !part ? 0 : 1);
     q->n_tile = sh.n_tile;
     q->num_k_tiles = (K + sh.n_tile - 1) / sh.n_tile;
     q->num_cb = (C + 63) / 64;
@@ -1067,12 +1080,12 @@ bool direct_geometry(const Plan& pl, int N, int C, int H, int W, int K, int stri
     q->flat = sh.flat;
     const int halo = stride == 1 ? 2 : 1;
     long long pp, num_m;
-    q->rows_img = pl.Ho + 1;
-    q->pk_pitch = pl.Wo + 1;
+    q->rows_img = win.h + (stride == 1 && part ? 2 : 1);
+    q->pk_pitch = win.w + (stride == 1 && part ? 2 : 1);
     q->pk_pieces = q->num_cb * 8;
     q->lead = 0;
     q->tiles_c = q->tiles_r = 1;
-    const long long positions = static_cast<long long>(N) * q->rows_img * q->pk_pitch;
+    const long long positions = static_cast<long long>(win.n) * q->rows_img * q->pk_pitch;
     if (positions + 4096 >= (1ll << 31)) return false;
     if (sh.flat) {
         q->pitch = q->pk_pitch;
@@ -1084,9 +1097,9 @@ bool direct_geometry(const Plan& pl, int N, int C, int H, int W, int K, int stri
     } else {
         q->pitch = 8 + halo;
         pp = (16 + halo) * static_cast<long long>(q->pitch);
-        q->tiles_c = (pl.Wo + 7) / 8;
-        q->tiles_r = (pl.Ho + 15) / 16;
-        num_m = static_cast<long long>(N) * q->tiles_c * q->tiles_r;
+        q->tiles_c = (win.w + 7) / 8;
+        q->tiles_r = (win.h + 15) / 16;
+        num_m = static_cast<long long>(win.n) * q->tiles_c * q->tiles_r;
         q->sbo = q->pitch;
         q->pk_positions = positions;
     }
@@ -1135,9 +1148,10 @@ double direct_cost(const DirectParams& q, bool vec, int sms) {
     return q.splits == 1 ? cost : cost + 2300.0 + static_cast<double>(items) * q.n_tile * 512.0 / 2000.0;
 }
 
-// The cheapest modelled shape; n_tile == 0 where none fits.  It depends on the layer alone and not on the workspace that was
-// passed (the order of the sums, and with it the bits, follow from it): parts may take what a one-pass workspace has
-// beside the packed copy.  Some hundred candidates are looked at, so the last choices are kept (by the layer's sizes).
+// The cheapest modelled shape; n_tile == 0 where none fits a one-pass workspace, packed copy and the parts of one pair.
+// It depends on the layer alone and not on the workspace that was passed: whether the layer takes this form and the order of
+// its sums, and with them the bits, follow from it.  Some hundred candidates are looked at, so the last choices are kept (by
+// the layer's sizes).
 DirectShape choose_direct_shape(const Plan& pl, int N, int C, int H, int W, int K, int stride, int sms) {
     struct Slot { int key[7]; DirectShape shape; bool used; };
     static Slot slots[64];
@@ -1163,7 +1177,8 @@ DirectShape choose_direct_shape(const Plan& pl, int N, int C, int H, int W, int 
                 const int per = (num_cb + s - 1) / s;
                 if ((num_cb + per - 1) / per != s) continue;             // a smaller s has parts as long
                 const DirectShape sh{flat, n, s};
-                if (!direct_geometry(pl, N, C, H, W, K, stride, sh, &q)) break;
+                if (!direct_geometry(pl, DirectWindow{0, N, 0, pl.Ho, 0, pl.Wo}, C, H, W, K, stride, sh, &q)) break;
+                if (direct_packed_bytes(q) > full) break;
                 const long long pairs = static_cast<long long>(q.num_m) * ktiles;
                 if (s > 1 && (pairs * (s - 1) >= 2ll * sms || direct_packed_bytes(q) + pairs * direct_part_bytes(q) > full))
                     break;
@@ -1229,26 +1244,81 @@ int launch_direct_as(const CUtensorMap& tmU, DirectParams& q, void* ws, size_t w
     return SDWINO_OK;
 }
 
-// SDWINO_ERR_UNSUPPORTED: the workspace does not hold the packed copy of x (the caller then takes the three steps).
+// The window sizes for a workspace that does not hold the packed copy of x: whole images, then whole rows, then pieces of
+// rows, as many as fit (next to parts: in half of the workspace).  The smallest, 4 rows of 8 outputs, takes 360 bytes per
+// channel (of up to twice as many channels as there are) and its parts 8 KB per split of at least 64 channels; the smallest
+// workspace has 2304 bytes per channel.
+bool direct_window(const Plan& pl, int N, int C, int H, int W, int K, int stride, int splits, size_t ws_bytes, DirectWindow* win) {
+    const size_t budget = splits > 1 ? ws_bytes / 2 : ws_bytes;
+    auto fits = [&](int n, int h, int w) {
+        DirectParams q;
+        *win = DirectWindow{0, n, 0, h, 0, w};
+        return direct_geometry(pl, *win, C, H, W, K, stride, DirectShape{0, 16, splits}, &q) && direct_packed_bytes(q) <= budget;
+    };
+    // the largest v in [lo, hi] (hi - lo a multiple of step or not) with fits(v); fits is monotone
+    auto largest = [&](int lo, int hi, int step, auto&& ok) {
+        int best = 0;
+        for (int a = 0, b = (hi - lo + step - 1) / step; a <= b;) {
+            const int mid = (a + b) / 2, v = std::min(hi, lo + mid * step);
+            if (ok(v)) { best = v; a = mid + 1; } else { b = mid - 1; }
+        }
+        return best;
+    };
+    if (const int n = largest(1, N, 1, [&](int v) { return fits(v, pl.Ho, pl.Wo); })) return fits(n, pl.Ho, pl.Wo);
+    if (const int h = largest(std::min(16, pl.Ho), pl.Ho, 16, [&](int v) { return fits(1, v, pl.Wo); })) return fits(1, h, pl.Wo);
+    for (int h = 16; h >= 4; h /= 2)
+        if (const int w = largest(std::min(8, pl.Wo), pl.Wo, 8, [&](int v) { return fits(1, std::min(h, pl.Ho), v); }))
+            return fits(1, std::min(h, pl.Ho), w);
+    return false;
+}
+
+// SDWINO_ERR_UNSUPPORTED: the layer has no shape of this form (the caller then takes the three steps).
 int launch_direct(const __half* x, const void* wT, const __half* bias, __half* y, const Plan& pl, int N, int C, int H, int W,
                   int K, int stride, void* ws, size_t ws_bytes, const Epilogue& ep, cudaStream_t st) {
     const int sms = sm_count();
     if (sms <= 0) return err_cuda(__LINE__);
+    DirectShape best = choose_direct_shape(pl, N, C, H, W, K, stride, sms);
+    if (best.n_tile == 0) return SDWINO_ERR_UNSUPPORTED;
     DirectParams q;
-    const DirectShape best = choose_direct_shape(pl, N, C, H, W, K, stride, sms);
-    if (best.n_tile == 0 || !direct_geometry(pl, N, C, H, W, K, stride, best, &q)) return SDWINO_ERR_UNSUPPORTED;
-    if (direct_packed_bytes(q) + direct_part_bytes(q) > ws_bytes) return SDWINO_ERR_UNSUPPORTED;
-    direct_finish(&q);
-    q.wt_header = wt_header_of(wT);
-    q.x = x; q.bias = bias; q.y = y;
-    q.residual = static_cast<const __half*>(ep.residual);
-    q.act = ep.act;
-    q.vec_store = !q.flat && pl.Wo % 8 == 0 && aligned(y, 16) && aligned(ep.residual, 16);
+    DirectWindow all{0, N, 0, pl.Ho, 0, pl.Wo}, step = all;
+    if (!direct_geometry(pl, all, C, H, W, K, stride, best, &q)) return SDWINO_ERR_UNSUPPORTED;
+    if (direct_packed_bytes(q) + direct_part_bytes(q) > ws_bytes) {
+        if (!direct_window(pl, N, C, H, W, K, stride, best.splits, ws_bytes, &step)) return SDWINO_ERR_WORKSPACE;
+        // a window has fewer tiles of pixels than the layer: as many channels per tile as are cheapest for it
+        const int splits = best.splits;
+        double best_cost = 1e300;
+        best = DirectShape{0, 0, splits};
+        for (int n = 16; n <= 256; n += 16) {
+            const DirectShape sh{0, n, splits};
+            if (n > 16 && (K + n - 1) / n == (K + n - 17) / (n - 16)) continue;
+            if (!direct_geometry(pl, step, C, H, W, K, stride, sh, &q) || direct_packed_bytes(q) + direct_part_bytes(q) > ws_bytes) continue;
+            const double cost = direct_cost(q, pl.Wo % 8 == 0, sms);
+            if (cost < best_cost) { best_cost = cost; best = sh; }
+        }
+        if (best.n_tile == 0) return SDWINO_ERR_WORKSPACE;
+    }
     CUtensorMap tmU;
     if (!encode_filter_map(&tmU, wt_filters_of(wT), pl.Cb, pl.Kb, 9, best.n_tile / 16)) return err_cuda(__LINE__);
-    return stride == 1 ? launch_direct_as<1>(tmU, q, ws, ws_bytes, st) : launch_direct_as<2>(tmU, q, ws, ws_bytes, st);
+    const long long hw = static_cast<long long>(H) * W, hw_o = static_cast<long long>(pl.Ho) * pl.Wo;
+    for (int n0 = 0; n0 < N; n0 += step.n)
+        for (int r0 = 0; r0 < pl.Ho; r0 += step.h)
+            for (int c0 = 0; c0 < pl.Wo; c0 += step.w) {
+                DirectWindow win{n0, std::min(step.n, N - n0), r0, std::min(step.h, pl.Ho - r0), c0, std::min(step.w, pl.Wo - c0)};
+                if (!direct_geometry(pl, win, C, H, W, K, stride, best, &q)) return SDWINO_ERR_WORKSPACE;
+                direct_finish(&q);
+                const long long first = n0 * K * hw_o + static_cast<long long>(r0) * pl.Wo + c0;
+                q.wt_header = wt_header_of(wT);
+                q.x = x + n0 * C * hw;
+                q.bias = bias;
+                q.y = y + first;
+                q.residual = ep.residual ? static_cast<const __half*>(ep.residual) + first : nullptr;
+                q.act = ep.act;
+                q.vec_store = !q.flat && pl.Wo % 8 == 0 && aligned(y, 16) && aligned(ep.residual, 16);
+                const int rc = stride == 1 ? launch_direct_as<1>(tmU, q, ws, ws_bytes, st) : launch_direct_as<2>(tmU, q, ws, ws_bytes, st);
+                if (rc != SDWINO_OK) return rc;
+            }
+    return SDWINO_OK;
 }
-
 
 int conv_impl(const void* x, const void* wT, const void* bias, void* y, int N, int C, int H, int W, int K, int tile,
               void* ws, size_t ws_bytes, cudaStream_t st, const Epilogue& ep_in = Epilogue{nullptr, 0, nullptr},

@@ -75,7 +75,7 @@ def test_direct_stride_1_agrees_with_winograd_and_passes_and_errors(B):
     y = _direct(B, layer, 1, x, w, b)
     ref = oracle.direct_conv3x3(x.numpy(), w.numpy(), b.numpy())
     assert np.abs(y.double().numpy() - ref).max() <= TOL_REGRESSION * np.abs(ref).max()
-    # several passes through a small workspace give the same bits
+    # a workspace of a tenth gives the same bits (layers that run in several passes or windows: test_gpu_direct_windows.py)
     small = 3 * 128 * 9 * (72 + 200) * 2 + 1024
     y_small = _direct(B, layer, 1, x, w, b, ws_bytes=small)
     assert torch.equal(y, y_small)
