@@ -354,6 +354,12 @@ int sdwino_set_gemm_shape(int ctas, int n_tile);
 int sdwino_set_input_staging(int mode);
 
 /*
+ * Host-only query for tests: the passes a layer takes with tile = 4, fp16 tensors (aligned x) and a workspace of that many
+ * bytes (0: too few, or invalid sizes), and in *staged how many of them take the staged activation transform.
+ */
+int sdwino_selftest_input_passes(int N, int C, int H, int W, int K, size_t workspace_bytes, int *staged);
+
+/*
  * Which of the two supported algorithms is expected to be faster for a layer: returns 2 for F(2x2,3x3),
  * 4 for F(4x4,3x3), 0 for non-positive sizes.  The paper leaves the tile size open; both satisfy the
  * accuracy bound (F4 with about 4x the error of F2).  Rule, with tiles = N * ceil(H/2) * ceil(W/2):

@@ -28,6 +28,7 @@ EXPORTS = [
     "sdwino_conv3x3_f32_scaled", "sdwino_filter_q8_bytes", "sdwino_filter_quantize", "sdwino_conv3x3_q8",
     "sdwino_workspace_bytes_direct", "sdwino_conv3x3_direct", "sdwino_choose_algorithm",
     "sdwino_workspace_bytes_sequence", "sdwino_conv3x3_sequence", "sdwino_selftest_window_reads",
+    "sdwino_selftest_input_passes",
 ]
 
 class SdwinoLayer(ctypes.Structure):
@@ -101,6 +102,8 @@ def _load() -> ctypes.CDLL:
     lib.sdwino_set_input_staging.argtypes = [i]
     lib.sdwino_selftest_wait_timeout.restype = i
     lib.sdwino_selftest_wait_timeout.argtypes = [ctypes.c_ulonglong, vp]
+    lib.sdwino_selftest_input_passes.restype = i
+    lib.sdwino_selftest_input_passes.argtypes = [i, i, i, i, i, sz, ctypes.POINTER(i)]
     lib.sdwino_selftest_window_reads.restype = i
     lib.sdwino_selftest_window_reads.argtypes = [i, i, i, i, i, i, ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(ctypes.c_longlong)]
     lib.sdwino_choose_tile.restype = i
@@ -192,6 +195,12 @@ def sdwino_last_device_status(stream: Optional[torch.cuda.Stream] = None) -> int
 def sdwino_selftest_wait_timeout(limit_ns: int, stream: Optional[torch.cuda.Stream] = None) -> None:
     """Launch the bounded-wait self-test; sdwino_last_device_status() reports ERR_TIMEOUT afterwards."""
     _check(lib.sdwino_selftest_wait_timeout(limit_ns, _stream_ptr(stream)), "sdwino_selftest_wait_timeout")
+
+
+def sdwino_selftest_input_passes(N: int, C: int, H: int, W: int, K: int, workspace_bytes: int):
+    """-> (passes, passes with the staged activation transform) of an F(4x4) layer; see include/sdwino.h."""
+    staged = ctypes.c_int(0)
+    return int(lib.sdwino_selftest_input_passes(N, C, H, W, K, workspace_bytes, staged)), staged.value
 
 
 def sdwino_selftest_window_reads(N: int, C: int, H: int, W: int, tile: int, odd_start: bool):

@@ -496,6 +496,15 @@ bool use_input_tma(const TileGeom& geo, int N, int C, const void* x, long long p
     return g_input_staging == 2 || (geo.TW % 16 == 0 && large);
 }
 
+// Several passes of F(4x4): cut at whole tile rows where the passes that result then take the staged transform.
+long long cut_passes(const Plan& pl, int N, int C, int H, int W, const void* x, long long pc) {
+    if (pc >= pl.P128) return pc;
+    long long a = pl.TW, b = GEMM_BLOCK_P;
+    while (b != 0) { const long long t = a % b; a = b; b = t; }
+    const long long lcm = static_cast<long long>(pl.TW) / a * GEMM_BLOCK_P, cut = pc / lcm * lcm;
+    return cut > 0 && use_input_tma(make_geom(H, W, pl.TH, pl.TW, pl.P), N, C, x, 0, cut) ? cut : pc;
+}
+
 int launch_input_tma(const __half* x, __half* V, const TileGeom& geo, int N, int C, long long p_begin, long long p_count,
                      long long Pstride, cudaStream_t st) {
     ProfScope prof(KIND_INPUT, st);
@@ -1348,14 +1357,7 @@ int conv_impl(const void* x, const void* wT, const void* bias, void* y, int N, i
                                      N, C, H, W, K, stride, ws, ws_bytes, ep_in, st);
         if (rc != SDWINO_ERR_UNSUPPORTED) return rc;
     }
-    if (tile == 4 && pc < pl.P128) {
-        // several passes: cut them at whole tile rows where that keeps the TMA-staged activation transform usable
-        const TileGeom g0 = make_geom(H, W, pl.TH, pl.TW, pl.P);
-        long long a = pl.TW, b = GEMM_BLOCK_P;
-        while (b != 0) { const long long t = a % b; a = b; b = t; }
-        const long long lcm = static_cast<long long>(pl.TW) / a * GEMM_BLOCK_P;
-        if (pc >= lcm && !io32 && use_input_tma(g0, N, C, x, 0, lcm)) pc = pc / lcm * lcm;
-    }
+    if (tile == 4 && !io32) pc = cut_passes(pl, N, C, H, W, x, pc);
     Epilogue ep = ep_in;
     if (range_safe) {
         // fp32 interface, range-safe call: max|x| goes into a word at the end of the workspace, which the transforms
@@ -2075,6 +2077,19 @@ void window_reads(int N, int C, int H, int W, uintptr_t x, long long* before, lo
 }  // namespace
 
 extern "C" {
+int sdwino_selftest_input_passes(int N, int C, int H, int W, int K, size_t workspace_bytes, int* staged) {
+    Plan pl;
+    if (!staged || !make_plan(N, C, H, W, K, 4, &pl)) return 0;
+    const void* x = reinterpret_cast<const void*>(uintptr_t(1) << 20);     // any aligned address
+    long long pc = tiles_per_pass(pl, workspace_bytes);
+    if (pc < GEMM_BLOCK_P) return 0;
+    pc = cut_passes(pl, N, C, H, W, x, pc);
+    int passes = *staged = 0;
+    for (long long p0 = 0; p0 < pl.P; p0 += pc, ++passes)
+        *staged += use_input_tma(make_geom(H, W, pl.TH, pl.TW, pl.P), N, C, x, p0, std::min(pc, pl.P128 - p0));
+    return passes;
+}
+
 int sdwino_selftest_window_reads(int N, int C, int H, int W, int tile, int odd_start, long long* before, long long* after) {
     if (N <= 0 || C <= 0 || H <= 0 || W <= 0 || !before || !after) return SDWINO_ERR_INVALID_ARG;
     if (tile != 2 && tile != 4) return SDWINO_ERR_UNSUPPORTED;
