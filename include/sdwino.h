@@ -347,7 +347,8 @@ int sdwino_set_gemm_shape(int ctas, int n_tile);
  * they can stage their operands in shared memory by TMA, several channels ahead of the arithmetic (the
  * overlapping input tiles of a block; the 36 transform positions of a block of tiles), instead of loading them
  * into registers; both forms produce the same bits.  mode 1 (the default) stages where that measured faster
- * (activation transform: W % 64 == 0; output transform: passes of 512 tiles or more), mode 2 wherever it is
+ * (activation transform: W % 64 == 0 and transformed activations of more than half the L2 cache, 2.5 times the L2 cache
+ * where a row has fewer than 64 tiles; output transform: passes of 512 tiles or more), mode 2 wherever it is
  * possible, mode 0 never.  Returns SDWINO_ERR_INVALID_ARG for any other value.  Not thread-safe against
  * concurrent compute calls.
  */

@@ -7,8 +7,8 @@
 // origin is rounded down to a 16-byte boundary, as TMA requires; the rows and columns outside the image are the
 // zero padding of the convolution and come back as zeros from the TMA unit, so the kernel has no border code at
 // all).  Loads run up to IN_TMA_STAGES steps ahead of the arithmetic, which is what the register-only kernel
-// (input_transform_f4_kernel: load, wait, compute, store per thread) lacks: worth it where V is far larger than L2
-// (512 channels at 512x512 147 us against 176).  A thread reads the six rows of its two tiles from
+// (input_transform_f4_kernel: load, wait, compute, store per thread) lacks: worth it on layers whose V does not fit L2
+// (512 channels at 512x512 148 us against 172).  A thread reads the six rows of its two tiles from
 // shared memory (one 16-byte and two 4-byte reads per row), releases the stage and applies B^T . B in packed
 // two-wide fp32 exactly like the register-only kernel, so both produce the same bits.
 //

@@ -98,6 +98,7 @@ constexpr int MAX_DYN_SMEM = 232448;  // 227 KB opt-in limit per CTA on sm_100
 // with 64 MB passes, 216 us with 128 MB, 202 us in a single pass).  The cap only bounds the memory asked for.
 constexpr size_t PASS_BUDGET = 4096ull << 20;
 constexpr size_t WS_ALIGN = 1024;
+constexpr size_t L2_BYTES = 126ull << 20;
 constexpr int STATIC_MAX_DEVICES_HOST = 64;
 
 // SDWINO_ERR_CUDA, with the place and the runtime's last error on stderr when SDWINO_LOG is set
@@ -486,14 +487,19 @@ bool use_input_tma(const TileGeom& geo, int N, int C, const void* x, long long p
     const bool possible = input_tma_possible(geo, N, C, x) && p_begin % geo.TW == 0 &&
                           (p_count % geo.TW == 0 || p_begin + p_count >= geo.P);
     if (!possible || g_input_staging == 0) return false;
-    // Faster where V is more than twice the L2 cache and a block row is a whole number of its 32-byte sectors (W % 64 == 0):
-    // 512 channels at 512x512 147 us against 176 with the register-only kernel, 256 channels at 1024x1024 293 / 316, at
-    // 768x768 177 / 187.  Below, the register-only kernel is, whose warps do not wait for one another: 320 channels at 64x64,
-    // batch 8, 15.7 / 12.1, 512 channels at 128x128 12.8 / 9.4, at 256x256 50 / 41 (V 151 MB), 256 channels at 512x512
-    // 82 / 80 (302 MB).  Other widths are up to 2x slower at any size: their rows leave runs of V that start and end inside
-    // sectors, where the register-only kernel, whose threads follow the tile index, always stores whole 128-byte lines.
-    const bool large = 72ll * C * p_count > (304ll << 20);
-    return g_input_staging == 2 || (geo.TW % 16 == 0 && large);
+    if (g_input_staging == 2) return true;
+    // A block row is a whole number of the 32-byte sectors of V (W % 64 == 0).  Other widths are up to 2x slower at any size:
+    // their rows leave runs of V that start and end inside sectors, where the register-only kernel, whose threads follow the
+    // tile index, always stores whole 128-byte lines.
+    if (geo.TW % 16 != 0) return false;
+    // Inside a pass over many layers (us of a layer, staged / registers): rows of at least 64 tiles gain from V of half the L2
+    // cache on, 512->512 at 256x256 146.5 / 148.7 (V 151 MB), 256->256 at 256x256 67.1 / 68.9 (75 MB), 128->128 at 384x384
+    // 79.3 / 82.3 (85 MB), 256->256 at 512x512 243 / 251 (302 MB), at 1024x1024 966 / 1001; not where the blocks leave a sixth
+    // of a row's threads idle, 256->256 at 320x320 114.2 / 111.8 (118 MB).  Narrower rows from twice that on: 320->320 at
+    // 128x128, batch 4, 100.6 / 98.8 (94 MB), 640->320 at 192x192, batch 2, 177 / 173 (212 MB), 960->640 at 128x128, batch 4,
+    // 275 / 278 (283 MB); the register-only kernel's warps do not wait for one another, 512->512 at 128x128 44.5 / 42.5.
+    const bool wide = geo.TW >= 64 && round_up(geo.TW, 32) * 7 <= geo.TW * 8;
+    return 72ll * C * p_count > static_cast<long long>(wide ? L2_BYTES / 2 : 5 * L2_BYTES / 2);
 }
 
 // Several passes of F(4x4): cut at whole tile rows where the passes that result then take the staged transform.
@@ -528,10 +534,14 @@ int launch_input_tma(const __half* x, __half* V, const TileGeom& geo, int N, int
     int best_half = 1, best_trb = 1;
     double best_score = -1e30;
     const int half_full = geo.TW / 2;   // W % 8 == 0: TW is even
+    // Blocks narrower than the image are whole sectors of V (16 tiles) wide where the rows are: 256->256 at 576x576 in blocks
+    // of 36 tiles (which leave no thread idle) 422 us, in blocks of 48 323; at 832x832, K = 128, 52 tiles 798, 32 tiles 535.
+    const int half_step = geo.TW % 16 == 0 ? 8 : 1;
     // two boxes side by side where a block row can then be 64 tiles = one 128-byte line of V per warp store
     // (256->256 at 1024x1024: 365 -> 340 us)
     q.nb = geo.TW % 64 == 0 ? 2 : 1;
-    for (int half = (half_full <= 30 ? half_full : 16); half <= (half_full <= 30 ? half_full : 30); ++half) {
+    for (int half = (half_full <= 30 ? half_full : 16); half <= (half_full <= 30 ? half_full : 30);
+         half += half_step) {
         const int sbc = (geo.TW + 2 * half * q.nb - 1) / (2 * half * q.nb);
         for (int trb = 1; trb <= 32 && half * q.nb * trb <= 128; ++trb) {
             const int sbr = (geo.TH + trb - 1) / trb;

@@ -27,3 +27,14 @@ def test_one_pass(B):
     assert B.sdwino_selftest_input_passes(1, 320, 64, 64, 320, 1 << 30) == (1, 0)        # small: registers
     assert B.sdwino_selftest_input_passes(1, 512, 516, 516, 512, 4 << 30) == (1, 0)      # rows that are not whole sectors of V
     assert B.sdwino_selftest_input_passes(1, 512, 512, 512, 512, 1000)[0] == 0
+
+
+@pytest.mark.parametrize("shape, expected", [
+    # N, C, H, W, K: rows of 64 tiles or more from half the L2 cache on
+    ((1, 512, 256, 256, 512), 1), ((1, 256, 256, 256, 256), 1), ((1, 256, 512, 512, 128), 1), ((1, 128, 512, 512, 128), 1),
+    ((1, 128, 256, 256, 128), 0), ((1, 256, 320, 320, 256), 0), ((2, 512, 320, 320, 512), 1),
+    # narrower rows: 2.5 times the L2 cache
+    ((2, 960, 128, 128, 320), 0), ((4, 1280, 128, 128, 640), 1), ((1, 512, 128, 128, 512), 0),
+])
+def test_where_the_staged_transform_is_taken(B, shape, expected):
+    assert B.sdwino_selftest_input_passes(*shape, B.sdwino_workspace_bytes(*shape, 4)) == (1, expected)
