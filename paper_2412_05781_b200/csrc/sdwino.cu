@@ -847,6 +847,127 @@ GemmShape choose_gemm_shape(int K, int C, long long p_tiles128, int a2, int sms,
     return best;
 }
 
+// Everything about the GEMM launch of a pass of pc tiles that its sizes decide.  one_pass: the layer is this pass.  force_*:
+// the test hook's shape.  false: no room for the rings of 8-bit filters.
+bool plan_gemm(int K, int C, long long pc, bool one_pass, int a2, int sms, int force_ctas, int force_n_tile, bool q8,
+               GemmShape* shape_out, GemmParams* prm_out) {
+    GemmParams& prm = *prm_out;
+    const bool forced = force_ctas != 0 || force_n_tile != 0;
+    GemmShape shape = choose_gemm_shape(K, C, pc / GEMM_BLOCK_P, a2, sms, q8 ? 1 : force_ctas);
+    if (q8) shape.dual = 0;
+    if (force_n_tile >= 16 && force_n_tile <= GEMM_MAX_N && force_n_tile % 16 == 0) shape.n_tile = force_n_tile;
+    if (shape.ctas == 2) shape.n_tile = round_up(shape.n_tile, 32);  // each CTA of a pair loads whole 16-row blocks
+    if (force_n_tile != 0) shape.dual = 0;
+    *shape_out = shape;
+    prm.K = K;
+    prm.C = C;
+    prm.n_tile = shape.n_tile;
+    prm.num_k_tiles = (K + prm.n_tile - 1) / prm.n_tile;
+    prm.num_pos = a2;
+    prm.fd_k = make_fastdiv(static_cast<uint32_t>(prm.num_k_tiles));
+    prm.fd_keys = make_fastdiv(static_cast<uint32_t>(prm.num_k_tiles * a2));
+    prm.num_c_blocks = (C + GEMM_BLOCK_C - 1) / GEMM_BLOCK_C;
+    const int b_rows = prm.n_tile / shape.ctas;
+    prm.dual = shape.dual;
+    prm.acc_bufs = dual_acc_bufs(prm.n_tile);
+    prm.acc_stride = prm.acc_bufs == 2 ? GEMM_MAX_N : prm.n_tile;
+    prm.resident = 0;
+    prm.group = 1;
+    {
+        // Single CTAs, one pass, at most one tile per CTA: the epilogue borrows the first pipeline stages, and the
+        // ring gets the 16-64 KB of the staging buffer (SD v2.1 sweep at batch 1, whose 144-tile layers run two
+        // blocks per CTA tile on three stages otherwise: 0.440 -> 0.425 ms; SD v1.5 sweep 0.3379 -> 0.3367 ms).
+        // A forced GEMM shape (test hook) keeps the separate buffer, so the tests that compare forced with automatic
+        // shapes bit for bit compare both placements.
+        const long long p_blocks = shape.dual ? 2 : 1;
+        const long long tiles = ((pc / GEMM_BLOCK_P + p_blocks - 1) / p_blocks) * prm.num_k_tiles * a2;
+        prm.epi_alias = (shape.ctas == 1 && one_pass && tiles <= sms && !forced) ? 1 : 0;
+    }
+    const EpiPlan whole = plan_epilogue(prm.n_tile, shape.ctas, shape.dual != 0, prm.epi_alias != 0, false);
+    const EpiPlan e = q8 || forced ? whole : plan_epilogue(prm.n_tile, shape.ctas, shape.dual != 0, prm.epi_alias != 0, true);
+    prm.epi_rows = e.rows;
+    prm.epi_bufs = e.bufs;
+    prm.epi_chunks = e.chunks;
+    prm.stages = e.stages;
+    prm.raw_slots = 0;
+    if (q8) {
+        // 8-bit filters: give up one operand stage (down to three at least) for a ring of raw filter boxes, which is
+        // what keeps the weight stream from HBM deep: a raw slot is a third of an operand stage or less
+        // The epilogue stages 32 channels at a time where that divides its half of the tile: the rings are short of memory
+        // (2560->1280 at 26x45, batch 4, n_tile 256: 155-176 -> 138 us; 16 at a time, for n_tile 160, costs 3-8 %).
+        if (!prm.epi_alias && prm.epi_rows > 32 && prm.epi_rows % 32 == 0) {
+            prm.epi_chunks = prm.epi_rows / 32;
+            prm.epi_rows = 32;
+        }
+        const int room = MAX_DYN_SMEM - GemmSmemLayout::dyn_bytes(b_rows, 0, prm.epi_rows, prm.epi_alias ? 0 : prm.epi_bufs);
+        const int raw = GemmSmemLayout::raw_bytes(b_rows), stage = GemmSmemLayout::stage_bytes(b_rows);
+        int best_s = 0, best_r = 0;
+        for (int sgs = 2; sgs <= GEMM_MAX_STAGES; ++sgs) {
+            int r = (room - sgs * stage) / raw;
+            if (r > GEMM_MAX_STAGES) r = GEMM_MAX_STAGES;
+            if (r < sgs + 1) continue;                       // the raw ring leads the operand ring
+            if (sgs <= 3 || r >= 6) { best_s = sgs; best_r = r; }
+        }
+        if (best_s == 0) return false;
+        prm.stages = best_s;
+        prm.raw_slots = best_r;
+    }
+    {
+        // Filter-resident mode (see wino_gemm.cuh): single CTAs, many tiles per CTA and long runs of tiles per
+        // (position, k-tile), the filter block two thirds of a stage (n_tile 224-256), and room for it beside a ring
+        // of at least four V stages once the epilogue stages 64 channels at a time.  Measured: 256->256 at 512x512
+        // GEMM 146 -> 120 us, at 1024x1024 570 -> 472 us; with n_tile 128-160 (filters half of a stage or less, the
+        // layer close to the HBM roof already) the pause at every change of filter block costs more than the
+        // re-reads: 128->128 at 512x512 57 -> 74 us.
+        const long long workers = sms / shape.ctas;
+        const long long p_tiles = (pc / GEMM_BLOCK_P + shape.ctas - 1) / shape.ctas;     // tiles of 128 (256) tiles p
+        const long long keys = prm.num_k_tiles * static_cast<long long>(a2);
+        const int ures = prm.num_c_blocks * GemmSmemLayout::b_bytes(b_rows);
+        const int grp = whole.rows;
+        const int rows = (grp > 64 && grp % 64 == 0) ? 64 : grp;   // (32 at a time for a fifth stage measured 2-10 % slower)
+        const int stages = (MAX_DYN_SMEM - GemmSmemLayout::dyn_bytes(0, 0, rows, prm.epi_bufs, ures)) / GemmSmemLayout::A_BYTES;
+        // (CTA pairs gain nothing from it: with their half of a 512-channel block resident only four 16 KB stages
+        // of V remain, too few bytes in flight: 512->512 at 256x256 99 against 94 us)
+        if (!q8 && !forced && shape.ctas == 1 && !shape.dual && p_tiles >= 16 && keys * p_tiles >= 4 * workers &&
+            prm.n_tile >= 224 && stages >= 4) {
+            prm.resident = 1;
+            // CTAs per (position, k-tile) pair.  A group walks `rounds` pairs, each CTA `run` tiles per pair,
+            // and every change of pair costs about a tile and a half (the MMAs that read the old filter block drain,
+            // the new block arrives): the group size with the smallest rounds * (run + 1.5) wins, larger groups on
+            // ties (their CTAs read neighbouring pieces of V at the same time); runs of at least 8 tiles.
+            auto cost = [&](int g) {
+                const long long ng = workers / g;
+                const long long rounds = (keys + ng - 1) / ng;
+                const long long run = (p_tiles + g - 1) / g;
+                return static_cast<double>(rounds) * (static_cast<double>(run) + 1.5);
+            };
+            const int g_max = static_cast<int>(std::min<long long>(workers, p_tiles / 8));
+            int best_g = 1;
+            for (int g = 2; g <= g_max; ++g)
+                if (cost(g) <= cost(best_g) + 1e-9) best_g = g;
+            prm.group = best_g;
+            prm.epi_chunks = grp / rows;
+            prm.epi_rows = rows;
+            prm.stages = stages > GEMM_MAX_STAGES ? GEMM_MAX_STAGES : stages;
+        }
+    }
+    // Epilogue staging: stmatrix into swizzled boxes where a CTA has several tiles (throughput: 3-8 % on those GEMMs),
+    // plain 2-byte stores into one box where it has one (its two TMA stores of 128-byte rows drain later at the tail
+    // of the launch: 0.5-1.5 us per layer of the SD v1.5 sweep).
+    prm.epi_dbuf = 0;
+    if (!q8 && prm.epi_chunks >= 2 && prm.epi_rows == 64) {
+        // Two buffers of 32 channels in the place of one of 64: a group then stages one piece while the TMA store still
+        // reads the other, instead of waiting 1.3-1.8 thousand cycles for it between the pieces (-1.5 to -2 % on the
+        // GEMMs with several tiles per CTA).
+        prm.epi_dbuf = 1;
+        prm.epi_rows = 32;
+        prm.epi_chunks *= 2;
+        prm.epi_bufs *= 2;
+    }
+    prm.epi_stm = (!q8 && !prm.epi_alias) ? 1 : 0;   // (an aliased staging buffer implies single CTAs in streaming mode)
+    return true;
+}
+
 template <int CTAS, bool RES, bool DUAL = false, bool U8 = false, bool STM = true>
 int launch_gemm_shape(const CUtensorMap& tmU, const CUtensorMap& tmV, const CUtensorMap& tmM, const GemmParams& prm,
                       int sms, int* status, cudaStream_t st) {
@@ -1440,132 +1561,15 @@ int conv_impl(const void* x, const void* wT, const void* bias, void* y, int N, i
     const int sms = sm_count();
     if (sms <= 0) return err_cuda(__LINE__);
     GemmParams prm;
+    GemmShape shape;
+    if (!plan_gemm(K, C, pc, pc >= pl.P128, pl.a2, sms, force_ctas, force_n_tile, q8, &shape, &prm)) return SDWINO_ERR_UNSUPPORTED;
     prm.wt_header = wt_header_of(wT);
-    prm.K = K;
     prm.tile = q8 ? (tile | static_cast<int>(WT_Q8_FLAG)) : tile;
     prm.scales = q8 ? reinterpret_cast<const float*>(static_cast<const uint8_t*>(wT) + WT_HEADER_BYTES +
                                                       q8_bytes_part(pl.a2, pl.Kb, pl.Cb))
                     : nullptr;
     prm.kpad = pl.Kb * 16;
-    GemmShape shape = choose_gemm_shape(K, C, pc / GEMM_BLOCK_P, pl.a2, sms, q8 ? 1 : force_ctas);
-    if (q8) shape.dual = 0;
-    if (force_n_tile >= 16 && force_n_tile <= GEMM_MAX_N && force_n_tile % 16 == 0) shape.n_tile = force_n_tile;
-    if (shape.ctas == 2) shape.n_tile = round_up(shape.n_tile, 32);  // each CTA of a pair loads whole 16-row blocks
-    prm.n_tile = shape.n_tile;
-    prm.num_k_tiles = (K + prm.n_tile - 1) / prm.n_tile;
-    prm.num_pos = pl.a2;
-    prm.fd_k = make_fastdiv(static_cast<uint32_t>(prm.num_k_tiles));
-    prm.fd_keys = make_fastdiv(static_cast<uint32_t>(prm.num_k_tiles * pl.a2));
-    prm.num_c_blocks = (C + GEMM_BLOCK_C - 1) / GEMM_BLOCK_C;
-    prm.C = C;
     const int b_rows = prm.n_tile / shape.ctas;
-    if (force_n_tile != 0) shape.dual = 0;
-    prm.dual = shape.dual;
-    prm.acc_bufs = dual_acc_bufs(prm.n_tile);
-    prm.acc_stride = prm.acc_bufs == 2 ? GEMM_MAX_N : prm.n_tile;
-    // epilogue staging: two groups of epilogue warps each take half a tile when that is a multiple of 16 channels
-    const bool split = (prm.n_tile / 2) % 16 == 0;
-    prm.epi_rows = split ? prm.n_tile / 2 : prm.n_tile;
-    prm.epi_bufs = split ? 2 : 1;
-    prm.epi_chunks = 1;
-    prm.resident = 0;
-    prm.group = 1;
-    {
-        // Single CTAs, one pass, at most one tile per CTA: the epilogue borrows the first pipeline stages, and the
-        // ring gets the 16-64 KB of the staging buffer (SD v2.1 sweep at batch 1, whose 144-tile layers run two
-        // blocks per CTA tile on three stages otherwise: 0.440 -> 0.425 ms; SD v1.5 sweep 0.3379 -> 0.3367 ms).
-        // A forced GEMM shape (test hook) keeps the separate buffer, so the tests that compare forced with automatic
-        // shapes bit for bit compare both placements.
-        const long long p_blocks = shape.dual ? 2 : 1;
-        const long long tiles = ((pc / GEMM_BLOCK_P + p_blocks - 1) / p_blocks) * prm.num_k_tiles * pl.a2;
-        prm.epi_alias = (shape.ctas == 1 && pc >= pl.P128 && tiles <= sms && force_ctas == 0 && force_n_tile == 0) ? 1 : 0;
-    }
-    prm.stages = (MAX_DYN_SMEM - GemmSmemLayout::dyn_bytes(b_rows, 0, prm.epi_rows, prm.epi_alias ? 0 : prm.epi_bufs)) /
-                 (GemmSmemLayout::stage_bytes(b_rows) + (shape.dual ? GemmSmemLayout::A_BYTES : 0));
-    if (prm.stages > GEMM_MAX_STAGES) prm.stages = GEMM_MAX_STAGES;
-    prm.raw_slots = 0;
-    if (q8) {
-        // 8-bit filters: give up one operand stage (down to three at least) for a ring of raw filter boxes, which is
-        // what keeps the weight stream from HBM deep: a raw slot is a third of an operand stage or less
-        // The epilogue stages 32 channels at a time where that divides its half of the tile: the rings are short of memory
-        // (2560->1280 at 26x45, batch 4, n_tile 256: 155-176 -> 138 us; 16 at a time, for n_tile 160, costs 3-8 %).
-        if (!prm.epi_alias && prm.epi_rows > 32 && prm.epi_rows % 32 == 0) {
-            prm.epi_chunks = prm.epi_rows / 32;
-            prm.epi_rows = 32;
-        }
-        const int room = MAX_DYN_SMEM - GemmSmemLayout::dyn_bytes(b_rows, 0, prm.epi_rows, prm.epi_alias ? 0 : prm.epi_bufs);
-        const int raw = GemmSmemLayout::raw_bytes(b_rows), stage = GemmSmemLayout::stage_bytes(b_rows);
-        int best_s = 0, best_r = 0;
-        for (int sgs = 2; sgs <= GEMM_MAX_STAGES; ++sgs) {
-            int r = (room - sgs * stage) / raw;
-            if (r > GEMM_MAX_STAGES) r = GEMM_MAX_STAGES;
-            if (r < sgs + 1) continue;                       // the raw ring leads the operand ring
-            if (sgs <= 3 || r >= 6) { best_s = sgs; best_r = r; }
-        }
-        if (best_s == 0) return SDWINO_ERR_UNSUPPORTED;
-        prm.stages = best_s;
-        prm.raw_slots = best_r;
-    }
-    {
-        // Filter-resident mode (see wino_gemm.cuh): single CTAs, many tiles per CTA and long runs of tiles per
-        // (position, k-tile), the filter block two thirds of a stage (n_tile 224-256), and room for it beside a ring
-        // of at least four V stages once the epilogue stages 64 channels at a time.  Measured: 256->256 at 512x512
-        // GEMM 146 -> 120 us, at 1024x1024 570 -> 472 us; with n_tile 128-160 (filters half of a stage or less, the
-        // layer close to the HBM roof already) the pause at every change of filter block costs more than the
-        // re-reads: 128->128 at 512x512 57 -> 74 us.
-        const long long workers = sms / shape.ctas;
-        const long long p_tiles = (pc / GEMM_BLOCK_P + shape.ctas - 1) / shape.ctas;     // tiles of 128 (256) tiles p
-        const long long keys = ((K + prm.n_tile - 1) / prm.n_tile) * static_cast<long long>(pl.a2);
-        const int ures = prm.num_c_blocks * GemmSmemLayout::b_bytes(b_rows);
-        const int grp = prm.epi_rows;
-        const int rows = (grp > 64 && grp % 64 == 0) ? 64 : grp;   // (32 at a time for a fifth stage measured 2-10 % slower)
-        const int stages = (MAX_DYN_SMEM - GemmSmemLayout::dyn_bytes(0, 0, rows, prm.epi_bufs, ures)) / GemmSmemLayout::A_BYTES;
-        // (CTA pairs gain nothing from it: with their half of a 512-channel block resident only four 16 KB stages
-        // of V remain, too few bytes in flight: 512->512 at 256x256 99 against 94 us)
-        if (!q8 && shape.ctas == 1 && !shape.dual && force_ctas == 0 && force_n_tile == 0 && p_tiles >= 16 && keys * p_tiles >= 4 * workers &&
-            prm.n_tile >= 224 && stages >= 4) {
-            prm.resident = 1;
-            // CTAs per (position, k-tile) pair.  A group walks `rounds` pairs, each CTA `run` tiles per pair,
-            // and every change of pair costs about a tile and a half (the MMAs that read the old filter block drain,
-            // the new block arrives): the group size with the smallest rounds * (run + 1.5) wins, larger groups on
-            // ties (their CTAs read neighbouring pieces of V at the same time); runs of at least 8 tiles.
-            auto cost = [&](int g) {
-                const long long ng = workers / g;
-                const long long rounds = (keys + ng - 1) / ng;
-                const long long run = (p_tiles + g - 1) / g;
-                return static_cast<double>(rounds) * (static_cast<double>(run) + 1.5);
-            };
-            const int g_max = static_cast<int>(std::min<long long>(workers, p_tiles / 8));
-            int best_g = 1;
-            for (int g = 2; g <= g_max; ++g)
-                if (cost(g) <= cost(best_g) + 1e-9) best_g = g;
-            prm.group = best_g;
-            prm.epi_chunks = grp / rows;
-            prm.epi_rows = rows;
-            prm.stages = stages > GEMM_MAX_STAGES ? GEMM_MAX_STAGES : stages;
-        }
-    }
-
-    if (!prm.resident && !prm.epi_alias && !q8 && force_ctas == 0 && force_n_tile == 0) {
-        const EpiPlan e = plan_epilogue(prm.n_tile, shape.ctas, shape.dual != 0, false, true);
-        prm.epi_chunks = e.chunks;
-        prm.epi_rows = e.rows;
-        prm.stages = e.stages;
-    }
-    // Epilogue staging: stmatrix into swizzled boxes where a CTA has several tiles (throughput: 3-8 % on those GEMMs),
-    // plain 2-byte stores into one box where it has one (its two TMA stores of 128-byte rows drain later at the tail
-    // of the launch: 0.5-1.5 us per layer of the SD v1.5 sweep).
-    prm.epi_dbuf = 0;
-    if (!q8 && prm.epi_chunks >= 2 && prm.epi_rows == 64) {
-        // Two buffers of 32 channels in the place of one of 64: a group then stages one piece while the TMA store still
-        // reads the other, instead of waiting 1.3-1.8 thousand cycles for it between the pieces (-1.5 to -2 % on the
-        // GEMMs with several tiles per CTA).
-        prm.epi_dbuf = 1;
-        prm.epi_rows = 32;
-        prm.epi_chunks *= 2;
-        prm.epi_bufs *= 2;
-    }
-    prm.epi_stm = (!q8 && !prm.epi_alias) ? 1 : 0;   // (an aliased staging buffer implies single CTAs in streaming mode)
     prm.p_stride = pc;
     CUtensorMap tmU, tmV, tmM;
     if (!(q8 ? encode_filter_map_q8(&tmU, wt_filters_of(wT), pl.Cb, pl.Kb, pl.a2, b_rows / 16)
