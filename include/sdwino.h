@@ -343,6 +343,13 @@ unsigned long long sdwino_launch_count(void);
 int sdwino_set_gemm_shape(int ctas, int n_tile);
 
 /*
+ * Host-only query for tests: the shape the GEMM of a layer (fp16 filters, no override) takes on 148 SMs in a workspace of
+ * that many bytes: CTAs per tile, output channels per tile, blocks of 128 tiles per CTA tile, stages of the operand ring.
+ */
+int sdwino_selftest_gemm_shape(int N, int C, int H, int W, int K, int tile, size_t workspace_bytes, int *ctas, int *n_tile,
+                               int *blocks, int *stages);
+
+/*
  * Test hook for the transforms of steps (i) and (iii) with tile = 4.  With W % 8 == 0 and 16-byte aligned x / y
  * they can stage their operands in shared memory by TMA, several channels ahead of the arithmetic (the
  * overlapping input tiles of a block; the 36 transform positions of a block of tiles), instead of loading them

@@ -28,7 +28,7 @@ EXPORTS = [
     "sdwino_conv3x3_f32_scaled", "sdwino_filter_q8_bytes", "sdwino_filter_quantize", "sdwino_conv3x3_q8",
     "sdwino_workspace_bytes_direct", "sdwino_conv3x3_direct", "sdwino_choose_algorithm",
     "sdwino_workspace_bytes_sequence", "sdwino_conv3x3_sequence", "sdwino_selftest_window_reads",
-    "sdwino_selftest_input_passes",
+    "sdwino_selftest_input_passes", "sdwino_selftest_gemm_shape",
 ]
 
 class SdwinoLayer(ctypes.Structure):
@@ -104,6 +104,8 @@ def _load() -> ctypes.CDLL:
     lib.sdwino_selftest_wait_timeout.argtypes = [ctypes.c_ulonglong, vp]
     lib.sdwino_selftest_input_passes.restype = i
     lib.sdwino_selftest_input_passes.argtypes = [i, i, i, i, i, sz, ctypes.POINTER(i)]
+    lib.sdwino_selftest_gemm_shape.restype = i
+    lib.sdwino_selftest_gemm_shape.argtypes = [i] * 6 + [sz] + [ctypes.POINTER(i)] * 4
     lib.sdwino_selftest_window_reads.restype = i
     lib.sdwino_selftest_window_reads.argtypes = [i, i, i, i, i, i, ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(ctypes.c_longlong)]
     lib.sdwino_choose_tile.restype = i
@@ -201,6 +203,13 @@ def sdwino_selftest_input_passes(N: int, C: int, H: int, W: int, K: int, workspa
     """-> (passes, passes with the staged activation transform) of an F(4x4) layer; see include/sdwino.h."""
     staged = ctypes.c_int(0)
     return int(lib.sdwino_selftest_input_passes(N, C, H, W, K, workspace_bytes, staged)), staged.value
+
+
+def sdwino_selftest_gemm_shape(N: int, C: int, H: int, W: int, K: int, tile: int, workspace_bytes: int):
+    """-> (CTAs per tile, output channels per tile, blocks of 128 tiles per CTA tile, ring stages); see include/sdwino.h."""
+    out = [ctypes.c_int(0) for _ in range(4)]
+    _check(lib.sdwino_selftest_gemm_shape(N, C, H, W, K, tile, workspace_bytes, *out), "sdwino_selftest_gemm_shape")
+    return tuple(v.value for v in out)
 
 
 def sdwino_selftest_window_reads(N: int, C: int, H: int, W: int, tile: int, odd_start: bool):

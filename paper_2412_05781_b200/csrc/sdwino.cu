@@ -810,16 +810,31 @@ int dual_acc_bufs(int n_tile) { return std::max(2, std::min(GEMM_MAX_ACC, 2 * GE
 // as single CTAs), and its epilogue, which crosses two CTAs, 1.66 times as much; tiles of fewer than 8 stages and launches
 // of one or two tiles per pair measured 4-35 % slower as pairs and are not offered.  Two blocks of tiles per CTA
 // tile (see wino_gemm.cuh) share a filter box, but their epilogues are added to the mainloop.
+//
+// Launches that HBM bounds, few channels and every piece of V read once: V and M stream at 6 TB/s, which 64 KB of V in
+// flight per SM sustain, and every further stage only makes the reads and writes interfere.  So no two blocks of tiles per
+// CTA, and stages up to 96 KB (112 from four blocks of channels on) of V and of the tile of M together: 256->128 at
+// 1024x1024 320 us with two blocks of tiles, 316 with six stages, 290 with five, 293 with four; 128->128 at 1024x1024 230
+// with six, 223 with five, 205 with four, 220 with three; 128->64 at 768x768 97 with eight, 85 with five.
+bool gemm_streams_hbm(int K, int C, long long tiles, int a2) {
+    return K <= GEMM_MAX_N && C <= 5 * GEMM_BLOCK_C && 2ll * a2 * (C + K) * tiles > 2ll * static_cast<long long>(L2_BYTES);
+}
+int streaming_stages(int c_blocks, int n_tile) {
+    if (c_blocks > 4) return GEMM_MAX_STAGES;      // 320->160 at 512x512: 97 with five stages, all it has, 105 with four
+    return std::max(4, ((c_blocks == 4 ? 112 : 96) - n_tile / 4) / 16);
+}
+
 struct GemmShape { int ctas; int n_tile; int dual; };   // dual: two blocks of 128 tiles per CTA tile (single CTAs)
 GemmShape choose_gemm_shape(int K, int C, long long p_tiles128, int a2, int sms, int force_ctas) {
     const long long cblocks = (C + GEMM_BLOCK_C - 1) / GEMM_BLOCK_C;
+    const bool streams = gemm_streams_hbm(K, C, p_tiles128 * GEMM_BLOCK_P, a2);
     GemmShape best{1, 16, 0};
     double best_cost = 1e300;
     const int max_ctas = p_tiles128 >= 2 && (cblocks >= 8 || force_ctas == 2) ? 2 : 1;
     for (int kind = 0; kind < 3; ++kind) {            // single CTAs, CTA pairs, single CTAs with two blocks of tiles
         const int ctas = kind == 1 ? 2 : 1;
         const bool dual = kind == 2;
-        if (ctas > max_ctas || (dual && (force_ctas != 0 || p_tiles128 < 2))) continue;
+        if (ctas > max_ctas || (dual && (force_ctas != 0 || p_tiles128 < 2 || streams))) continue;
         if (force_ctas != 0 && ctas != (force_ctas < max_ctas ? force_ctas : max_ctas)) continue;
         const int blocks = kind == 0 ? 1 : 2;         // blocks of 128 tiles per tile of the launch
         const long long p_tiles = (p_tiles128 + blocks - 1) / blocks;
@@ -951,6 +966,8 @@ bool plan_gemm(int K, int C, long long pc, bool one_pass, int a2, int sms, int f
             prm.stages = stages > GEMM_MAX_STAGES ? GEMM_MAX_STAGES : stages;
         }
     }
+    if (!q8 && !forced && !prm.resident && shape.ctas == 1 && prm.num_k_tiles == 1 && gemm_streams_hbm(K, C, pc, a2))
+        prm.stages = std::min(prm.stages, streaming_stages(prm.num_c_blocks, prm.n_tile));
     // Epilogue staging: stmatrix into swizzled boxes where a CTA has several tiles (throughput: 3-8 % on those GEMMs),
     // plain 2-byte stores into one box where it has one (its two TMA stores of 128-byte rows drain later at the tail
     // of the launch: 0.5-1.5 us per layer of the SD v1.5 sweep).
@@ -2102,6 +2119,23 @@ int sdwino_selftest_input_passes(int N, int C, int H, int W, int K, size_t works
     for (long long p0 = 0; p0 < pl.P; p0 += pc, ++passes)
         *staged += use_input_tma(make_geom(H, W, pl.TH, pl.TW, pl.P), N, C, x, p0, std::min(pc, pl.P128 - p0));
     return passes;
+}
+
+int sdwino_selftest_gemm_shape(int N, int C, int H, int W, int K, int tile, size_t workspace_bytes, int* ctas, int* n_tile,
+                               int* blocks, int* stages) {
+    Plan pl;
+    if (!ctas || !n_tile || !blocks || !stages || !make_plan(N, C, H, W, K, tile, &pl)) return SDWINO_ERR_INVALID_ARG;
+    const long long pc = tiles_per_pass(pl, workspace_bytes);
+    if (pc < GEMM_BLOCK_P) return SDWINO_ERR_WORKSPACE;
+    GemmShape shape;
+    GemmParams prm;
+    constexpr int B200_SMS = 148;
+    if (!plan_gemm(K, C, pc, pc >= pl.P128, pl.a2, B200_SMS, 0, 0, false, &shape, &prm)) return SDWINO_ERR_UNSUPPORTED;
+    *ctas = shape.ctas;
+    *n_tile = shape.n_tile;
+    *blocks = shape.dual ? 2 : 1;
+    *stages = prm.stages;
+    return SDWINO_OK;
 }
 
 int sdwino_selftest_window_reads(int N, int C, int H, int W, int tile, int odd_start, long long* before, long long* after) {
