@@ -288,6 +288,7 @@ def alloc_workspace(nbytes: int, device="cuda") -> torch.Tensor:
     buf = torch.empty(nbytes, dtype=torch.uint8, device=device)
     if buf.data_ptr() % 1024 == 0:
         return buf
+    del buf                # given back first: two of them may not fit the device
     buf = torch.empty(nbytes + 1024, dtype=torch.uint8, device=device)
     off = (-buf.data_ptr()) % 1024
     return buf[off:off + nbytes]
