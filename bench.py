@@ -10,7 +10,7 @@ time is reported separately.
 
 By default all five workloads are measured (single layer, SD v1.5 UNet, SD VAE decoder, SD v2.1 UNet,
 SDXL at 1024x1024) and the headline `value` sits on the largest one, `sdxl_1024`; the others are in
-`workloads`.  Prints ONE JSON line (rank 0).  With --gpus N > 1 (under torchrun) every rank runs an
+`workloads`.  Prints ONE JSON line (rank 0); --detail FILE takes its rows per layer and kernel.  With --gpus N > 1 (under torchrun) every rank runs an
 independent replica of the sweep on its own GPU (the path has no exchange step); the time is the max
 over ranks.
 """
@@ -255,6 +255,22 @@ def host_inputs(layers):
 
 def headline_of(args) -> str:
     return HEADLINE if args.workload == "all" else args.workload
+
+
+def summary_line(line):
+    """The line that goes to stdout: what identifies the run and its figures, short enough to be kept whole in a log's tail.
+    The rows per layer and per workload go to the file that --detail names."""
+    out = {k: v for k, v in line.items() if k not in ("layers", "workloads", "transforms", "sustained", "cudnn_yardstick", "paper_context")}
+    out["config"] = {k: v for k, v in line["config"].items() if k not in ("tile_per_layer", "other_workloads_in_this_line")}
+    if out.get("cpu_baseline"):
+        out["cpu_baseline"] = {k: v for k, v in out["cpu_baseline"].items() if k != "sample"}
+    keep = ("kernel", "bound", "achieved", "peak", "unit", "frac", "traffic", "launches_per_step", "avg_launch_us", "share_of_step")
+    if out.get("roofline"):
+        out["roofline"] = {k: out["roofline"].get(k) for k in keep}
+    out["sustained"] = {k: line["sustained"][k] for k in ("value", "ms_per_step")} if line.get("sustained") else None
+    out["workloads"] = {n: {"value": w["value"], "ms_per_step": w["ms_per_step"], "e2e": (w["e2e"] or {}).get("value"),
+                            "cudnn": (w["cudnn_yardstick"] or {}).get("value")} for n, w in line["workloads"].items()}
+    return out
 
 
 def run_reference(args):
@@ -807,7 +823,10 @@ def run_ours(args):
             "kernel_source_hash": kernel_source_hash(),
             "paper_context": PAPER_CONTEXT,
         }
-        print(json.dumps(line), flush=True)
+        if args.detail:
+            with open(args.detail, "w") as f:
+                json.dump(line, f)
+        print(json.dumps(summary_line(line)), flush=True)
     if ctx.dist is not None:
         ctx.dist.destroy_process_group()
 
@@ -837,6 +856,7 @@ def main():
     ap.add_argument("--prefetch-mb", type=int, default=0,
                     help="with --sequence: MB of the next layer's filters prefetched into L2 per layer (0: none)")
     ap.add_argument("--no-graph", action="store_true", help="launch every step directly instead of replaying a CUDA graph")
+    ap.add_argument("--detail", default="", metavar="FILE", help="write the whole record, with its rows per layer and workload, to FILE")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-yardstick", action="store_true")
     ap.add_argument("--no-e2e", action="store_true", help="skip the host-buffer pass (profiling runs)")
