@@ -467,9 +467,9 @@ int launch_input(const XT* x, __half* V, const TileGeom& geo, int C, long long p
         bool edge = false;
         if constexpr (sizeof(XT) == 2) edge = x_cuts_words(reinterpret_cast<uintptr_t>(x), elems);
         e = edge ? launch_pdl(input_transform_any_kernel<M, XT, sizeof(XT) == 2>, grid, dim3(128), 0, st, 0, x, V, geo, C, p_begin,
-                              p_count, Pstride, amax, elems)
+                              p_count, Pstride, amax)
                  : launch_pdl(input_transform_any_kernel<M, XT>, grid, dim3(128), 0, st, 0, x, V, geo, C, p_begin, p_count, Pstride,
-                              amax, elems);
+                              amax);
     }
     g_launches.fetch_add(1);
     return e == cudaSuccess ? SDWINO_OK : err_cuda(__LINE__);
@@ -2078,6 +2078,7 @@ int sdwino_selftest_wait_timeout(unsigned long long limit_ns, void* stream) {
 }  // extern "C"
 
 namespace {
+// The loads of load_window (transforms_any.cuh), all windows of x
 template <int M>
 void window_reads(int N, int C, int H, int W, uintptr_t x, long long* before, long long* after) {
     constexpr int A = M + 2;
@@ -2088,17 +2089,17 @@ void window_reads(int N, int C, int H, int W, uintptr_t x, long long* before, lo
     for (long long img = 0; img < static_cast<long long>(N) * C; ++img)
         for (int i0 = -1; i0 < H; i0 += M)
             for (int j0 = -1; j0 < W; j0 += M) {
-                int lo, hi;
-                window_columns<A>(j0, W, lo, hi);
+                const int lo = j0 < 0 ? -j0 : 0, hi = W - j0 < A ? W - j0 : A;
                 for (int r = 0; r < A; ++r) {
                     if (i0 + r < 0 || i0 + r >= H) continue;
                     const uintptr_t a = x + static_cast<uintptr_t>((img * H + i0 + r) * W + j0) * 2;
                     for (int i = 0; i <= A / 2; ++i) {
-                        uintptr_t word;
-                        if (!window_word(a, i, lo, hi, &word)) continue;
-                        const int in = edge && (img % C == 0 || img % C == C - 1) ? word_pixels_in_x(word, x, x_hi) : 3;
-                        first = std::min(first, in & 1 ? word : word + 2);
-                        last = std::max(last, in & 2 ? word + 4 : word + 2);
+                        const int par = static_cast<int>((a >> 1) & 1);
+                        if (2 * i - par + 1 < lo || 2 * i - par >= hi) continue;
+                        const uintptr_t word = (a & ~uintptr_t(3)) + 4 * static_cast<uintptr_t>(i);
+                        const bool pixels = window_by_pixels(edge, static_cast<int>(img % C), C);
+                        first = std::min(first, pixels && 2 * i - par < lo ? word + 2 : word);
+                        last = std::max(last, pixels && 2 * i - par + 1 >= hi ? word + 2 : word + 4);
                     }
                 }
             }

@@ -43,51 +43,16 @@ __device__ __forceinline__ void at_packed(const float2 (&m)[M + 2], float2 (&o)[
     }
 }
 
-// Which bytes of the aligned 4-byte word at `word` lie in x, the bytes [x_lo, x_hi): bit 0 the lower pixel, bit 1 the upper
-// one.  Only the word of the first pixel of x (x at an odd pixel) or of its last one can have a pixel outside.
-__host__ __device__ __forceinline__ int word_pixels_in_x(uintptr_t word, uintptr_t x_lo, uintptr_t x_hi) {
-    return (word >= x_lo ? 1 : 0) | (word + 4 <= x_hi ? 2 : 0);
-}
-// Whether x begins or ends inside a word.
-inline bool x_cuts_words(uintptr_t x, long long elems) {
-    return (x & 3) != 0 || ((x + 2 * static_cast<uintptr_t>(elems)) & 3) != 0;
-}
-// The columns [lo, hi) of a window that lie inside the image; j0 is the image column of its column 0.
-template <int A>
-__host__ __device__ __forceinline__ void window_columns(int j0, int W, int& lo, int& hi) {
-    lo = j0 < 0 ? -j0 : 0;
-    hi = W - j0 < A ? W - j0 : A;
-}
-// Word i of a window row that begins at address `a` (its pixel 0) and has the pixels [lo, hi) inside the image: it holds the
-// pixels 2 i - par and 2 i - par + 1 and is loaded if one of them is inside.
-__host__ __device__ __forceinline__ bool window_word(uintptr_t a, int i, int lo, int hi, uintptr_t* word) {
-    const int par = static_cast<int>((a >> 1) & 1);
-    *word = (a & ~uintptr_t(3)) + 4 * static_cast<uintptr_t>(i);
-    return 2 * i - par + 1 >= lo && 2 * i - par < hi;
-}
-
-// Predicated, so that the loads of a window stay together (as branches they wait for one another).
-__device__ __forceinline__ void ld_nc_u32_if(uint32_t& v, const void* p, bool pred) {
-    asm("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q ld.global.nc.b32 %0, [%1];\n\t}"
-        : "+r"(v) : "l"(p), "r"(static_cast<int>(pred)));
-}
-
 // Window rows of one tile, all A of them: row r in h[r] as A / 2 words of two pixels, zeros outside the image.  Every
-// word that is loaded holds at least one pixel of the row (the other one may lie outside: it shares the aligned word).
-// EDGE: x begins or ends in the middle of a word, whose other half is not x's to read: that pixel is loaded alone.
-// (Tested on every word of the layer, 256 channels at 324x300, x odd, took 70 us instead of 46; only the first and last channel do, and go first.)
-// (Reading whole rows without the tests of window_word, masked afterwards, measured 5-8 % slower.)
-template <int M, bool EDGE>
+// word that is loaded holds at least one pixel of the row (the other one may lie outside: it shares the aligned word).  Only
+// the words of the first and of the last pixel of x can reach outside x, see load_window_pixels.
+// (Reading whole rows without these tests, masked afterwards, measured 5-8 % slower.)
+template <int M>
 __device__ __forceinline__ void load_window(const __half* __restrict__ img, const TileGeom& geo, int i0, int j0, bool valid,
-                                            uintptr_t x_lo, uintptr_t x_hi, uint32_t (&h)[M + 2][(M + 2) / 2]) {
+                                            uint32_t (&h)[M + 2][(M + 2) / 2]) {
     constexpr int A = M + 2;
-    int lo, hi;
-    window_columns<A>(j0, geo.W, lo, hi);
-    [[maybe_unused]] uint32_t first = 0u, last = 0u;      // the pixels that share a word with something else, in their places
-    if constexpr (EDGE) {
-        first = static_cast<uint32_t>(__ldg(reinterpret_cast<const unsigned short*>(x_lo))) << 16;
-        last = __ldg(reinterpret_cast<const unsigned short*>(x_hi) - 1);
-    }
+    const int lo = j0 < 0 ? -j0 : 0;
+    const int hi = geo.W - j0 < A ? geo.W - j0 : A;
     uint32_t mask[A / 2];
 #pragma unroll
     for (int i = 0; i < A / 2; ++i)
@@ -96,32 +61,52 @@ __device__ __forceinline__ void load_window(const __half* __restrict__ img, cons
     for (int r = 0; r < A; ++r) {
         const bool row_ok = valid && static_cast<unsigned>(i0 + r) < static_cast<unsigned>(geo.H);
         const uintptr_t a = reinterpret_cast<uintptr_t>(img) + (static_cast<long long>(i0 + r) * geo.W + j0) * 2;
+        const int par = static_cast<int>((a >> 1) & 1);
+        const uint32_t* wp = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
         uint32_t w[A / 2 + 1];
 #pragma unroll
         for (int i = 0; i <= A / 2; ++i) {
+            // word i holds the pixels 2 i - par and 2 i - par + 1 of the row
             w[i] = 0u;
-            uintptr_t word;
-            const bool want = window_word(a, i, lo, hi, &word) && row_ok;
-            if constexpr (EDGE) {
-                const int in = word_pixels_in_x(word, x_lo, x_hi);
-                if (want && in != 3) w[i] = in == 2 ? first : last;
-                ld_nc_u32_if(w[i], reinterpret_cast<const void*>(word), want && in == 3);
-            } else if (want) {
-                w[i] = __ldg(reinterpret_cast<const uint32_t*>(word));
-            }
+            if (row_ok && 2 * i - par + 1 >= lo && 2 * i - par < hi) w[i] = __ldg(wp + i);
         }
-        const uint32_t sel = (a >> 1) & 1 ? 0x5432u : 0x3210u;
+        const uint32_t sel = par ? 0x5432u : 0x3210u;
 #pragma unroll
         for (int i = 0; i < A / 2; ++i) h[r][i] = __byte_perm(w[i], w[i + 1], sel) & mask[i];
     }
 }
 
+// Whether x begins or ends in the middle of a word, whose other half is then not x's to read.
+inline bool x_cuts_words(uintptr_t x, long long elems) {
+    return (x & 3) != 0 || ((x + 2 * static_cast<uintptr_t>(elems)) & 3) != 0;
+}
+// The same rows pixel by pixel, for the channels whose words may reach outside x: the first and the last one of an x that
+// cuts words.  (Every word of such an x tested instead: 256 channels at 324x300 70 us, 46 without.)
+__host__ __device__ inline bool window_by_pixels(bool cuts, int c, int C) { return cuts && (c == 0 || c == C - 1); }
+template <int M>
+__device__ __forceinline__ void load_window_pixels(const __half* __restrict__ img, const TileGeom& geo, int i0, int j0, bool valid,
+                                                   uint32_t (&h)[M + 2][(M + 2) / 2]) {
+    const unsigned short* px = reinterpret_cast<const unsigned short*>(img);
+#pragma unroll
+    for (int r = 0; r < M + 2; ++r)
+#pragma unroll
+        for (int i = 0; i < (M + 2) / 2; ++i) {
+            uint32_t v[2] = {0u, 0u};
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                if (valid && static_cast<unsigned>(i0 + r) < static_cast<unsigned>(geo.H) &&
+                    static_cast<unsigned>(j0 + 2 * i + k) < static_cast<unsigned>(geo.W))
+                    v[k] = __ldg(px + static_cast<long long>(i0 + r) * geo.W + j0 + 2 * i + k);
+            h[r][i] = v[0] | (v[1] << 16);
+        }
+}
+
 // Activation preprocess of the pair (p, p + 1) for one channel; p - p_begin even.  Tiles past the last one are zeros.
-// x_elems: the elements of x (only used with EDGE, see load_window).
+// EDGE: x cuts words.
 template <int M, typename XT = __half, bool EDGE = false>
 __global__ void __launch_bounds__(128)
 input_transform_any_kernel(const XT* __restrict__ x, __half* __restrict__ V, TileGeom geo, int C, long long p_begin,
-                           int p_count, long long Pstride, const float* __restrict__ amax, long long x_elems) {
+                           int p_count, long long Pstride, const float* __restrict__ amax) {
     constexpr int A = M + 2;
     const int pl = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x) * 2;
     int c = static_cast<int>(blockIdx.z * gridDim.y + blockIdx.y);   // grid.z continues grid.y past 65535
@@ -150,13 +135,12 @@ input_transform_any_kernel(const XT* __restrict__ x, __half* __restrict__ V, Til
     float2 e2[A][A];   // rows transformed along the columns, (tile 0, tile 1)
     if constexpr (sizeof(XT) == 2) {
         uint32_t h0[A][A / 2], h1[A][A / 2];
-        const uintptr_t x_lo = reinterpret_cast<uintptr_t>(x), x_hi = x_lo + 2 * static_cast<uintptr_t>(x_elems);
-        if (EDGE && (c == 0 || c == C - 1)) {    // the first and the last pixel of x are in these channels
-            load_window<M, EDGE>(img[0], geo, i0[0], j0[0], valid[0], x_lo, x_hi, h0);
-            load_window<M, EDGE>(img[1], geo, i0[1], j0[1], valid[1], x_lo, x_hi, h1);
+        if (window_by_pixels(EDGE, c, C)) {
+            load_window_pixels<M>(img[0], geo, i0[0], j0[0], valid[0], h0);
+            load_window_pixels<M>(img[1], geo, i0[1], j0[1], valid[1], h1);
         } else {
-            load_window<M, false>(img[0], geo, i0[0], j0[0], valid[0], x_lo, x_hi, h0);
-            load_window<M, false>(img[1], geo, i0[1], j0[1], valid[1], x_lo, x_hi, h1);
+            load_window<M>(img[0], geo, i0[0], j0[0], valid[0], h0);
+            load_window<M>(img[1], geo, i0[1], j0[1], valid[1], h1);
         }
 #pragma unroll
         for (int r = 0; r < A; ++r) {

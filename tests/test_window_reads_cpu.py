@@ -1,5 +1,5 @@
 """The activation transforms of any width load x in aligned 4-byte words of two pixels.  No word may reach outside x: not
-where x begins at an odd pixel, not where it ends at one (the addresses are computed by the code the kernels run)."""
+where x begins at an odd pixel, not where it ends at one (the walk computes the addresses as the kernels do, with their rules for what may be loaded)."""
 import pytest
 
 
