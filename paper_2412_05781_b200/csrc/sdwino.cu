@@ -1438,8 +1438,10 @@ int launch_direct(const __half* x, const void* wT, const __half* bias, __half* y
     if (best.n_tile == 0) return SDWINO_ERR_UNSUPPORTED;
     DirectParams q;
     DirectWindow all{0, N, 0, pl.Ho, 0, pl.Wo}, step = all;
+    bool windows = false;
     if (!direct_geometry(pl, all, C, H, W, K, stride, best, &q)) return SDWINO_ERR_UNSUPPORTED;
     if (direct_packed_bytes(q) + direct_part_bytes(q) > ws_bytes) {
+        windows = true;
         if (!direct_window(pl, N, C, H, W, K, stride, best.splits, ws_bytes, &step)) return SDWINO_ERR_WORKSPACE;
         // a window has fewer tiles of pixels than the layer: as many channels per tile as are cheapest for it
         const int splits = best.splits;
@@ -1461,7 +1463,7 @@ int launch_direct(const __half* x, const void* wT, const __half* bias, __half* y
         for (int r0 = 0; r0 < pl.Ho; r0 += step.h)
             for (int c0 = 0; c0 < pl.Wo; c0 += step.w) {
                 DirectWindow win{n0, std::min(step.n, N - n0), r0, std::min(step.h, pl.Ho - r0), c0, std::min(step.w, pl.Wo - c0)};
-                if (!direct_geometry(pl, win, C, H, W, K, stride, best, &q)) return SDWINO_ERR_WORKSPACE;
+                if (windows && !direct_geometry(pl, win, C, H, W, K, stride, best, &q)) return SDWINO_ERR_WORKSPACE;
                 direct_finish(&q);
                 const long long first = n0 * K * hw_o + static_cast<long long>(r0) * pl.Wo + c0;
                 q.wt_header = wt_header_of(wT);
