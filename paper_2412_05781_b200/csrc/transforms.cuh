@@ -626,12 +626,12 @@ input_transform_vec_kernel(const XT* __restrict__ x, __half* __restrict__ V, Til
 // permutes.  The kernel is bound by instruction issue, so this is where its time goes: 3-10 % per layer over
 // the generic vector kernel.  CH = 1 is what runs: with 2 or 4 channels per thread the per-thread set-up is
 // amortised, but the serial load -> compute chain per channel and the lower thread count cost more (measured).
-// EARLY (fp16 input): all six row segments of a channel are loaded before the first one is used, so that a thread
+// fp16 input: all six row segments of a channel are loaded before the first one is used, so that a thread
 // pays one memory latency per channel instead of several, also with 20 warps per SM: 320 channels at 96x96, batch 4,
 // 19.2 -> 13.9 us (77 MB: 4.0 -> 5.5 TB/s), 960 channels 64 -> 44, 1920 channels at 48x48 36 -> 25.6.  (With four CTAs per
 // SM instead of five 14.5, 47 and 28.7.)  fp32 input, three rows at a time: 640 channels at 64x64, batch 2, 9.4 -> 8.0 us,
 // 320 at 96x96, batch 4, 23.5 -> 18.6.
-template <int CH, typename XT = __half, bool PDL = true, bool EARLY = false>
+template <int CH, typename XT = __half, bool PDL = true>
 __device__ __forceinline__ void input_unit_f4(const XT* __restrict__ x, __half* __restrict__ V, const TileGeom& geo,
                                               int C, long long p_begin, const FastDiv& gdiv, long long Pstride,
                                               uint32_t idx, const float* __restrict__ amax = nullptr) {
@@ -676,7 +676,7 @@ __device__ __forceinline__ void input_unit_f4(const XT* __restrict__ x, __half* 
         [[maybe_unused]] float fl[3], fr[3];
         [[maybe_unused]] uint4 raw_v[A];
         [[maybe_unused]] uint32_t raw_l[A], raw_r[A];
-        if constexpr (EARLY && sizeof(XT) == 2) {
+        if constexpr (sizeof(XT) == 2) {
 #pragma unroll
             for (int r = 0; r < A; ++r) {
                 raw_v[r] = make_uint4(0u, 0u, 0u, 0u);
@@ -718,16 +718,8 @@ __device__ __forceinline__ void input_unit_f4(const XT* __restrict__ x, __half* 
                 d[4] = make_float2(a.w * xs, b.w * xs);
                 d[5] = make_float2(b.x * xs, R * xs);
             } else {
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            uint32_t lw = 0u, rw = 0u;   // aligned words before / after the segment
-            if constexpr (EARLY) {
-                v = raw_v[r]; lw = raw_l[r]; rw = raw_r[r];
-            } else if ((rowmask >> r) & 1) {
-                const __half* rp = xp + r * geo.W;
-                v = __ldg(reinterpret_cast<const uint4*>(rp));
-                if (left_ok) lw = __ldg(reinterpret_cast<const uint32_t*>(rp - 2));
-                if (right_ok) rw = __ldg(reinterpret_cast<const uint32_t*>(rp + 8));
-            }
+            const uint4 v = raw_v[r];
+            const uint32_t lw = raw_l[r], rw = raw_r[r];   // aligned words before / after the segment
             // pixels: L = lw.hi, px0..px7 = v.x.lo, v.x.hi, ..., v.w.hi, R = rw.lo; tile 0 uses L..px4, tile 1 px3..R
             uint32_t h[A];
             h[0] = __byte_perm(lw, v.y, 0x7632);    // (L,   px3)
@@ -760,7 +752,7 @@ template <int CH, typename XT = __half>
 __global__ void __launch_bounds__(128, 5)
 input_transform_f4_kernel(const XT* __restrict__ x, __half* __restrict__ V, TileGeom geo, int C, long long p_begin,
                           FastDiv gdiv, long long Pstride, const float* __restrict__ amax) {
-    input_unit_f4<CH, XT, true, true>(x, V, geo, C, p_begin, gdiv, Pstride, blockIdx.x * blockDim.x + threadIdx.x, amax);   // < 2^31
+    input_unit_f4<CH, XT>(x, V, geo, C, p_begin, gdiv, Pstride, blockIdx.x * blockDim.x + threadIdx.x, amax);   // < 2^31
 }
 
 // Eight output pixels of one row (bias already added): residual (its eight values loaded by the caller, ahead of

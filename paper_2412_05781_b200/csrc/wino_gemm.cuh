@@ -78,11 +78,8 @@ struct GemmSmemLayout {
     __host__ __device__ static constexpr int stage_bytes(int rows) {
         return (A_BYTES + b_bytes(rows) + 1023) / 1024 * 1024;
     }
-    // 8-bit filters: a stage also holds the raw bytes of its filter box (64 per row) next to their fp16 expansion
+    // 8-bit filters: a slot of the raw ring, the bytes of a filter box (64 per row)
     __host__ __device__ static constexpr int raw_bytes(int rows) { return rows * GEMM_BLOCK_C; }
-    __host__ __device__ static constexpr int stage_bytes_u8(int rows) {
-        return (A_BYTES + b_bytes(rows) + raw_bytes(rows) + 1023) / 1024 * 1024;
-    }
     // epilogue staging: `bufs` buffers of [epi_rows k][128 p] fp16
     __host__ __device__ static constexpr int epi_bytes(int epi_rows, int bufs) {
         return bufs * epi_rows * EPI_ROW_BYTES;
@@ -1056,7 +1053,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
             if (kind == 0) {
                 const int c_end = (sub + 1) * pp.cg < prm.C ? (sub + 1) * pp.cg : prm.C;
                 for (int c = sub * pp.cg + (tt >> 6); c < c_end; c += PIPE_TRANSFORM_THREADS / 64)
-                    input_unit_f4<1, __half, false, true>(pp.x, pp.V + slot_off, pp.geo, prm.C, p_begin, pp.fd64, ring_p,
+                    input_unit_f4<1, __half, false>(pp.x, pp.V + slot_off, pp.geo, prm.C, p_begin, pp.fd64, ring_p,
                                                           static_cast<uint32_t>(c) * 64u + pair);
             } else {
                 const int k_end = (sub + 1) * pp.kg < prm.K ? (sub + 1) * pp.kg : prm.K;
