@@ -65,7 +65,7 @@ __device__ __forceinline__ bool mbar_try_wait_a32(uint32_t bar, uint32_t parity)
 }
 // Slow path of the bounded wait: polls, and every 4096 failed polls looks at the abort flag and at
 // the (slow to read) global timer.  Kept out of line so that the hot path stays a handful of
-// instructions: the waiting roles are single threads, whose instruction latency is the pipeline's.
+// instructions: a waiting role is one warp, whose instruction latency is the pipeline's.
 __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                             uint64_t limit_ns) {
     uint32_t polls = 0;

@@ -656,7 +656,7 @@ cudaError_t launch_output_any(const __half* Mws, const YT* bias, YT* y, const Ti
     const int sms = sm_count();
     if (sms <= 0) return cudaErrorInvalidDevice;
     const unsigned blocks = static_cast<unsigned>((p_count / 2 + OUT_ANY_THREADS - 1) / OUT_ANY_THREADS);
-    // channels per CTA (the tiles are decoded once): as many as leave several waves of the six CTAs that fit an SM
+    // channels per CTA (the tiles are decoded once): as many as leave 24 CTAs per SM, about five waves of the five that fit
     const long long steps = std::max(1ll, std::min(4ll, static_cast<long long>(blocks) * K / (24ll * sms)));
     const dim3 grid = grid_rows(blocks, (K + steps - 1) / steps);
     if (ep.residual != nullptr || ep.act != 0)
@@ -1691,8 +1691,9 @@ int sdwino_choose_algorithm(int N, int C, int H, int W, int K) {
     if (N <= 0 || C <= 0 || H <= 0 || W <= 0 || K <= 0) return 0;
     // Layers whose whole batch is at most one block of 128 output pixels (the 8x8 layers of the UNet at batch 2):
     // F(2x2) would fill a quarter of its block of 128 tiles and stream 16 values per weight, the direct form fills
-    // its block and streams 9.  Measured: 1280->1280 at 8x8, batch 2: 22.5 against 26.6 us, 2560->1280: 32.8 against
-    // 36.9 us; from two blocks of pixels on (12x12, 16x16) the direct form re-reads the filters per block and loses.
+    // its block and streams 9.  Measured (filters from HBM): 1280->1280 at 64 pixels 13.5 against 17.4 us with F(2x2), at
+    // 128 14.4 / 17.5, 2560->1280 at 128 20.8 / 26.3, 320->320 7.7 / 8.0; from two blocks of pixels on it re-reads the filters
+    // per block: at 256 pixels 17.3 / 17.4, 25.5 / 26.4, 8.7 / 7.9, at 512, as one implicit GEMM, 21.8 / 17.8, 30.8 / 26.6, 9.7 / 8.1.
     if (C > 8 && K > 8 && static_cast<long long>(N) * H * W <= GEMM_BLOCK_P) return 1;
     return sdwino_choose_tile(N, C, H, W, K);
 }

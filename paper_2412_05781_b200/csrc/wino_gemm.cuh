@@ -34,14 +34,17 @@
 // (batch 2) 51.3 -> 50.1.
 //
 // One persistent CTA (pair) per SM (pair) walks the list of (pos, k-tile, p-tile) output tiles.
-//   warp 0   : TMA producer        (one lane)
-//   warp 1   : TMEM owner + MMA issuer (one lane)
+// Warps 0 and 1, and the producers after warp 9, run their roles as whole warps of which one elected lane issues.
+//   warp 0   : TMA producer (V; the filters too for CTA pairs and in the filter-resident and pipelined modes)
+//   warp 1   : TMEM owner + MMA issuer
 //   warps 2-9: epilogue in two groups of four warps (one TMEM lane quarter per warp); group g drains
-//              channels [g * epi_rows, (g + 1) * epi_rows) of the tile; TMEM accumulators are double-buffered so
-//              the epilogue of tile i overlaps the MMAs of tile i+1.  A thread owns one tile p and
+//              channels [g * epi_rows, (g + 1) * epi_rows) of the tile; two accumulators in TMEM (up to four with two
+//              blocks of tiles) let the epilogue of tile i overlap the MMAs of tile i+1.  A thread owns one tile p and
 //              reads its channels from TMEM; the fp16 results are transposed through a shared-memory
 //              staging buffer [k][128 p] and leave with one TMA store per epi_rows channels, so M is
 //              written in full 256-byte rows.
+//   then     : streaming single CTAs: warp 10 produces the filter boxes; 8-bit filters: warps 10-17 expand the filter
+//              bytes and warp 18 produces them; pipelined mode: warps 10-19 run the transforms.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -120,8 +123,8 @@ struct GemmParams {
     const float* scales; // 8-bit filters: S[pos][kpad], the factor of every (position, output channel) row
     int kpad;            // Kb * 16
     int raw_slots;       // 8-bit filters: slots of the raw ring (at most GEMM_MAX_STAGES)
-    FastDiv fd_p, fd_k, fd_keys;   // divisions by num_p_tiles, num_k_tiles, num_k_tiles * num_pos (the roles are single
-                                   // threads: a hardware-less integer division is a few hundred cycles of their time)
+    FastDiv fd_p, fd_k, fd_keys;   // divisions by num_p_tiles, num_k_tiles, num_k_tiles * num_pos (a role is one warp: an
+                                   // integer division without hardware is a few hundred cycles of its time)
 };
 
 // Pipelined mode (template flag PIPE): the three steps of a layer run inside ONE persistent launch.  V and M are rings
@@ -415,7 +418,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
         } else if (!resident) {
             // the full barrier of a pair lives in the leader and counts the bytes of both CTAs
             const uint32_t tx_bytes = CTAS * (a_bytes + L::b_bytes(b_rows));
-            // single-thread loop: shared-memory and barrier addresses are running 32-bit values
+            // shared-memory and barrier addresses are running 32-bit values
             const uint32_t smem_base = smem_u32(smem);
             const uint32_t full0_local = smem_u32(&full_bar[0]);
             const uint32_t full0 = CTAS == 2 ? map_to_cta(full0_local, 0) : full0_local;
@@ -549,7 +552,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
         // back-to-back MMAs 86 cycles each; as it stands 80 at N = 160, the tensor rate).
         if (leader) {
             const uint32_t idesc = make_idesc_f16_f32(GEMM_BLOCK_P * CTAS, prm.n_tile, true, false);
-            // This loop is executed by ONE thread, so every instruction in it costs its full latency: the
+            // One warp runs this loop with nothing to overlap it, so every instruction in it costs its full latency: the
             // descriptors of stage 0 are built once and then only advanced by additions (the 14-bit
             // address field cannot overflow inside 227 KB of shared memory).
             //   A (M-major): 16 channels = 16 rows of 128 bytes = +2048 bytes; the two 64-wide p blocks are
@@ -875,7 +878,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
         }
     } else if constexpr (SPLIT && !U8) {
         // ------------------------------ second producer: the filter boxes ------------------------------
-        // The filters depend on nothing before this launch (see the comment in the first producer), so this thread
+        // The filters depend on nothing before this launch (see the comment in the first producer), so this warp
         // never waits for the preceding kernel: the first ring-full of boxes goes out at once, the rest as stages
         // are released.
         {

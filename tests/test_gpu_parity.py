@@ -389,7 +389,7 @@ def _random_shapes(count, seed):
 
 @pytest.mark.parametrize("shape", _random_shapes(24, seed=2412))
 def test_seeded_random_shapes_both_tiles(B, shape):
-    # a seeded draw over channel counts (few / ragged / several blocks), odd and even sizes, scalar and vector
+    # a seeded draw over channel counts (few / ragged / several blocks), odd and even sizes, any-width and vector
     # transform paths, small batches: every path of the dispatcher must agree with the oracle
     C, K, H, W, N = shape
     layer = ConvLayer(C=C, K=K, H=H, W=W, N=N)
@@ -601,7 +601,7 @@ def test_async_host_entry_with_layers_of_different_sizes(B, shared):
                                         ((20, 24, 9, 11, 1), 4), ((4, 40, 12, 16, 1), 2), ((40, 4, 12, 16, 2), 2),
                                         ((64, 64, 64, 64, 1), 4), ((17, 33, 13, 24, 3), 4)])
 def test_fused_residual_and_activation(B, shape, tile, act):
-    # y = act(conv + bias + residual) in the output transform: vector and scalar kernels, both tiles, layers that
+    # y = act(conv + bias + residual) in the output transform: vector and any-width kernels, both tiles, layers that
     # would otherwise take a single-kernel path, the residual aliasing y
     C, K, H, W, N = shape
     layer = ConvLayer(C=C, K=K, H=H, W=W, N=N)

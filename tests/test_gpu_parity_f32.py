@@ -45,7 +45,7 @@ def _rel_err(y, ref):
 
 
 SHAPES = [
-    # C, K, H, W, N: scalar kernels (odd widths), vector kernels (W % 8 == 0), few channels, ragged everything
+    # C, K, H, W, N: any-width kernels (odd widths), vector kernels (W % 8 == 0), few channels, ragged everything
     (1, 1, 4, 4, 1), (3, 4, 5, 7, 2), (7, 33, 2, 9, 1), (33, 3, 13, 1, 2), (4, 40, 16, 16, 1), (40, 4, 24, 32, 2),
     (64, 128, 16, 16, 1), (65, 129, 17, 19, 1), (96, 160, 18, 24, 2), (130, 257, 33, 40, 1), (16, 16, 40, 56, 3),
     (72, 200, 50, 48, 2),
@@ -163,7 +163,7 @@ def test_fp32_interface_argument_errors(B):
     assert lib.sdwino_filter_transform_f32(None, wT.data_ptr(), 16, 16, 2, None) == B.ERR_INVALID_ARG
     assert lib.sdwino_filter_transform_f32(w.cuda().data_ptr(), wT.data_ptr(), 16, 16, 6, None) == B.ERR_UNSUPPORTED
     torch.cuda.synchronize()
-    # a 4-byte aligned but not 16-byte aligned x takes the scalar kernel: same result
+    # a 4-byte aligned but not 16-byte aligned x takes the any-width kernel: same result
     buf = torch.empty(x.numel() + 1, device="cuda")
     buf[1:].copy_(xd.flatten())
     y2 = torch.empty_like(y)
@@ -244,7 +244,7 @@ def test_fp32_interface_few_input_channels_fused_kernel(B, shape):
         B.sdwino_set_gemm_shape(0, 0)
     assert _rel_err(y3[:, ks], ref) <= TOL_F2_REGRESSION
     assert float((y - y3).abs().max()) <= 2 * TOL_F2_REGRESSION * float(np.abs(ref).max())
-    # y 4-byte aligned only: the scalar stores
+    # y 4-byte aligned only: the any-width kernel
     buf = torch.empty(N * K * H * W + 1, device="cuda")
     yv = buf[1:].view(N, K, H, W)
     wT = B.sdwino_filter_transform_f32(w.cuda(), 2)
@@ -261,7 +261,7 @@ def test_fp32_interface_few_input_channels_fused_kernel(B, shape):
                                         ((20, 24, 9, 11, 1), 4), ((4, 40, 12, 16, 1), 2), ((40, 4, 12, 16, 2), 2),
                                         ((64, 64, 64, 64, 1), 4), ((17, 33, 13, 24, 3), 4)])
 def test_fp32_interface_fused_residual_and_activation(B, shape, tile, act):
-    # y = act(conv + bias + residual), all fp32: vector, scalar and TMA-staged output kernels, both tiles, layers that
+    # y = act(conv + bias + residual), all fp32: vector, any-width and TMA-staged output kernels, both tiles, layers that
     # would otherwise take a single-kernel path, the residual aliasing y
     C, K, H, W, N = shape
     layer = ConvLayer(C=C, K=K, H=H, W=W, N=N)

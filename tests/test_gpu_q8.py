@@ -66,7 +66,7 @@ def test_quantised_filter_matches_oracle(B, KC, tile):
 
 SHAPES = [
     # C, K, H, W, N
-    (64, 96, 16, 16, 1), (72, 200, 18, 22, 2), (130, 257, 9, 11, 1), (16, 24, 40, 56, 2),   # ragged, scalar and vector kernels
+    (64, 96, 16, 16, 1), (72, 200, 18, 22, 2), (130, 257, 9, 11, 1), (16, 24, 40, 56, 2),   # ragged, any-width and vector kernels
     (1280, 1280, 16, 16, 2), (2560, 1280, 8, 8, 2),                                          # weight streaming: one tile per CTA
     (320, 320, 64, 64, 2),                                                                   # several tiles per CTA
     (4, 40, 12, 12, 1), (40, 4, 24, 32, 1),                                                  # few channels: the GEMM path all the same
