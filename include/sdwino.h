@@ -197,6 +197,9 @@ int sdwino_conv3x3_q8(const void *x, const void *wTq, const void *bias, void *y,
  *   sdwino_conv3x3_ws.
  */
 size_t sdwino_workspace_bytes_direct(int N, int C, int H, int W, int K, int stride);
+/* Host-only query for tests: the shape of the single GEMM on 148 SMs (flat: pixels in the order of the padded image, else a
+ * grid of 16 x 8; output channels per tile; parts of the input channels), or SDWINO_ERR_UNSUPPORTED for the three steps. */
+int sdwino_selftest_direct_shape(int N, int C, int H, int W, int K, int stride, int *flat, int *n_tile, int *splits);
 int sdwino_conv3x3_direct(const void *x, const void *wT, const void *bias, void *y,
                           int N, int C, int H, int W, int K, int stride,
                           void *workspace, size_t workspace_bytes, void *stream);

@@ -28,7 +28,7 @@ EXPORTS = [
     "sdwino_conv3x3_f32_scaled", "sdwino_filter_q8_bytes", "sdwino_filter_quantize", "sdwino_conv3x3_q8",
     "sdwino_workspace_bytes_direct", "sdwino_conv3x3_direct", "sdwino_choose_algorithm",
     "sdwino_workspace_bytes_sequence", "sdwino_conv3x3_sequence", "sdwino_selftest_window_reads",
-    "sdwino_selftest_input_passes", "sdwino_selftest_gemm_shape",
+    "sdwino_selftest_input_passes", "sdwino_selftest_gemm_shape", "sdwino_selftest_direct_shape",
 ]
 
 class SdwinoLayer(ctypes.Structure):
@@ -106,6 +106,8 @@ def _load() -> ctypes.CDLL:
     lib.sdwino_selftest_input_passes.argtypes = [i, i, i, i, i, sz, ctypes.POINTER(i)]
     lib.sdwino_selftest_gemm_shape.restype = i
     lib.sdwino_selftest_gemm_shape.argtypes = [i] * 6 + [sz] + [ctypes.POINTER(i)] * 4
+    lib.sdwino_selftest_direct_shape.restype = i
+    lib.sdwino_selftest_direct_shape.argtypes = [i] * 6 + [ctypes.POINTER(i)] * 3
     lib.sdwino_selftest_window_reads.restype = i
     lib.sdwino_selftest_window_reads.argtypes = [i, i, i, i, i, i, ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(ctypes.c_longlong)]
     lib.sdwino_choose_tile.restype = i
@@ -209,6 +211,16 @@ def sdwino_selftest_gemm_shape(N: int, C: int, H: int, W: int, K: int, tile: int
     """-> (CTAs per tile, output channels per tile, blocks of 128 tiles per CTA tile, ring stages); see include/sdwino.h."""
     out = [ctypes.c_int(0) for _ in range(4)]
     _check(lib.sdwino_selftest_gemm_shape(N, C, H, W, K, tile, workspace_bytes, *out), "sdwino_selftest_gemm_shape")
+    return tuple(v.value for v in out)
+
+
+def sdwino_selftest_direct_shape(N: int, C: int, H: int, W: int, K: int, stride: int):
+    """-> (flat, output channels per tile, channel parts) of the direct convolution's single GEMM; None for the three steps."""
+    out = [ctypes.c_int(0) for _ in range(3)]
+    rc = lib.sdwino_selftest_direct_shape(N, C, H, W, K, stride, *out)
+    if rc == ERR_UNSUPPORTED:
+        return None
+    _check(rc, "sdwino_selftest_direct_shape")
     return tuple(v.value for v in out)
 
 

@@ -99,6 +99,7 @@ constexpr int MAX_DYN_SMEM = 232448;  // 227 KB opt-in limit per CTA on sm_100
 constexpr size_t PASS_BUDGET = 4096ull << 20;
 constexpr size_t WS_ALIGN = 1024;
 constexpr size_t L2_BYTES = 126ull << 20;
+constexpr int B200_SMS = 148;            // for the host-only queries; launches ask the device
 constexpr int STATIC_MAX_DEVICES_HOST = 64;
 
 // SDWINO_ERR_CUDA, with the place and the runtime's last error on stderr when SDWINO_LOG is set
@@ -2133,13 +2134,23 @@ int sdwino_selftest_gemm_shape(int N, int C, int H, int W, int K, int tile, size
     if (pc < GEMM_BLOCK_P) return SDWINO_ERR_WORKSPACE;
     GemmShape shape;
     GemmParams prm;
-    constexpr int B200_SMS = 148;
     if (!plan_gemm(K, C, pc, pc >= pl.P128, pl.a2, B200_SMS, 0, 0, false, &shape, &prm)) return SDWINO_ERR_UNSUPPORTED;
     *ctas = shape.ctas;
     *n_tile = shape.n_tile;
     *blocks = shape.dual ? 2 : 1;
     *stages = prm.stages;
     return SDWINO_OK;
+}
+
+int sdwino_selftest_direct_shape(int N, int C, int H, int W, int K, int stride, int* flat, int* n_tile, int* splits) {
+    Plan pl;
+    if (!flat || !n_tile || !splits || stride < 1 || !make_plan(N, C, H, W, K, 1, &pl, stride)) return SDWINO_ERR_INVALID_ARG;
+    if (!use_direct_conv(pl, N, C, stride)) return SDWINO_ERR_UNSUPPORTED;
+    const DirectShape sh = choose_direct_shape(pl, N, C, H, W, K, stride, B200_SMS);
+    *flat = sh.flat;
+    *n_tile = sh.n_tile;
+    *splits = sh.splits;
+    return sh.n_tile ? SDWINO_OK : SDWINO_ERR_UNSUPPORTED;
 }
 
 int sdwino_selftest_window_reads(int N, int C, int H, int W, int tile, int odd_start, long long* before, long long* after) {

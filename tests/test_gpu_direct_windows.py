@@ -32,12 +32,17 @@ def _kinds(B, call):
         B.sdwino_profile_enable(0)
 
 
-@pytest.mark.parametrize("shape", [
+# (layouts, channel ranges and wide tiles: test_direct_shape_cpu.py checks that the model still picks each for one of them)
+WINDOW_SHAPES = [
     # stride, C, K, H, W, N: one image or many, odd sizes, channels that end inside a block, split channel ranges
     (1, 64, 64, 16, 16, 2), (1, 72, 200, 30, 26, 2), (1, 640, 136, 16, 16, 2), (1, 33, 300, 17, 40, 1), (1, 40, 17, 600, 1, 1),
     (1, 64, 16, 1, 1, 512), (1, 32, 9, 1, 600, 1), (1, 32, 1, 23, 24, 1), (1, 1280, 1280, 8, 8, 8),
     (2, 48, 56, 48, 55, 2), (2, 33, 1, 64, 64, 1), (2, 320, 328, 16, 16, 10), (2, 40, 24, 5, 900, 1), (2, 1280, 48, 50, 51, 1),
-])
+    (1, 32, 320, 23, 56, 5), (1, 200, 160, 66, 41, 5), (1, 100, 16, 15, 37, 1), (2, 32, 100, 10, 66, 5), (2, 100, 16, 27, 45, 2),
+]
+
+
+@pytest.mark.parametrize("shape", WINDOW_SHAPES)
 def test_the_workspace_does_not_change_the_bits(B, shape):
     stride, C, K, H, W, N = shape
     x, w, b = workloads.make_inputs(ConvLayer(C=C, K=K, H=H, W=W, N=N), seed=sum(shape))
@@ -47,7 +52,7 @@ def test_the_workspace_does_not_change_the_bits(B, shape):
     least = 128 * 9 * (C + K) * 2
     n, pad = ref.size, 64
     first = None
-    launches = []
+    launches, parts_in_turn = [], False
     for size in sorted({full, full // 2, full // 3, full // 7, 3 * least, least + 1024, least}, reverse=True):
         if size < least:
             continue
@@ -65,10 +70,14 @@ def test_the_workspace_does_not_change_the_bits(B, shape):
             assert np.abs(y.cpu().double().numpy() - ref).max() <= 1e-3 * np.abs(ref).max()
         assert torch.equal(first, y), size
         launches.append(len(kinds))
+        # one packed input, but the parts of the channel ranges of some tiles at a time
+        parts_in_turn |= kinds.count("input_transform") == 1 and kinds.count("output_transform") > 1
     # the smallest workspace does take several windows, unless the layer's packed input fits it
     positions = N * ((H - 1) // stride + 2) * ((W - 1) // stride + 2)
     if positions * (4 if stride == 2 else 1) * -(-C // 64) * 128 > least:
         assert launches[-1] >= 4
+    if shape in ((1, 640, 136, 16, 16, 2), (1, 1280, 1280, 8, 8, 8)):
+        assert parts_in_turn
 
 
 def test_residual_and_activation_window_by_window(B):
