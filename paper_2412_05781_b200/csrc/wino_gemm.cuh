@@ -34,7 +34,8 @@
 // (batch 2) 51.3 -> 50.1.
 //
 // One persistent CTA (pair) per SM (pair) walks the list of (pos, k-tile, p-tile) output tiles.
-// Warps 0 and 1, and the producers after warp 9, run their roles as whole warps of which one elected lane issues.
+// Warps 0 and 1, and the producers after warp 9, run their roles as whole warps of which one elected lane issues (in the
+// pipelined mode that lane alone runs them).
 //   warp 0   : TMA producer (V; the filters too for CTA pairs and in the filter-resident and pipelined modes)
 //   warp 1   : TMEM owner + MMA issuer
 //   warps 2-9: epilogue in two groups of four warps (one TMEM lane quarter per warp); group g drains
@@ -209,6 +210,18 @@ __device__ __forceinline__ void signal_counter_release(unsigned int* ctr) {
 // STM: the epilogue stages M through stmatrix into two swizzled boxes of 64 tiles (launches whose CTAs have several
 // tiles); without it, through 2-byte stores into one plain box of 128 tiles (one tile per CTA, 8-bit filters).  A
 // template flag like the others: with both forms in one kernel either was 1-3 % slower.
+// The waits of the producer and MMA roles: a whole warp, or (PIPE) its elected lane alone, beside which the transform warps
+// need the issue slots: 512->512 at 256x256 242 us with whole warps, 216 with one lane each, 256->256 at 512x512 451 / 425.
+template <bool PIPE>
+__device__ __forceinline__ bool wait_role(uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint64_t limit_ns) {
+    if constexpr (PIPE) return mbar_wait_bounded(bar, parity, abort_flag, limit_ns);
+    else return mbar_wait_warp(bar, parity, abort_flag, limit_ns);
+}
+template <bool PIPE>
+__device__ __forceinline__ bool wait_role_a32(uint32_t bar_a, uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint64_t limit_ns) {
+    if constexpr (PIPE) return mbar_try_wait_a32(bar_a, parity) || mbar_wait_slow(bar, parity, abort_flag, limit_ns);
+    else return mbar_wait_warp_a32(bar_a, bar, parity, abort_flag, limit_ns);
+}
 template <int CTAS, bool RES = false, bool DUAL = false, bool PIPE = false, bool U8 = false, bool STM = true>
 __global__ void __launch_bounds__(PIPE ? PIPE_THREADS : (U8 ? GEMM_U8_THREADS : GEMM_LAUNCH_THREADS), 1)
 wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmV,
@@ -346,7 +359,8 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
         if (threadIdx.x == 0) atomicCAS(status_word, 0, 1 | (9 << 8));   // 1 = SDWINO_ERR_INVALID_ARG
     } else if (warp == 0) {
         // ------------------------------ TMA producer ------------------------------
-        if (resident) {
+        if (PIPE && !elected) {
+        } else if (resident) {
             // filter-resident mode: the filter block of a (position, k-tile) is loaded once, V streams through the ring
             const uint32_t smem_base = smem_u32(smem);
             const uint32_t ures_a = smem_u32(ures_base);
@@ -379,7 +393,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                 decode(tile_of(i), pt, kt, pos);
                 if (pos * prm.num_k_tiles + kt != cur_key) {
                     // the MMAs of the previous run of tiles have finished reading the resident block
-                    ok = mbar_wait_warp(ures_empty_bar, reloads & 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                    ok = wait_role<PIPE>(ures_empty_bar, reloads & 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                     if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 5, cta_rank); break; }
                     ++reloads;
                     load_filters(pos, kt);
@@ -390,7 +404,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                     // V of this block of tiles is written by the transform warps of this launch.  The counter was read
                     // one tile ahead (the read is a round trip to L2 on this one thread's critical path).
                     if (seen_pt != pt || seen < static_cast<unsigned int>(pp.it_items)) {
-                        ok = __all_sync(0xffffffffu, wait_counter(&pp.v_ready[pt], static_cast<unsigned int>(pp.it_items), pp.abort_word, GEMM_WAIT_LIMIT_NS)) != 0;
+                        ok = wait_counter(&pp.v_ready[pt], static_cast<unsigned int>(pp.it_items), pp.abort_word, GEMM_WAIT_LIMIT_NS);
                         if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 12, cta_rank); break; }
                     }
                     fence_proxy_async_all();
@@ -402,7 +416,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                     }
                 }
                 for (int c0 = 0; c0 < prm.C; c0 += GEMM_BLOCK_C) {
-                    ok = mbar_wait_warp(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                    ok = wait_role<PIPE>(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                     if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 1, cta_rank); break; }
                     if (elected) {
                         mbar_arrive_expect_tx_a32(fb, L::A_BYTES);
@@ -442,7 +456,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                     decode(tile_of(i), pt, kt, pos);
                     const int p0 = pt * PT * GEMM_BLOCK_P;
                     for (int c0 = 0; c0 < prm.C; c0 += GEMM_BLOCK_C) {
-                        ok = mbar_wait_warp(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                        ok = wait_role<PIPE>(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                         if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 1, cta_rank); break; }
                         if (elected) {
                             mbar_arrive_expect_tx_a32(fb, static_cast<uint32_t>(a_bytes));
@@ -491,7 +505,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                     // V of this block of tiles is written by the transform warps of this launch (counter read one
                     // tile ahead, as in the filter-resident producer)
                     if (seen_pt != pt || seen < static_cast<unsigned int>(pp.it_items)) {
-                        ok = __all_sync(0xffffffffu, wait_counter(&pp.v_ready[pt], static_cast<unsigned int>(pp.it_items), pp.abort_word, GEMM_WAIT_LIMIT_NS)) != 0;
+                        ok = wait_counter(&pp.v_ready[pt], static_cast<unsigned int>(pp.it_items), pp.abort_word, GEMM_WAIT_LIMIT_NS);
                         if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 12, cta_rank); break; }
                     }
                     fence_proxy_async_all();
@@ -518,7 +532,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                         if (++stage == stages) { stage = 0; phase ^= 1u; sa = smem_base; fb = full0; fb_local = full0_local; }
                         continue;
                     }
-                    ok = mbar_wait_warp(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                    ok = wait_role<PIPE>(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                     if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 1, cta_rank); break; }
                     if (!elected) {
                     } else if constexpr (CTAS == 2) {
@@ -550,7 +564,7 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
         // descriptors pass through vector registers: an MMA then costs 52 cycles of issue and a wait on a barrier that
         // has already completed about 270, i.e. 480 per stage against the 320 of its MMAs at n_tile 160 (in a loop of
         // back-to-back MMAs 86 cycles each; as it stands 80 at N = 160, the tensor rate).
-        if (leader) {
+        if (leader && (!PIPE || elected)) {
             const uint32_t idesc = make_idesc_f16_f32(GEMM_BLOCK_P * CTAS, prm.n_tile, true, false);
             // One warp runs this loop with nothing to overlap it, so every instruction in it costs its full latency: the
             // descriptors of stage 0 are built once and then only advanced by additions (the 14-bit
@@ -581,17 +595,17 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                 if (resident) {
                     key = static_cast<int>(fast_div(static_cast<uint32_t>(tile), prm.fd_p));      // pos * num_k_tiles + kt
                     if (key != cur_key) {
-                        ok = mbar_wait_warp(ures_full_bar, loads_seen & 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                        ok = wait_role<PIPE>(ures_full_bar, loads_seen & 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                         if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 6, cta_rank); break; }
                         ++loads_seen;
                         cur_key = key;
                     }
                 }
-                ok = mbar_wait_warp(&acc_empty_bar[buf], acc_phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                ok = wait_role<PIPE>(&acc_empty_bar[buf], acc_phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                 [[maybe_unused]] const int buf1 = buf + 1 == acc_bufs ? 0 : buf + 1;
                 if constexpr (DUAL) {   // this tile fills two accumulators
                     const uint32_t phase1 = buf1 == 0 ? acc_phase ^ 1u : acc_phase;
-                    if (ok) ok = mbar_wait_warp(&acc_empty_bar[buf1], phase1 ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+                    if (ok) ok = wait_role<PIPE>(&acc_empty_bar[buf1], phase1 ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
                 }
                 if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 2, cta_rank); break; }
                 tc_fence_after_sync();
@@ -599,10 +613,8 @@ wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant_
                 [[maybe_unused]] const uint32_t d_tmem1 = tmem_base + static_cast<uint32_t>(buf1 * acc_stride);
                 [[maybe_unused]] constexpr uint64_t a_sub = static_cast<uint64_t>(L::A_BYTES >> 4);   // second block of tiles
                 for (int cb = 0; cb < prm.num_c_blocks; ++cb) {
-                    if (!__all_sync(0xffffffffu, mbar_try_wait_a32(full_a, phase))) {
-                        ok = __all_sync(0xffffffffu, mbar_wait_slow(&full_bar[stage], phase, abort_flag, GEMM_WAIT_LIMIT_NS)) != 0;
-                        if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 3, cta_rank); break; }
-                    }
+                    ok = wait_role_a32<PIPE>(full_a, &full_bar[stage], phase, abort_flag, GEMM_WAIT_LIMIT_NS);
+                    if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 3, cta_rank); break; }
                     tc_fence_after_sync();
                     const uint64_t bd = resident ? ures_desc0 + static_cast<uint64_t>(cb) * ures_step : bdesc;
                     if (!elected) {
