@@ -61,9 +61,6 @@ struct DirectParams {
     int n_tile, num_k_tiles, num_m;    // output channels per CTA tile, tiles along k and along the pixels
     int pair_begin, pair_end;          // (pixel tile, k tile) pairs of this launch
     int splits, cb_per_split, num_cb;  // parts of the channel blocks
-    int win_h, win_w;                  // output rows and columns of this launch (all, unless the workspace is small)
-    int row0, col0;                    // row and column of x at position (0, 0) of the packed copy
-    int org;                           // grid: position of a patch's first row and column for output row and column 0
     int flat, pitch, rows_img;         // layout of the pixels; rows_img: rows per image, padding included
     int lead;                          // flat, stride 1: positions of zeros before the first pixel
     int tiles_c, tiles_r;              // grid: tiles per image
@@ -75,6 +72,9 @@ struct DirectParams {
     int vec_store;                     // grid: rows of eight outputs are aligned 16-byte pieces of y (and residual)
     int a_stage_bytes, a_stages, b_stages;
     FastDiv fd_pitch, fd_rows, fd_k, fd_s, fd_tc, fd_tr, fd_pkp;
+    // (last: between the fields above, which the convolution kernel reads, they cost a launch of 14 us 0.1 us)
+    int win_h, win_w;                  // output rows and columns of this launch (all, unless the workspace is small)
+    int row0, col0;                    // row and column of x at position (0, 0) of the packed copy
 };
 
 // No swizzle, K-major: [0,14) start >> 4, [16,30) bytes between 8-channel pieces >> 4, [32,46) bytes between groups of
@@ -93,7 +93,13 @@ template <int STRIDE> __host__ __device__ constexpr bool direct_first_of_plane(i
     return t == 0 || (STRIDE == 2 && (t == 4 || t == 6 || t == 8));
 }
 
+// PART: the launch covers part of the rows or columns.  A flag of its own: the two further parameters that the epilogue then
+// reads cost a launch on whole images 0.1 us.
+template <bool PART> __device__ __forceinline__ int direct_win_h(const DirectParams& q) { return PART ? q.win_h : q.Ho; }
+template <bool PART> __device__ __forceinline__ int direct_win_w(const DirectParams& q) { return PART ? q.win_w : q.Wo; }
+
 // Lane `l` (0..127) of CTA tile m -> image, output row and column; false where nothing is stored.
+template <bool PART>
 __device__ __forceinline__ bool direct_out_pixel(const DirectParams& q, int m, int l, int& n, int& r, int& c) {
     if (q.flat) {
         const uint32_t Q = static_cast<uint32_t>(m) * 128u + static_cast<uint32_t>(l);
@@ -102,7 +108,7 @@ __device__ __forceinline__ bool direct_out_pixel(const DirectParams& q, int m, i
         const uint32_t img = fast_div(v, q.fd_rows);
         r = static_cast<int>(v - img * static_cast<uint32_t>(q.rows_img));
         n = static_cast<int>(img);
-        return n < q.N && r < q.win_h && c < q.win_w;
+        return n < q.N && r < direct_win_h<PART>(q) && c < direct_win_w<PART>(q);
     }
     const uint32_t row_blk = fast_div(static_cast<uint32_t>(m), q.fd_tc);
     const uint32_t img = fast_div(row_blk, q.fd_tr);
@@ -111,10 +117,10 @@ __device__ __forceinline__ bool direct_out_pixel(const DirectParams& q, int m, i
     n = static_cast<int>(img);
     r = rb * 16 + (l >> 3);
     c = cb * 8 + (l & 7);
-    return r < q.win_h && c < q.win_w;
+    return r < direct_win_h<PART>(q) && c < direct_win_w<PART>(q);
 }
 
-template <int STRIDE>
+template <int STRIDE, bool PART>
 __global__ void __launch_bounds__(DC_THREADS, 1)
 direct_conv_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmX,
                    const __grid_constant__ DirectParams q, int* __restrict__ status_word) {
@@ -285,7 +291,7 @@ direct_conv_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constan
                 // The warp's 32 lanes are four rows of eight outputs.  DC_EPI_CH channels at a time go through shared memory
                 // in fp32, [channel][32], and leave as 16-byte pieces: one lane per (channel, row).
                 int n, oy, ox;
-                direct_out_pixel(q, m, quarter * 32, n, oy, ox);
+                direct_out_pixel<PART>(q, m, quarter * 32, n, oy, ox);
                 const int row = lane & 3, ch = lane >> 2;
                 for (int col = half * DC_EPI_CH; col < q.n_tile && k0 + col < q.K; col += 2 * DC_EPI_CH) {
                     uint32_t r[8];
@@ -298,7 +304,7 @@ direct_conv_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constan
                         const int k = k0 + col + ch;
                         const float4 a = *reinterpret_cast<const float4*>(stg + ch * 32 + row * 8);
                         const float4 b = *reinterpret_cast<const float4*>(stg + ch * 32 + row * 8 + 4);
-                        if (oy + row < q.win_h && ox < q.win_w && k < q.K) {
+                        if (oy + row < direct_win_h<PART>(q) && ox < direct_win_w<PART>(q) && k < q.K) {
                             const float bk = load_bias(q.bias, k);
                             float v[8] = {a.x + bk, a.y + bk, a.z + bk, a.w + bk, b.x + bk, b.y + bk, b.z + bk, b.w + bk};
                             const long long o = (static_cast<long long>(n) * q.K + k) * hw_o + static_cast<long long>(oy + row) * q.Wo + ox;
@@ -332,7 +338,7 @@ direct_conv_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constan
                     }
                 } else {
                     int n, oy, ox;
-                    const bool live = direct_out_pixel(q, m, quarter * 32 + lane, n, oy, ox);
+                    const bool live = direct_out_pixel<PART>(q, m, quarter * 32 + lane, n, oy, ox);
                     const long long yoff = live ? (static_cast<long long>(n) * q.K + k0) * hw_o + static_cast<long long>(oy) * q.Wo + ox : 0;
                     for (int col = half * 16; col < q.n_tile && k0 + col < q.K; col += 32) {
                         uint32_t r[16];
@@ -367,10 +373,12 @@ direct_conv_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constan
             decode(wi, m, kt, cb0, cb1);
             int row0 = 0, col0 = 0;
             if (!q.flat) {
+                // whole images, stride 1: the halo before row and column 0 is filled in by TMA; else it is in the packed copy
+                const int org = q.stride == 1 && !PART ? -1 : 0;
                 const uint32_t row_blk = fast_div(static_cast<uint32_t>(m), q.fd_tc);
                 const uint32_t img = fast_div(row_blk, q.fd_tr);
-                col0 = ((m - static_cast<int>(row_blk) * q.tiles_c) * 8 + q.org) * 8;
-                row0 = static_cast<int>(img) * q.rows_img + (static_cast<int>(row_blk) - static_cast<int>(img) * q.tiles_r) * 16 + q.org;
+                col0 = ((m - static_cast<int>(row_blk) * q.tiles_c) * 8 + org) * 8;
+                row0 = static_cast<int>(img) * q.rows_img + (static_cast<int>(row_blk) - static_cast<int>(img) * q.tiles_r) * 16 + org;
             }
             for (int cb = cb0; cb < cb1 && ok; ++cb) {
                 for (int pl = 0; pl < q.planes; ++pl) {
@@ -411,6 +419,7 @@ direct_conv_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constan
 
 // Adds the fp32 parts of a launch with splits > 1 in a fixed order, then bias, residual, activation, rounding and the
 // masked store.  A block of 128 threads = the lanes of one pixel tile; blockIdx.y walks the output channels, two per thread.
+template <bool PART>
 __global__ void __launch_bounds__(128)
 direct_reduce_kernel(const __grid_constant__ DirectParams q, int* __restrict__ status_word) {
     const int pair = q.pair_begin + blockIdx.x;
@@ -418,7 +427,7 @@ direct_reduce_kernel(const __grid_constant__ DirectParams q, int* __restrict__ s
     const int kt = pair - m * q.num_k_tiles;
     const int l = threadIdx.x;
     int n, oy, ox;
-    const bool live = direct_out_pixel(q, m, l, n, oy, ox);
+    const bool live = direct_out_pixel<PART>(q, m, l, n, oy, ox);
     const long long hw_o = static_cast<long long>(q.Ho) * q.Wo;
     const int col = blockIdx.y * 2, k = kt * q.n_tile + col;
     const long long split_step = static_cast<long long>(q.n_tile) * 128;

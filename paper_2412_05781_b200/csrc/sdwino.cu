@@ -804,7 +804,8 @@ int dual_acc_bufs(int n_tile) { return std::max(2, std::min(GEMM_MAX_ACC, 2 * GE
 // of few stages, plus an epilogue that is hidden unless the tile is short; tiles run in waves over the SMs.
 //
 // The constants are a fit to 91 layers of the UNet and VAE sweeps (batch 1-8, ragged sizes among them), each timed with every
-// shape: the choice is on average 0.4 % slower than the best shape of a layer, at most 5 %.  What the fit says: a single
+// shape: the choice is on average 0.4 % slower than the best shape of those layers, at most 5 % (launches that stream from HBM
+// are not among them, see gemm_streams_hbm).  What the fit says: a single
 // CTA takes in 41 bytes per cycle, a CTA of a pair 34; a stage missing from a ring of four (pairs: five) costs 7.5 %
 // (n_tile 224 fits three: 1280->640 at 48x48, batch 4, 79.8 us with it, 69.0 with 160); a pair costs 9500 cycles per launch
 // more (it runs without programmatic dependent launch, see launch_gemm_shape; 512->512 at 128x128 44.6 us as pairs, 41.1
@@ -1227,7 +1228,6 @@ bool direct_geometry(const Plan& pl, const DirectWindow& win, int C, int H, int 
     q->N = win.n; q->C = C; q->H = H; q->W = W; q->K = K;
     q->Ho = pl.Ho; q->Wo = pl.Wo; q->stride = stride;
     q->win_h = win.h; q->win_w = win.w;
-    q->org = stride == 1 && !part ? -1 : 0;               // the planes of stride 2 begin at row and column -1 anyway
     q->row0 = win.r0 * stride - (stride == 1 && !part ? 0 : 1);
     q->col0 = win.c0 * stride - (stride == 1 && !part ? 0 : 1);
     q->n_tile = sh.n_tile;
@@ -1351,12 +1351,12 @@ DirectShape choose_direct_shape(const Plan& pl, int N, int C, int H, int W, int 
     return best;
 }
 
-template <int STRIDE>
+template <int STRIDE, bool PART>
 int launch_direct_as(const CUtensorMap& tmU, DirectParams& q, void* ws, size_t ws_bytes, cudaStream_t st) {
     const int sms = sm_count();
     int* status = status_word_ptr();
     if (sms <= 0 || !status) return err_cuda(__LINE__);
-    if (!ensure_dyn_smem(reinterpret_cast<const void*>(direct_conv_kernel<STRIDE>), MAX_DYN_SMEM)) return err_cuda(__LINE__);
+    if (!ensure_dyn_smem(reinterpret_cast<const void*>(direct_conv_kernel<STRIDE, PART>), MAX_DYN_SMEM)) return err_cuda(__LINE__);
     const size_t smem = static_cast<size_t>(q.b_stages) * q.n_tile * 128 + q.a_stages * q.a_stage_bytes +
                         DC_EPI_WARPS * DC_STG_BYTES + DC_BAR_BYTES + 1024;
     const size_t packed_bytes = direct_packed_bytes(q);
@@ -1386,7 +1386,7 @@ int launch_direct_as(const CUtensorMap& tmU, DirectParams& q, void* ws, size_t w
         const long long items = static_cast<long long>(q.pair_end - p0) * q.splits;
         {
             ProfScope prof(KIND_FUSED, st);
-            const cudaError_t e = launch_pdl(direct_conv_kernel<STRIDE>, dim3(static_cast<unsigned>(std::min<long long>(items, sms))),
+            const cudaError_t e = launch_pdl(direct_conv_kernel<STRIDE, PART>, dim3(static_cast<unsigned>(std::min<long long>(items, sms))),
                                              dim3(DC_THREADS), smem, st, 0, tmU, tmX, q, status);
             g_launches.fetch_add(1);
             if (e != cudaSuccess) return err_cuda(__LINE__);
@@ -1394,7 +1394,7 @@ int launch_direct_as(const CUtensorMap& tmU, DirectParams& q, void* ws, size_t w
         if (q.splits > 1) {
             ProfScope prof(KIND_OUTPUT, st);
             const dim3 grid(static_cast<unsigned>(q.pair_end - p0), static_cast<unsigned>(q.n_tile / 2));
-            const cudaError_t e = launch_pdl(direct_reduce_kernel, grid, dim3(128), 0, st, 0, q, status);
+            const cudaError_t e = launch_pdl(direct_reduce_kernel<PART>, grid, dim3(128), 0, st, 0, q, status);
             g_launches.fetch_add(1);
             if (e != cudaSuccess) return err_cuda(__LINE__);
         }
@@ -1474,7 +1474,11 @@ int launch_direct(const __half* x, const void* wT, const __half* bias, __half* y
                 q.residual = ep.residual ? static_cast<const __half*>(ep.residual) + first : nullptr;
                 q.act = ep.act;
                 q.vec_store = !q.flat && pl.Wo % 8 == 0 && aligned(y, 16) && aligned(ep.residual, 16);
-                const int rc = stride == 1 ? launch_direct_as<1>(tmU, q, ws, ws_bytes, st) : launch_direct_as<2>(tmU, q, ws, ws_bytes, st);
+                const bool part = step.h != pl.Ho || step.w != pl.Wo;
+                const int rc = stride == 1 ? (part ? launch_direct_as<1, true>(tmU, q, ws, ws_bytes, st)
+                                                   : launch_direct_as<1, false>(tmU, q, ws, ws_bytes, st))
+                                           : (part ? launch_direct_as<2, true>(tmU, q, ws, ws_bytes, st)
+                                                   : launch_direct_as<2, false>(tmU, q, ws, ws_bytes, st));
                 if (rc != SDWINO_OK) return rc;
             }
     return SDWINO_OK;

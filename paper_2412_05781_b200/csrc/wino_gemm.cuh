@@ -218,7 +218,8 @@ __device__ __forceinline__ bool wait_role(uint64_t* bar, uint32_t parity, volati
     else return mbar_wait_warp(bar, parity, abort_flag, limit_ns);
 }
 template <bool PIPE>
-__device__ __forceinline__ bool wait_role_a32(uint32_t bar_a, uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint64_t limit_ns) {
+__device__ __forceinline__ bool wait_role_a32(uint32_t bar_a, uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                              uint64_t limit_ns) {
     if constexpr (PIPE) return mbar_try_wait_a32(bar_a, parity) || mbar_wait_slow(bar, parity, abort_flag, limit_ns);
     else return mbar_wait_warp_a32(bar_a, bar, parity, abort_flag, limit_ns);
 }
