@@ -389,12 +389,15 @@ int sdwino_choose_tile(int N, int C, int H, int W, int K);
 int sdwino_choose_algorithm(int N, int C, int H, int W, int K);
 
 /*
- * Tuning and test knob.  F(2x2,3x3) layers with at most 8 output channels (the 320 -> 4 and 128 -> 3
- * output convolutions) run as ONE kernel that keeps V and M on chip (input transform into shared memory,
+ * Tuning and test knob.  Layers with at most 8 output channels (the 320 -> 4 and 128 -> 3 output convolutions) run as ONE
+ * kernel.  With fp16 tensors, tile 2 or 4, H * W a multiple of 8 and x 16-byte aligned it takes the taps back out of the
+ * transformed filter and reads x as it lies in memory, at any size, unless the rows are too wide for its buffers (K = 3: about
+ * 4100 pixels, K = 8: about 1000; fewer with many input channels).  Other F(2x2,3x3) layers with so few output channels (fp32
+ * tensors, wider rows) run one that keeps V and M on chip (input transform into shared memory,
  * tcgen05 MMAs into TMEM, output transform from TMEM) when the batch has at least `p_tiles` blocks of 128
  * tiles (default 48: below that too few SMs get work and the three-kernel path is faster), W % 8 == 0,
  * x is 16-byte and y 4-byte aligned.  p_tiles = 0 restores the default; 1 sends every eligible layer
- * through the kernel (used by the tests).  Forcing a GEMM shape with sdwino_set_gemm_shape disables it.
+ * through that kernel (used by the tests).  Forcing a GEMM shape with sdwino_set_gemm_shape disables both.
  * Returns SDWINO_ERR_INVALID_ARG for a negative value.  Not thread-safe against concurrent compute calls.
  */
 int sdwino_set_fused_min_tiles(long long p_tiles);

@@ -1,0 +1,378 @@
+// Layers with few output channels (K <= 8: the 128->3 and 320->4 output convolutions) as one kernel without V, M or a
+// workspace.  With so few channels the nine taps fit the columns of one small accumulator: for 128 consecutive pixels q of
+// an image
+//   D[q][(tap, k)] = sum_c x[c][q] g[tap][k][c]
+// is one GEMM with N = 9 K columns whose A operand is x itself (NCHW: pixels contiguous, M-major), brought in by TMA as it
+// lies in memory, and y[k][q] is the sum of nine shifted columns of D, taken in fp32.  x crosses memory once, nothing of it
+// is rounded, and no thread touches it.
+//
+// The taps g are taken back out of the transformed filter: G has full column rank, so g = T U T^t with T G = 1.  For F(2x2)
+// T = {U0, U1 - U2, U3}; for F(4x4) the middle tap is the scaled difference of the points +-3/4 (a rounding of U then counts
+// 1.3 times; all six rows would bring that to 0.94, at 36 instead of 16 positions that every CTA reads).  The result is nearer
+// to the convolution than either Winograd path, whose V or M are rounded to fp16.
+//
+// A CTA takes a run of consecutive pixels of one image and walks it in tiles of 128, two at a time, one row and one pixel further than
+// the run at both ends.  The row above and below a pixel are other tiles of the walk: the sums over the three columns of each
+// tap row go into two rings in shared memory, of two rows (P0) and one row (P1) and two tiles each.  Odd CTAs walk backwards,
+// so that the rows that two neighbours both need are read by both at their beginning or by both at their end, the second
+// time from L2.  A backward walk is the forward one on a mirrored image: its taps are stored in mirrored order.
+//
+// Warp 0 loads x, warps 1 and 2 issue the MMAs of alternate tiles (a small MMA costs its issuer 70 cycles whatever its N, and
+// two issuers overlap), warps 4-7 and 8-11 sum the taps of a pair of tiles; before that, warps 1-15 recover the taps.
+//
+// 128->3 at 1024x1024 170 us with fused_small_k_kernel, which is bound by the load instructions of its threads, 64.2 here: x
+// crosses HBM exactly once (269 MB, 4.2 TB/s), and the CTAs on the slower third of the SMs take 25 % longer than the mean.  At
+// 512x512 53.1 -> 19.1; 320->4 with F(4x4) filters, three kernels before, 24.7 -> 10.9 at 128x128 (batch 2), 27.7 -> 9.9 at 96x96
+// (batch 4) and 10.4 -> 7.3 at 64x64 (batch 2), a chain of filters (1.5 us), first tile and sums.  Relative error (2-norm)
+// against fp64 3.0e-4, 6.0e-4 with F(2x2), 3.3e-4 instead of 1.9e-3 with F(4x4).
+#pragma once
+#include <cuda_fp16.h>
+
+#include "ptx.cuh"
+#include "transforms.cuh"
+#include "wino_gemm.cuh"
+
+namespace sdw {
+
+constexpr int FO_THREADS = 512;
+constexpr int FO_TILE = 128;                   // pixels per tile (UMMA M)
+constexpr int FO_PAIR = 2 * FO_TILE;           // pixels whose taps are summed at a time
+constexpr int FO_SUM_WARP0 = 4;                // warps 4-11
+constexpr int FO_ACCS = 4;                     // accumulators in tensor memory
+constexpr int FO_KMAX = 8;
+constexpr int FO_STAGE_BYTES = 2 * 64 * 128;   // 64 channels of a tile: two boxes [64 c][64 q]
+constexpr int FO_MAX_STAGES = 10;
+constexpr int FO_DPITCH = FO_PAIR + 2;         // columns of D of a pair of tiles, behind the last two before it
+constexpr int FO_BAR_BYTES = (2 * FO_MAX_STAGES + 2 * FO_ACCS) * 8 + 16;
+__host__ __device__ constexpr int fo_k(int K) { return K <= 3 ? 3 : (K <= 4 ? 4 : 8); }             // columns per tap
+__host__ __device__ constexpr int fo_n(int kp) { return (9 * kp + 15) / 16 * 16; }                  // UMMA N
+__host__ __device__ constexpr int fo_acc_cols(int kp) { return kp == 3 ? 32 : (kp == 4 ? 64 : 128); }   // four of them: a power of two
+__host__ __device__ constexpr int fo_ring0(int W) { return 2 * W + FO_PAIR; }
+__host__ __device__ constexpr int fo_ring1(int W) { return W + FO_PAIR; }
+// dynamic shared memory: filters and stages (1 KB aligned), rings, columns of D, barriers
+__host__ __device__ constexpr long long fo_smem(int kp, int W, int cblocks, int stages) {
+    return static_cast<long long>(cblocks) * fo_n(kp) * 128 + static_cast<long long>(stages) * FO_STAGE_BYTES +
+           4ll * kp * (3ll * W + 2 * FO_PAIR) + 4ll * 6 * kp * FO_DPITCH + 16 + FO_BAR_BYTES + 1024;
+}
+
+struct FewOutputsParams {
+    const uint32_t* wt_header;
+    const __half* U;
+    const __half* bias;
+    __half* y;
+    int C, K, tile, W;
+    int hw;             // pixels per image, a multiple of 8
+    int cblocks;        // ceil(C / 64)
+    int per_image;      // CTAs per image
+    int run;            // pixels per CTA
+    int stages;
+    FastDiv w_div;
+};
+
+// T: rows of the left inverse of G.
+template <int M> __device__ __forceinline__ float fo_left_inverse(int i, int j);
+template <> __device__ __forceinline__ float fo_left_inverse<2>(int i, int j) {
+    constexpr float m[3][4] = {{1, 0, 0, 0}, {0, 1, -1, 0}, {0, 0, 0, 1}};
+    return m[i][j];
+}
+template <> __device__ __forceinline__ float fo_left_inverse<4>(int i, int j) {
+    constexpr float m[3][4] = {{81.f / 64.f, 0, 0, 0}, {0, -81.f / 64.f, 81.f / 64.f, 0}, {0, 0, 0, 1}};   // rows 0, 1, 2 and 5 of U
+    return m[i][j];
+}
+
+// The taps of all output channels as the B operand: blocks of 64 channels, rows n = tap * KP + k of 128 bytes, 128-byte
+// swizzle; zeros in the rows past 9 KP and k >= K.
+template <int M, int KP>
+__device__ __forceinline__ void fo_recover_taps(const FewOutputsParams& q, uint8_t* b_smem, int tid, int threads, bool mirror) {
+    constexpr int A = 4, NP = fo_n(KP);        // rows and columns 0, 1, 2 and the last of U
+    const int pairs = q.cblocks * 32;          // pairs of input channels, up to the padding of U
+    const size_t plane = static_cast<size_t>(q.cblocks) * 1024;     // K <= 8: one block of output channels
+    for (int item = tid; item < q.K * pairs; item += threads) {
+        const int k = item / pairs, cp = item - k * pairs, cb = cp >> 5, c = (cp & 31) * 2;
+        const __half2* u = reinterpret_cast<const __half2*>(q.U + cb * 1024 + k * 64 + c);
+        __half2 uv[A][A];
+#pragma unroll
+        for (int i = 0; i < A; ++i)
+#pragma unroll
+            for (int j = 0; j < A; ++j) uv[i][j] = u[((i < 3 ? i : M + 1) * (M + 2) + (j < 3 ? j : M + 1)) * (plane / 2)];
+        float2 t[3][A];
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int j = 0; j < A; ++j) {
+                float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int i = 0; i < A; ++i) {
+                    const float f = fo_left_inverse<M>(r, i);
+                    if (f != 0.f) {
+                        const float2 v = __half22float2(uv[i][j]);
+                        s.x = fmaf(f, v.x, s.x);
+                        s.y = fmaf(f, v.y, s.y);
+                    }
+                }
+                t[r][j] = s;
+            }
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int s = 0; s < 3; ++s) {
+                float2 g = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int j = 0; j < A; ++j) {
+                    const float f = fo_left_inverse<M>(s, j);
+                    if (f != 0.f) {
+                        g.x = fmaf(f, t[r][j].x, g.x);
+                        g.y = fmaf(f, t[r][j].y, g.y);
+                    }
+                }
+                const int tap = mirror ? 8 - (3 * r + s) : 3 * r + s;
+                const int n = tap * KP + k;
+                *reinterpret_cast<__half2*>(b_smem + cb * (NP * 128) + n * 128 + (((c >> 3) ^ (n & 7)) << 4) + (c & 7) * 2) =
+                    __floats2half2_rn(g.x, g.y);
+            }
+    }
+    for (int i = tid; i < q.cblocks * NP * 8; i += threads) {
+        const int n = (i >> 3) % NP;
+        if (n >= 9 * KP || n % KP >= q.K) *reinterpret_cast<uint4*>(b_smem + static_cast<size_t>(i) * 16) = make_uint4(0, 0, 0, 0);
+    }
+}
+
+// tmX: fp16 [N][C][H * W], box {64 q, 64 c, 1}, 128-byte swizzle (A operand, M-major; pixels and channels outside read as 0)
+template <int KP>
+__global__ void __launch_bounds__(FO_THREADS, 1)
+few_outputs_kernel(const __grid_constant__ CUtensorMap tmX, const FewOutputsParams q, int* __restrict__ status_word) {
+    constexpr int NP = fo_n(KP), ACC = fo_acc_cols(KP);
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* a_smem = smem;
+    uint8_t* b_smem = smem + q.stages * FO_STAGE_BYTES;
+    const int r0_len = fo_ring0(q.W), r1_len = fo_ring1(q.W);
+    float* ring0 = reinterpret_cast<float*>(b_smem + q.cblocks * NP * 128);
+    float* ring1 = ring0 + KP * r0_len;
+    float* dcol = ring1 + KP * r1_len;         // [tap row][tap column 0, 1][k][FO_DPITCH]
+    uint64_t* full_bar = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(dcol + 6 * KP * FO_DPITCH) + 7) & ~uintptr_t(7));
+    uint64_t* empty_bar = full_bar + FO_MAX_STAGES;
+    uint64_t* acc_full = empty_bar + FO_MAX_STAGES;
+    uint64_t* acc_empty = acc_full + FO_ACCS;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + FO_ACCS);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);
+
+    // the run of this CTA and its walk
+    const int img = blockIdx.x / q.per_image;
+    const int part = blockIdx.x - img * q.per_image;
+    const int q0 = part * q.run, q1 = min(q0 + q.run, q.hw);
+    const bool mirror = part & 1;
+    // a walk starts at the first pixel that D is needed for, on a 128-byte line of x
+    const int start = mirror ? (q1 + q.W + 1 + 63) & ~63 : (q0 - q.W - 1) & ~63;
+    const int tiles = q0 >= q1 ? 0 : ((mirror ? start - q0 : q1 - start) + q.W + 1 + FO_TILE - 1) / FO_TILE;
+
+    if (threadIdx.x < 2 * FO_MAX_STAGES + 2 * FO_ACCS) {
+        mbar_init(&full_bar[threadIdx.x], threadIdx.x >= 2 * FO_MAX_STAGES + FO_ACCS ? 4 : 1);   // acc_empty: four summing warps
+        fence_barrier_init();
+    }
+    if (threadIdx.x == FO_THREADS - 32) {
+        *abort_flag = 0;
+        prefetch_tmap(&tmX);
+    }
+    if (warp == 1) { tmem_alloc(tmem_slot, FO_ACCS * ACC); tmem_relinquish(); }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    const bool elected = elect_one() != 0;
+    pdl_wait();                 // x and the filters may be the preceding kernel's
+    pdl_launch_dependents();
+    const bool wt_ok = wt_header_ok(q.wt_header, q.K, q.C, q.tile, status_word);   // the same answer for the whole grid
+
+    const uint32_t a_base = smem_u32(a_smem), full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
+    // ------------------------------ x ------------------------------
+    int tile = 0, cb = 0, stage = 0;           // of the load to issue next
+    uint32_t phase = 0;
+    auto load = [&]() {                        // issues it and moves on
+        if (elected) {
+            const uint32_t bar = full0 + stage * 8, dst = a_base + stage * FO_STAGE_BYTES;
+            const int p0 = mirror ? start - (tile + 1) * FO_TILE : start + tile * FO_TILE;
+            mbar_arrive_expect_tx_a32(bar, FO_STAGE_BYTES);
+            tma_load_3d_a32(dst, &tmX, bar, p0, cb * 64, img);
+            tma_load_3d_a32(dst + FO_STAGE_BYTES / 2, &tmX, bar, p0 + 64, cb * 64, img);
+        }
+        // a block of channels of both tiles of a pair, one after the other: 512 contiguous bytes of every channel
+        if (!(tile & 1) && tile + 1 < tiles) ++tile;
+        else if (++cb < q.cblocks) tile &= ~1;
+        else { cb = 0; ++tile; }
+        if (++stage == q.stages) { stage = 0; phase ^= 1u; }
+    };
+    if (wt_ok) {
+        if (warp == 0) {                       // the first ring-full is on its way while the other warps work on the taps
+            for (int i = 0; i < q.stages && tile < tiles; ++i) load();
+        } else {
+            const int tid = threadIdx.x - 32;
+            if (q.tile == 2) fo_recover_taps<2, KP>(q, b_smem, tid, FO_THREADS - 32, mirror);
+            else fo_recover_taps<4, KP>(q, b_smem, tid, FO_THREADS - 32, mirror);
+            fence_proxy_async_smem();          // the tensor core reads them through the async proxy
+        }
+    }
+    __syncthreads();
+
+    if (!wt_ok) {
+        // a filter buffer of another layer: nothing is computed
+    } else if (warp == 0) {
+        bool ok = true;
+        while (tile < tiles) {
+            ok = mbar_wait_warp(&empty_bar[stage], phase ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+            if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 1, 0); break; }
+            load();
+        }
+        if (!ok) *abort_flag = 1;
+    } else if (warp <= 2) {
+        // ------------------------------ MMA ------------------------------
+        const uint32_t idesc = make_idesc_f16_f32(FO_TILE, NP, true, false);
+        const uint64_t adesc0 = make_smem_desc_sw128(a_base, FO_STAGE_BYTES / 2, 1024);
+        const uint64_t bdesc0 = make_smem_desc_sw128(smem_u32(b_smem), 16, 1024);
+        bool ok = true;
+        for (int t = warp - 1; t < tiles && ok; t += 2) {
+            const int buf = t % FO_ACCS;
+            const int by = (t | 1) < tiles ? 2 : 1;  // the loads of a pair of tiles alternate between them
+            const int first = (t & ~1) * q.cblocks + (by == 2 ? (t & 1) : 0);
+            int ms = first % q.stages;
+            uint32_t mphase = (first / q.stages) & 1;
+            ok = mbar_wait_warp(&acc_empty[buf], ((t / FO_ACCS) & 1) ^ 1u, abort_flag, GEMM_WAIT_LIMIT_NS);
+            if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 2, 0); break; }
+            tc_fence_after_sync();
+            const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * ACC);
+            for (int b = 0; b < q.cblocks; ++b) {
+                ok = mbar_wait_warp_a32(full0 + ms * 8, &full_bar[ms], mphase, abort_flag, GEMM_WAIT_LIMIT_NS);
+                if (!ok) { if (*abort_flag == 0) report_timeout(status_word, 3, 0); break; }
+                tc_fence_after_sync();
+                const uint64_t ad = adesc0 + static_cast<uint64_t>(ms * (FO_STAGE_BYTES >> 4));
+                const uint64_t bd = bdesc0 + static_cast<uint64_t>(b * (NP * 128 >> 4));
+                const int ksteps = min(4, (q.C - b * 64 + 15) >> 4);
+                if (elected) {
+#pragma unroll
+                    for (int s = 0; s < 4; ++s)
+                        if (s < ksteps) umma_f16(d_tmem, ad + 128 * s, bd + 2 * s, idesc, (b > 0 || s > 0) ? 1u : 0u);
+                    umma_commit_a32(empty0 + ms * 8);
+                }
+                ms += by;
+                if (ms >= q.stages) { ms -= q.stages; mphase ^= 1u; }
+            }
+            if (!ok) break;
+            if (elected) umma_commit(&acc_full[buf]);
+        }
+        if (!ok) *abort_flag = 1;
+    } else if (warp >= FO_SUM_WARP0 && warp < FO_SUM_WARP0 + 8) {
+        // ------------------------------ sums over the taps ------------------------------
+        // Thread l (in the order of the walk) holds D of pixel own = l and sums the columns of the pixel before it, whose
+        // neighbours are l - 2, l - 1 and l: tap columns 0 and 1 come from the threads before it.
+        const int quarter = warp & 3;
+        const int lane_px = quarter * 32 + (threadIdx.x & 31);          // TMEM lane = pixel within the tile
+        const int half = (warp - FO_SUM_WARP0) >> 2;                    // which tile of the pair
+        const int l = half * FO_TILE + (mirror ? FO_TILE - 1 - lane_px : lane_px);
+        const int step = mirror ? -q.W : q.W;
+        float bias[KP];
+#pragma unroll
+        for (int k = 0; k < KP; ++k) bias[k] = k < q.K ? load_bias(q.bias, k) : 0.f;
+        const uint32_t wrap = static_cast<uint32_t>((FO_PAIR / q.W + 4) * q.W);   // a multiple of W that makes every pixel positive
+        __half* y = q.y + static_cast<long long>(img) * q.K * q.hw;
+        int s0 = l, s1 = l;                    // ring slots of this thread's pixel
+        for (int t0 = 0; t0 < tiles; t0 += 2) {
+            const int t = t0 + half, buf = t % FO_ACCS;
+            const bool live = t < tiles;                 // (the second tile of the last pair may not be there)
+            bool ok = !live || mbar_wait_bounded(&acc_full[buf], (t / FO_ACCS) & 1, abort_flag, GEMM_WAIT_LIMIT_NS);
+            ok = named_barrier_and(1, 2 * FO_TILE, ok);  // the eight warps give up together or not at all
+            if (!ok) {
+                if (l == 0) {
+                    if (*abort_flag == 0) report_timeout(status_word, 4, 0);
+                    *abort_flag = 1;
+                }
+                break;
+            }
+            tc_fence_after_sync();
+            const uint32_t t_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(buf * ACC);
+            float d[NP];
+#pragma unroll
+            for (int c = 0; c + 32 <= NP; c += 32) {
+                uint32_t r[32];
+                tmem_ld_32x32_sync(t_addr + c, r);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) d[c + i] = __uint_as_float(r[i]);
+            }
+            if constexpr (NP % 32 != 0) {
+                uint32_t r[16];
+                tmem_ld_32x16_sync(t_addr + NP - 16, r);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) d[NP - 16 + i] = __uint_as_float(r[i]);
+            }
+            tc_fence_before_sync();
+            __syncwarp();
+            if (live && (threadIdx.x & 31) == 0) mbar_arrive(&acc_empty[buf]);
+#pragma unroll
+            for (int r = 0; r < 3; ++r)
+#pragma unroll
+                for (int s = 0; s < 2; ++s)
+#pragma unroll
+                    for (int k = 0; k < KP; ++k) dcol[((r * 2 + s) * KP + k) * FO_DPITCH + l + 2] = d[(r * 3 + s) * KP + k];
+            named_barrier_sync(1, 2 * FO_TILE);
+            // the pixel before this thread's own, and whether its neighbours (in the order of the walk) are in its row
+            const int px = mirror ? start - t0 * FO_TILE - l : start + t0 * FO_TILE + l - 1;
+            const uint32_t pw = static_cast<uint32_t>(px + static_cast<int>(wrap));
+            const int w = static_cast<int>(pw - fast_div(pw, q.w_div) * static_cast<uint32_t>(q.W));
+            const bool west = w > 0, east = w + 1 < q.W;
+            const bool has_before = mirror ? east : west, has_after = mirror ? west : east;
+            float p2[KP];
+#pragma unroll
+            for (int r = 0; r < 3; ++r)
+#pragma unroll
+                for (int k = 0; k < KP; ++k) {
+                    const float before = dcol[((r * 2 + 0) * KP + k) * FO_DPITCH + l];
+                    float v = dcol[((r * 2 + 1) * KP + k) * FO_DPITCH + l + 1];
+                    if (has_before) v += before;
+                    if (has_after) v += d[(r * 3 + 2) * KP + k];
+                    if (r == 0) ring0[k * r0_len + s0] = v;
+                    else if (r == 1) ring1[k * r1_len + s1] = v;
+                    else p2[k] = v;
+                }
+            named_barrier_sync(1, 2 * FO_TILE);
+            if (l >= FO_PAIR - 2) {            // the last two columns stand before the next pair's
+#pragma unroll
+                for (int r = 0; r < 3; ++r)
+#pragma unroll
+                    for (int s = 0; s < 2; ++s)
+#pragma unroll
+                        for (int k = 0; k < KP; ++k)
+                            dcol[((r * 2 + s) * KP + k) * FO_DPITCH + l + 2 - FO_PAIR] = d[(r * 3 + s) * KP + k];
+            }
+            const int o = px - step;           // the output pixel whose last tap row this was
+            if (live && o >= q0 && o < q1) {
+                int b0 = s0 - 2 * q.W, b1 = s1 - q.W;
+                if (b0 < 0) b0 += r0_len;
+                if (b1 < 0) b1 += r1_len;
+#pragma unroll
+                for (int k = 0; k < KP; ++k)
+                    if (k < q.K)
+                        y[static_cast<long long>(k) * q.hw + o] =
+                            __float2half_rn(((ring0[k * r0_len + b0] + ring1[k * r1_len + b1]) + p2[k]) + bias[k]);
+            }
+            s0 += FO_PAIR;
+            if (s0 >= r0_len) s0 -= r0_len;
+            s1 += FO_PAIR;
+            if (s1 >= r1_len) s1 -= r1_len;
+        }
+    }
+
+    __syncwarp();
+    __syncthreads();
+    if (*abort_flag != 0) {
+        // copies and MMAs that may still be in flight get a bounded time to land before their memory is released
+        const uint64_t t0 = global_timer_ns();
+        while (global_timer_ns() - t0 < 200000ull) __nanosleep(1000);
+        __syncthreads();
+    }
+    if (warp == 1) {
+        tc_fence_after_sync();
+        tmem_dealloc(tmem_base, FO_ACCS * ACC);
+    }
+}
+
+}  // namespace sdw

@@ -18,6 +18,7 @@
 #include "transforms.cuh"
 #include "transforms_any.cuh"
 #include "wino_gemm.cuh"
+#include "few_outputs.cuh"
 #include "fused_small_k.cuh"
 #include "input_tma.cuh"
 #include "output_tma.cuh"
@@ -711,7 +712,8 @@ int launch_fused_small_c(const __half* x, const void* wT, const __half* bias, __
     return e == cudaSuccess ? SDWINO_OK : err_cuda(__LINE__);
 }
 
-// Layers with at most 8 output channels run F(2x2,3x3) as one fused tensor-core kernel (no workspace traffic):
+// Layers with at most 8 output channels that few_outputs_kernel does not take (fp32 tensors, rows or filters too long for its
+// buffers) run F(2x2,3x3) as one fused tensor-core kernel (no workspace traffic):
 // see fused_small_k.cuh.  It needs the vector loads of the input transform (W % 8 == 0, aligned x) and
 // 4-byte output stores.
 // A CTA takes 128 tiles and all input channels, so the kernel only pays off when there are enough blocks
@@ -745,6 +747,57 @@ int launch_fused_small_k(const T* x, const void* wT, const T* bias, T* y, const 
                                      static_cast<size_t>(FK_DYN_SMEM), st, 1, tmU, x, bias, y, prm, status);
     g_launches.fetch_add(1);
     return e == cudaSuccess ? SDWINO_OK : err_cuda(__LINE__);
+}
+
+// Layers with at most 8 output channels, fp16 tensors: see few_outputs.cuh.  TMA reads x as [N][C][H * W], whose rows must be
+// whole 16-byte pieces, and the rings of two rows must fit beside at least three stages (K = 3: up to about 4000 pixels wide).
+bool plan_few_outputs(int N, int C, int H, int W, int K, int tile, const void* x, int sms, FewOutputsParams* q) {
+    const long long hw = static_cast<long long>(H) * W;
+    if (K > FO_KMAX || (tile != 2 && tile != 4) || hw % 8 != 0 || !aligned(x, 16) || hw >= (1ll << 30) || W > 8192) return false;
+    const int kp = fo_k(K);
+    q->C = C; q->K = K; q->tile = tile; q->W = W;
+    q->hw = static_cast<int>(hw);
+    q->cblocks = (C + 63) / 64;
+    q->stages = FO_MAX_STAGES;
+    while (q->stages >= 3 && fo_smem(kp, W, q->cblocks, q->stages) > MAX_DYN_SMEM) --q->stages;
+    if (q->stages < 3) return false;
+    // One or two waves of CTAs, whichever finishes first.  A CTA walks its run and a row and a pixel beyond both ends in tiles
+    // of 128, and takes about two tiles' time to begin.
+    double best = 1e300;
+    for (int waves = 1; waves <= 2; ++waves) {
+        const long long want = std::max<long long>(1, static_cast<long long>(sms) * waves / N);
+        const long long run = (hw + want - 1) / want, ctas = (hw + run - 1) / run;
+        const long long tiles = (run + 2ll * W + 2 + 63 + FO_TILE - 1) / FO_TILE;
+        const double cost = static_cast<double>((ctas * N + sms - 1) / sms) * (tiles + 2.0);
+        if (cost < best) { best = cost; q->per_image = static_cast<int>(ctas); q->run = static_cast<int>(run); }
+    }
+    q->w_div = make_fastdiv(static_cast<uint32_t>(W));
+    return static_cast<long long>(q->per_image) * N < (1ll << 31);
+}
+
+template <int KP>
+int launch_few_outputs_as(const CUtensorMap& tmX, const FewOutputsParams& q, int N, int* status, cudaStream_t st) {
+    if (!ensure_dyn_smem(reinterpret_cast<const void*>(few_outputs_kernel<KP>), MAX_DYN_SMEM)) return err_cuda(__LINE__);
+    ProfScope prof(KIND_FUSED, st);
+    const cudaError_t e = launch_pdl(few_outputs_kernel<KP>, dim3(static_cast<unsigned>(q.per_image * N)), dim3(FO_THREADS),
+                                     static_cast<size_t>(fo_smem(KP, q.W, q.cblocks, q.stages)), st, 0, tmX, q, status);
+    g_launches.fetch_add(1);
+    return e == cudaSuccess ? SDWINO_OK : err_cuda(__LINE__);
+}
+
+int launch_few_outputs(const __half* x, const void* wT, const __half* bias, __half* y, int N, FewOutputsParams& q, cudaStream_t st) {
+    int* status = status_word_ptr();
+    CUtensorMap tmX;
+    if (!status || !encode_map(&tmX, x, q.hw, q.C, N, q.hw, static_cast<uint64_t>(q.C) * q.hw, 64, 64, true)) return err_cuda(__LINE__);
+    q.wt_header = wt_header_of(wT);
+    q.U = static_cast<const __half*>(wt_filters_of(wT));
+    q.bias = bias;
+    q.y = y;
+    switch (fo_k(q.K)) {
+        case 3: return launch_few_outputs_as<3>(tmX, q, N, status, st);
+        case 4: return launch_few_outputs_as<4>(tmX, q, N, status, st);
+        default: return launch_few_outputs_as<8>(tmX, q, N, status, st);
+    }
 }
 
 // F(2x2,3x3) layers with at most 8 input channels: one warp-MMA kernel (see fused_small_c_mma_kernel).
@@ -1537,6 +1590,13 @@ int conv_impl(const void* x, const void* wT, const void* bias, void* y, int N, i
     // (8-bit filters: only the GEMM can read them, so neither the single-kernel paths nor the pipelined launch)
     const bool no_ep = ep.residual == nullptr && ep.act == 0 && ep.amax == nullptr && !q8;
     const bool plain = no_ep && !io32;
+    if (plain && K <= FO_KMAX && !use_fused_small_c(C, tile) && !disable_fused) {
+        const int sms = sm_count();
+        if (sms <= 0) return err_cuda(__LINE__);
+        FewOutputsParams q;
+        if (plan_few_outputs(N, C, H, W, K, tile, x, sms, &q))
+            return launch_few_outputs(static_cast<const __half*>(x), wT, static_cast<const __half*>(bias), static_cast<__half*>(y), N, q, st);
+    }
     if (no_ep && use_fused_small_k(K, W, tile, pl.P128 / 128, x, y) && !use_fused_small_c(C, tile) &&
         (!io32 || aligned(y, 8)) && !disable_fused) {
         if (io32)

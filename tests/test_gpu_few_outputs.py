@@ -1,0 +1,58 @@
+"""Layers with at most 8 output channels, fp16 tensors: one kernel that reads x as it lies in memory."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2412_05781_b200 import workloads
+from paper_2412_05781_b200.workloads import ConvLayer
+
+pytestmark = pytest.mark.gpu
+
+# C, K, H, W, N: runs shorter and longer than a tile and a row, several images, channel blocks of 64 and their rests, one and
+# several rounds of the ring of stages, each column layout (K <= 3, 4, 8), images one pixel wide or high, and rows that do
+# not begin on 16 bytes (H * W is a multiple of 8, W is not)
+SHAPES = [(16, 4, 8, 8, 1), (70, 3, 10, 16, 2), (130, 8, 17, 24, 2), (320, 4, 64, 64, 2), (300, 5, 7, 8, 3), (129, 1, 9, 48, 1),
+          (64, 2, 130, 136, 1), (128, 3, 96, 160, 1), (24, 4, 8, 1, 2), (24, 3, 1, 264, 1), (40, 6, 16, 37, 2), (9, 8, 24, 131, 1),
+          (1280, 4, 24, 24, 1), (72, 3, 8, 1500, 3)]
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2412_05781_b200 import binding
+    return binding
+
+
+@pytest.mark.parametrize("tile", [2, 4])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_against_the_oracle(B, shape, tile):
+    C, K, H, W, N = shape
+    x, w, b = workloads.make_inputs(ConvLayer(C=C, K=K, H=H, W=W, N=N), seed=sum(shape))
+    ref = oracle.direct_conv3x3(x.numpy(), w.numpy(), b.numpy())
+    wT = B.sdwino_filter_transform(w.cuda(), tile)
+    ws = B.alloc_workspace(B.sdwino_workspace_bytes(N, C, H, W, K, tile))
+    y = torch.full((N, K, H, W), float("nan"), dtype=torch.float16, device="cuda")
+    n0 = B.sdwino_launch_count()
+    B.sdwino_conv3x3(x.cuda(), wT, b.cuda(), K, tile, y=y, workspace=ws)
+    assert B.sdwino_launch_count() - n0 == 1
+    again = B.sdwino_conv3x3(x.cuda(), wT, b.cuda(), K, tile, workspace=ws)
+    assert B.sdwino_last_device_status() == B.OK
+    assert torch.equal(y, again)
+    # What is rounded: U (2**-11 of a value whose share in a tap is at most twice the tap for F(2x2), 0.94 of a rounding in the
+    # mean for F(4x4)), the tap and y.  A sum of 9 C products of independent signs errs by a few times 2**-11 of its rms, which
+    # is a fifth to a third of max|ref|.
+    assert np.abs(y.cpu().double().numpy() - ref).max() <= 1.2e-3 * np.abs(ref).max()
+
+
+def test_wrong_filters_are_refused(B):
+    x, w, b = workloads.make_inputs(ConvLayer(C=32, K=4, H=16, W=16, N=1), seed=1)
+    wT = B.sdwino_filter_transform(w.cuda(), 2)
+    ws = B.alloc_workspace(B.sdwino_workspace_bytes(1, 32, 16, 16, 4, 4))
+    y = torch.full((1, 4, 16, 16), 7.0, dtype=torch.float16, device="cuda")
+    B.sdwino_conv3x3(x.cuda(), wT, b.cuda(), 4, 2, y=y, workspace=ws)
+    assert B.sdwino_last_device_status() == B.OK
+    y.fill_(7.0)
+    wT[:16].view(torch.int32)[3] = 4            # a header that says F(4x4)
+    B.sdwino_conv3x3(x.cuda(), wT, b.cuda(), 4, 2, y=y, workspace=ws)
+    assert B.sdwino_last_device_status() == B.ERR_INVALID_ARG
+    assert torch.all(y == 7.0)
