@@ -436,7 +436,10 @@ int launch_filter(const WT* w, void* wT, int K, int C, int Kb, int Cb, cudaStrea
     ProfScope prof(KIND_FILTER, st);
     uint32_t* header = static_cast<uint32_t*>(wT);
     __half* U = reinterpret_cast<__half*>(static_cast<uint8_t*>(wT) + WT_HEADER_BYTES);
-    const cudaError_t e = launch_pdl(filter_transform_kernel<M, WT>, grid, dim3(128), 0, st, 0, w, header, U, K, C, Kb, Cb);
+    // the 18 weights of a thread's two channels begin at a multiple of their pairs: C even
+    const bool words = C % 2 == 0 && aligned(w, 2 * sizeof(WT));
+    const cudaError_t e = words ? launch_pdl(filter_transform_kernel<M, WT, true>, grid, dim3(128), 0, st, 0, w, header, U, K, C, Kb, Cb)
+                                : launch_pdl(filter_transform_kernel<M, WT>, grid, dim3(128), 0, st, 0, w, header, U, K, C, Kb, Cb);
     g_launches.fetch_add(1);
     return e == cudaSuccess ? SDWINO_OK : err_cuda(__LINE__);
 }

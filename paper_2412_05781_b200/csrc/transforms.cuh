@@ -12,6 +12,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "ptx.cuh"
 
 namespace sdw {
@@ -194,9 +196,11 @@ __device__ __forceinline__ bool wt_check(const WtCheck& c) {
 // with the blocks of consecutive output channels next to each other, so that the [n_tile k][64 c]
 // operand box of one GEMM pipeline stage is ONE contiguous piece of n_tile/16 x 2 KB of DRAM instead of
 // n_tile separate 128-byte rows (the weights are the one operand that is streamed from HBM).  One thread per (k, pair of c) of the padded plane.
-// Writes all a*a positions.
+// Writes all a*a positions.  WORDS: the 18 weights of the pair are nine aligned words (C even); read one by one they are
+// twice as many load instructions, each over as many cache lines, which is what bounded F(2x2): 1280x1280 18.7 -> 15.4 us
+// (82 MB, 5.3 TB/s), 2560x1280 35.6 -> 28.5, fp32 weights 22.1 -> 19.0; F(4x4), bound by its 36 stores, 27.4 -> 26.8.
 // ---------------------------------------------------------------------------------------
-template <int M, typename WT = __half>
+template <int M, typename WT = __half, bool WORDS = false>
 __global__ void __launch_bounds__(128)
 filter_transform_kernel(const WT* __restrict__ w, uint32_t* __restrict__ header, __half* __restrict__ U, int K,
                         int C, int Kb, int Cb) {
@@ -214,15 +218,33 @@ filter_transform_kernel(const WT* __restrict__ w, uint32_t* __restrict__ header,
                                                        static_cast<uint32_t>(M));
     if (c >= Cb * 64) return;
     float u[2][A][A];
+    float wv[18];
+    if constexpr (WORDS) {
+        using W2 = std::conditional_t<sizeof(WT) == 2, __half2, float2>;
+        const W2* wp = reinterpret_cast<const W2*>(w + (static_cast<size_t>(k) * C + c) * 9);
+        const bool live = c < C && k < K;          // C is even
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            float2 v = make_float2(0.f, 0.f);
+            if (live) {
+                if constexpr (sizeof(WT) == 2) v = __half22float2(wp[i]);
+                else v = wp[i];
+            }
+            wv[2 * i] = v.x;
+            wv[2 * i + 1] = v.y;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 18; ++i)
+            wv[i] = c + i / 9 < C && k < K ? to_f32(w[(static_cast<size_t>(k) * C + c) * 9 + i]) : 0.f;
+    }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         float g[3][3];
-        const bool live = (c + h < C) && (k < K);
 #pragma unroll
         for (int r = 0; r < 3; ++r)
 #pragma unroll
-            for (int s = 0; s < 3; ++s)
-                g[r][s] = live ? to_f32(w[(static_cast<size_t>(k) * C + c + h) * 9 + r * 3 + s]) : 0.f;
+            for (int s = 0; s < 3; ++s) g[r][s] = wv[9 * h + 3 * r + s];
         // t = G g  (A x 3), u = t G^T (A x A)
         float t[A][3];
 #pragma unroll
