@@ -18,6 +18,7 @@
 #include "transforms.cuh"
 #include "transforms_any.cuh"
 #include "wino_gemm.cuh"
+#include "few_inputs.cuh"
 #include "few_outputs.cuh"
 #include "fused_small_k.cuh"
 #include "input_tma.cuh"
@@ -801,6 +802,43 @@ int launch_few_outputs(const __half* x, const void* wT, const __half* bias, __ha
         case 4: return launch_few_outputs_as<4>(tmX, q, N, status, st);
         default: return launch_few_outputs_as<8>(tmX, q, N, status, st);
     }
+}
+
+// Layers with at most 4 input channels, fp16 tensors: see few_inputs.cuh.  TMA writes y as [N][K][H * W], whose rows must be
+// whole 16-byte pieces.  F(2x2) filters and fewer than a million outputs stay with fused_small_c_mma_kernel, whose chain is
+// shorter: 4->320 at 32x32 4.2 us there, 5.3 here, at 48x48 5.1 / 5.3, at 64x64 (batch 2) 7.8 / 7.3.  The F(4x4) kernel takes 16.
+bool use_few_inputs(int N, int C, int H, int W, int K, int tile, const void* y) {
+    const long long hw = static_cast<long long>(H) * W;
+    return C <= FI_CMAX && (tile == 4 || (tile == 2 && hw * N * K >= (1ll << 20))) && hw % 8 == 0 && aligned(y, 16) &&
+           (hw + FI_TILE - 1) / FI_TILE * N < (1ll << 24) && hw < (1ll << 30) && K <= 65535 * FI_K;
+}
+
+int launch_few_inputs(const __half* x, const void* wT, const __half* bias, __half* y, int N, int C, int H, int W, int K, int tile,
+                      int Kb, cudaStream_t st) {
+    const int sms = sm_count();
+    int* status = status_word_ptr();
+    if (sms <= 0 || !status || !ensure_dyn_smem(reinterpret_cast<const void*>(few_inputs_kernel), FI_SMEM)) return err_cuda(__LINE__);
+    const uint64_t hw = static_cast<uint64_t>(H) * W;
+    CUtensorMap tmY;
+    if (!encode_map(&tmY, y, hw, K, N, hw, static_cast<uint64_t>(K) * hw, 64, FI_K, true)) return err_cuda(__LINE__);
+    FewInputsParams q;
+    q.wt_header = wt_header_of(wT);
+    q.U = static_cast<const __half*>(wt_filters_of(wT));
+    q.x = x; q.bias = bias;
+    q.C = C; q.K = K; q.tile = tile; q.H = H; q.W = W; q.Kb = Kb;
+    q.hw = static_cast<int>(hw);
+    q.tiles_image = (q.hw + FI_TILE - 1) / FI_TILE;
+    q.tiles = q.tiles_image * N;
+    q.w_div = make_fastdiv(static_cast<uint32_t>(W));
+    q.image_div = make_fastdiv(static_cast<uint32_t>(q.tiles_image));
+    // two CTAs per SM, each with one block of channels and every grid.x-th tile
+    const int blocks = (K + FI_K - 1) / FI_K;
+    const int most = std::max(1, 2 * sms / blocks), rounds = (q.tiles + most - 1) / most;
+    const dim3 grid(static_cast<unsigned>((q.tiles + rounds - 1) / rounds), static_cast<unsigned>(blocks));
+    ProfScope prof(KIND_FUSED, st);
+    const cudaError_t e = launch_pdl(few_inputs_kernel, grid, dim3(FI_THREADS), static_cast<size_t>(FI_SMEM), st, 0, tmY, q, status);
+    g_launches.fetch_add(1);
+    return e == cudaSuccess ? SDWINO_OK : err_cuda(__LINE__);
 }
 
 // F(2x2,3x3) layers with at most 8 input channels: one warp-MMA kernel (see fused_small_c_mma_kernel).
@@ -1614,6 +1652,9 @@ int conv_impl(const void* x, const void* wT, const void* bias, void* y, int N, i
         return launch_fused_small_c_mma(static_cast<const float*>(x), wT, static_cast<const float*>(bias),
                                         static_cast<float*>(y), geo, C, K, pl.Kb, st);
     }
+    if (plain && !disable_fused && use_few_inputs(N, C, H, W, K, tile, y))
+        return launch_few_inputs(static_cast<const __half*>(x), wT, static_cast<const __half*>(bias), static_cast<__half*>(y), N, C, H, W,
+                                 K, tile, pl.Kb, st);
     if (plain && use_fused_small_c(C, tile) && !disable_fused) {
         const TileGeom geo = make_geom(H, W, pl.TH, pl.TW, pl.P);
         const __half* xh = static_cast<const __half*>(x);

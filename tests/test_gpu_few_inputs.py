@@ -1,0 +1,56 @@
+"""Layers with at most 4 input channels, fp16 tensors: one kernel that gathers the nine taps for the tensor core."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2412_05781_b200 import workloads
+from paper_2412_05781_b200.workloads import ConvLayer
+
+pytestmark = pytest.mark.gpu
+
+# C, K, H, W, N: one tile and several, tiles that end inside a row or hang over the image, several images, blocks of 128
+# output channels and their rests, images one pixel wide or high, widths that no vector divides, several tiles per CTA; with
+# tile 2 the shapes below a million outputs run the F(2x2) kernel
+SHAPES = [(4, 40, 8, 8, 1), (3, 17, 10, 16, 2), (4, 320, 64, 64, 2), (1, 5, 7, 8, 3), (2, 128, 17, 24, 2), (4, 129, 9, 48, 1),
+          (4, 9, 8, 1, 2), (3, 12, 1, 264, 1), (4, 300, 16, 37, 2), (4, 512, 40, 52, 1), (4, 256, 136, 130, 3), (4, 1, 24, 131, 1)]
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2412_05781_b200 import binding
+    return binding
+
+
+@pytest.mark.parametrize("tile", [2, 4])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_against_the_oracle(B, shape, tile):
+    C, K, H, W, N = shape
+    x, w, b = workloads.make_inputs(ConvLayer(C=C, K=K, H=H, W=W, N=N), seed=sum(shape))
+    ref = oracle.direct_conv3x3(x.numpy(), w.numpy(), b.numpy())
+    wT = B.sdwino_filter_transform(w.cuda(), tile)
+    ws = B.alloc_workspace(B.sdwino_workspace_bytes(N, C, H, W, K, tile))
+    # what lies before and behind y is not written
+    room = torch.full((N * K * H * W + 128,), float("nan"), dtype=torch.float16, device="cuda")
+    y = room[64:-64].view(N, K, H, W)
+    n0 = B.sdwino_launch_count()
+    B.sdwino_conv3x3(x.cuda(), wT, b.cuda(), K, tile, y=y, workspace=ws)
+    assert B.sdwino_launch_count() - n0 == 1
+    again = B.sdwino_conv3x3(x.cuda(), wT, b.cuda(), K, tile, workspace=ws)
+    assert B.sdwino_last_device_status() == B.OK
+    assert torch.equal(y, again)
+    assert torch.isnan(room[:64]).all() and torch.isnan(room[-64:]).all()
+    # U, the tap and y are rounded, 2**-11 of each; a middle tap is a difference of two roundings of U, which is up to 1.9 times
+    # a tap: at most a few times 2**-11 of the root of the sum over 9 C products, a quarter of max|ref|
+    assert np.abs(y.cpu().double().numpy() - ref).max() <= 1.5e-3 * np.abs(ref).max()
+
+
+def test_wrong_filters_are_refused(B):
+    x, w, b = workloads.make_inputs(ConvLayer(C=4, K=32, H=16, W=16, N=1), seed=1)
+    wT = B.sdwino_filter_transform(w.cuda(), 2)
+    ws = B.alloc_workspace(B.sdwino_workspace_bytes(1, 4, 16, 16, 32, 4))
+    wT[:16].view(torch.int32)[3] = 4            # a header that says F(4x4)
+    y = torch.full((1, 32, 16, 16), 7.0, dtype=torch.float16, device="cuda")
+    B.sdwino_conv3x3(x.cuda(), wT, b.cuda(), 32, 2, y=y, workspace=ws)
+    assert B.sdwino_last_device_status() == B.ERR_INVALID_ARG
+    assert torch.all(y == 7.0)
