@@ -223,8 +223,17 @@ __device__ __forceinline__ bool wait_role_a32(uint32_t bar_a, uint64_t* bar, uin
     if constexpr (PIPE) return mbar_try_wait_a32(bar_a, parity) || mbar_wait_slow(bar, parity, abort_flag, limit_ns);
     else return mbar_wait_warp_a32(bar_a, bar, parity, abort_flag, limit_ns);
 }
+//
+// Registers of the launches of one tile per CTA: shared memory leaves room for one CTA per SM, but the CTAs of the output
+// transform (6-8 thousand registers each, no shared memory) and of the next activation transform wait beside it for their turn,
+// and what does not fit the register file starts only when it has left.  So that instantiation is compiled for three CTAs
+// (56 registers instead of 76, nothing spilled): 1280->1280 at 16x16, batch 2, 18.6 -> 18.1 us, 640->640 at 32x32, batch 2,
+// 17.0 -> 16.5, 320->320 at 32x32 9.85 -> 9.37, 2560->1280 at 16x16 28.3 -> 27.8; with 64 registers 18.6, 16.8 and 9.36.  The
+// other instantiations lose more to fewer registers than their successors gain (stmatrix staging with 96 instead of 123:
+// 320->320 at 64x64, batch 2, 17.1 -> 17.5).
 template <int CTAS, bool RES = false, bool DUAL = false, bool PIPE = false, bool U8 = false, bool STM = true>
-__global__ void __launch_bounds__(PIPE ? PIPE_THREADS : (U8 ? GEMM_U8_THREADS : GEMM_LAUNCH_THREADS), 1)
+__global__ void __launch_bounds__(PIPE ? PIPE_THREADS : (U8 ? GEMM_U8_THREADS : GEMM_LAUNCH_THREADS),
+                                  CTAS == 1 && !RES && !DUAL && !PIPE && !U8 && !STM ? 3 : 1)
 wino_gemm_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmV,
                  const __grid_constant__ CUtensorMap tmM, const GemmParams prm, int* __restrict__ status_word,
                  const PipeParams pp) {
