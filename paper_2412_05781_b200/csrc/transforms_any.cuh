@@ -101,15 +101,19 @@ __device__ __forceinline__ void load_window_pixels(const __half* __restrict__ im
         }
 }
 
-// Activation preprocess of the pair (p, p + 1) for one channel; p - p_begin even.  Tiles past the last one are zeros.
-// EDGE: x cuts words.
+// Activation preprocess of the pair (p, p + 1) for one channel; p - p_begin even.  The threads are numbered over (channel, pair
+// of tiles of the image): few are idle, and what V holds past the last tile stays as it is (the GEMM multiplies it, but a tile is
+// a row of its product and no thread reads those rows).  Numbered per channel up to the next block of 128 tiles,
+// half of the threads of 640 channels at 50x37, batch 2, had nothing to load: with both steps numbered so the layer went 32.4 ->
+// 29.4 us, 320 channels 20.0 -> 18.6, 1280 at 25x19 37.5 -> 36.0, 640 at 50x37 in fp32 35.5 -> 33.7.  EDGE: x cuts words.
 template <int M, typename XT = __half, bool EDGE = false>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, M == 4 ? (sizeof(XT) == 4 ? 4 : (EDGE ? 5 : 6)) : 8)
 input_transform_any_kernel(const XT* __restrict__ x, __half* __restrict__ V, TileGeom geo, int C, long long p_begin,
-                           int p_count, long long Pstride, const float* __restrict__ amax) {
+                           FastDiv pairs, long long Pstride, const float* __restrict__ amax) {
     constexpr int A = M + 2;
-    const int pl = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x) * 2;
-    int c = static_cast<int>(blockIdx.z * gridDim.y + blockIdx.y);   // grid.z continues grid.y past 65535
+    const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x;      // < 2^31
+    int c = static_cast<int>(fast_div(idx, pairs));                  // pairs.d = pairs of tiles per channel in this pass
+    const int pl = static_cast<int>(idx - static_cast<uint32_t>(c) * pairs.d) * 2;
     if (EDGE && c < C) c = c == 0 ? C - 1 : c - 1;     // the two channels that take longer go first (1-2 us less)
     const long long hw = static_cast<long long>(geo.H) * geo.W;
     int i0[2] = {0, 0}, j0[2] = {0, 0};
@@ -118,7 +122,7 @@ input_transform_any_kernel(const XT* __restrict__ x, __half* __restrict__ V, Til
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
         const long long p = p_begin + pl + t;
-        valid[t] = p < geo.P && pl < p_count && c < C;
+        valid[t] = p < geo.P && c < C;
         if (valid[t]) {
             int tw, th;
             long long n;
@@ -131,7 +135,7 @@ input_transform_any_kernel(const XT* __restrict__ x, __half* __restrict__ V, Til
     // Wait first, release the GEMM second (see input_direct_kernel); the index arithmetic needs nothing from memory.
     pdl_wait();
     pdl_launch_dependents();
-    if (pl >= p_count || c >= C) return;
+    if (c >= C || p_begin + pl >= geo.P) return;
     float2 e2[A][A];   // rows transformed along the columns, (tile 0, tile 1)
     if constexpr (sizeof(XT) == 2) {
         uint32_t h0[A][A / 2], h1[A][A / 2];
@@ -184,7 +188,8 @@ input_transform_any_kernel(const XT* __restrict__ x, __half* __restrict__ V, Til
     }
 }
 
-// Postprocess.  A warp owns 64 consecutive tiles, two per thread, and walks `steps` output channels.  Stored from the
+// Postprocess.  A warp owns 64 consecutive tiles, two per thread, and walks `steps` output channels; the warps are numbered over
+// (steps of channels, 64 tiles of the image), as the threads of the activation step.  Stored from the
 // registers, a warp's rows of eight pixels would leave as 4-byte or 2-byte pieces 16 bytes apart, each of them a partial
 // write of its sector; the output rows of the warp's tiles go through shared memory instead ([M][64 tiles][M pixels],
 // private to the warp) and leave with neighbouring lanes on neighbouring pixel pairs.
@@ -196,7 +201,7 @@ constexpr int OUT_ANY_THREADS = 128;
 template <int M, bool EP, typename YT = __half>
 __global__ void __launch_bounds__(OUT_ANY_THREADS, 5)
 output_transform_any_kernel(const __half* __restrict__ Mws, const YT* __restrict__ bias, YT* __restrict__ y, TileGeom geo,
-                            int K, long long p_begin, int p_count, long long Pstride, int steps, WtCheck chk, Epilogue ep) {
+                            int K, long long p_begin, FastDiv chunks, long long Pstride, int steps, WtCheck chk, Epilogue ep) {
     constexpr int A = M + 2;
     constexpr int WORDS = M;                     // pixel pairs per thread and output row: 64 tiles * M pixels / 2 / 32
     // with something to add after the convolution the gathered values are not rounded yet
@@ -205,9 +210,11 @@ output_transform_any_kernel(const __half* __restrict__ Mws, const YT* __restrict
     pdl_launch_dependents();
     const bool wt_ok = wt_check(chk);            // before the wait: see output_direct_kernel
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int pl0 = (static_cast<int>(blockIdx.x) * (OUT_ANY_THREADS / 32) + warp) * 64;     // first tile of the warp in the pass
+    const uint32_t unit = blockIdx.x * (OUT_ANY_THREADS / 32) + warp;                        // < 2^31
+    const uint32_t kg = fast_div(unit, chunks);                                              // chunks.d = chunks of 64 tiles in this pass
+    const int pl0 = static_cast<int>(unit - kg * chunks.d) * 64;                             // first tile of the warp in the pass
     const long long hw = static_cast<long long>(geo.H) * geo.W;
-    const int k_first = static_cast<int>(blockIdx.z * gridDim.y + blockIdx.y) * steps;       // grid.z continues grid.y
+    const int k_first = static_cast<int>(kg) * steps;
     const int k_end = min(K, k_first + steps);
     // the pixel pairs this lane stores: pair w = j * 32 + lane of a row of 64 * M pixels
     long long off[WORDS];                        // first output row of the pair in channel 0 of its image
@@ -218,7 +225,7 @@ output_transform_any_kernel(const __half* __restrict__ Mws, const YT* __restrict
         const long long p = p_begin + pl0 + px / M;
         off[j] = 0;
         rows[j] = cols[j] = 0;
-        if (pl0 < p_count && p < geo.P) {
+        if (p < geo.P) {
             int tw, th;
             long long n;
             decode_tile(geo, p, n, th, tw);
@@ -229,7 +236,7 @@ output_transform_any_kernel(const __half* __restrict__ Mws, const YT* __restrict
         }
     }
     pdl_wait();
-    if (!wt_ok || pl0 >= p_count) return;
+    if (!wt_ok || k_first >= K || p_begin + pl0 >= geo.P) return;
     [[maybe_unused]] float ys = 1.f;
     if constexpr (sizeof(YT) == 4) ys = scalbnf(1.f, range_exponent(ep.amax));
     const long long plane = static_cast<long long>(K) * Pstride;

@@ -53,3 +53,23 @@ def test_any_width_and_alignment(B, shape, tile, offset):
     refe = oracle.epilogue(ref, res.numpy(), "silu")
     assert np.abs(y.cpu().double().numpy() - refe).max() <= 1e-2 * np.abs(refe).max()
     assert bool((canary[:pad + offset] == 1234.0).all()) and bool((canary[pad + offset + n:] == 1234.0).all())
+
+
+@pytest.mark.parametrize("tile", [2, 4])
+@pytest.mark.parametrize("shape", [
+    # C, K, H, W, N: less than one block of 128 tiles and more, an odd number of tiles, threads numbered over whole warps (from 512
+    # pairs of tiles per channel on) and over pairs, CTA pairs and two blocks of tiles per CTA in the GEMM
+    (16, 24, 5, 7, 1), (72, 40, 19, 23, 1), (16, 16, 67, 129, 1), (512, 512, 63, 65, 1), (320, 320, 45, 37, 2), (12, 16, 131, 259, 1),
+])
+def test_what_the_workspace_held_reaches_no_output(B, shape, tile):
+    # the activation step leaves V past the last tile as it was: all bytes 255 are NaNs
+    C, K, H, W, N = shape
+    x, w, b = workloads.make_inputs(ConvLayer(C=C, K=K, H=H, W=W, N=N), seed=sum(shape))
+    wT = B.sdwino_filter_transform(w.cuda(), tile)
+    ws = B.alloc_workspace(B.sdwino_workspace_bytes(N, C, H, W, K, tile))
+    ys = []
+    for fill in (255, 0):
+        ws.fill_(fill)
+        ys.append(B.sdwino_conv3x3(x.cuda(), wT, b.cuda(), K, tile, workspace=ws))
+    assert B.sdwino_last_device_status() == B.OK
+    assert bool(torch.isfinite(ys[0]).all()) and torch.equal(ys[0], ys[1])
